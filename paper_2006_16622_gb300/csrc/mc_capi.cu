@@ -2,6 +2,7 @@
 // library (declared in include/mcfmm.h).  Host code only: argument checks,
 // device memory ownership, kernel launches and copies.
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <math.h>
 #include <stdint.h>
 #include <stdlib.h>
@@ -15,6 +16,7 @@
 
 #include "../../include/mcfmm.h"
 #include "mc_dev.cuh"
+#include "mc_fixsum.cuh"
 
 // kernels defined in the other translation units
 cudaError_t mc_launch_chain(const McSys* d_sys, const RunParams& rp, int prec, int var, int nCTA,
@@ -63,6 +65,8 @@ struct mc_ctx {
   int schedule;                // MC_SCHEDULE_*
   double* d_mpole;             // per-level multipoles (fast setup), allocated on first use
   double* d_otab;              // offset harmonics table (fast setup)
+  bool fixed;                  // charges within the span of the fixed-point sums
+  int qexp;                    // |q| <= 2^qexp
   std::vector<void*> allocs;
 };
 
@@ -99,8 +103,24 @@ double scale_of(int k) {
   return sqrt(fact(n - m) * fact(n + m));
 }
 
-// chunks of the interaction list per target on level l (1 = write in place)
-// chunks per target cell of the Alg. L.3 gather on level l: about eight
+// the fixed-point sums of this context's charges
+FixSource fix_source(const McSys& h) {
+  return FixSource{reinterpret_cast<const double*>(h.cpos), h.ccount, h.cap, nullptr, nullptr};
+}
+FixPass fix_pass(const mc_ctx* c, int l, bool irregular) {
+  const McSys& h = c->h;
+  return FixPass{h.L, l, h.p, irregular, h.bc == MC_BC_PBC, h.a, c->qexp, 1};
+}
+// chunks of one fixed-point pass, as many as the scratch holds
+int fix_chunks_for(const McSys& h, int sms, int l, bool irregular, size_t max_doubles) {
+  const size_t ncl = (size_t)1 << (3 * (l - 1));
+  const int n = fix_chunks(h.L, l, irregular, sms, (double)h.n / (double)h.ncellL, h.p);
+  const size_t most = max_doubles / (ncl * h.C);
+  return (int)std::max<size_t>(1, std::min<size_t>((size_t)n, most));
+}
+
+// chunks per target cell of the FP64 Alg. L.3 gather on level l (charges too
+// uneven for the fixed-point sums): about eight
 // equal tasks per resident warp (one CTA per SM), at most one chunk per
 // source unit (189 finest cells of the list per target and level cell)
 int chunks_for_level(const McSys& h, int sms, int l, size_t max_doubles) {
@@ -173,20 +193,25 @@ int launch_chain(mc_ctx* c, RunParams& rp) {
 int run_setup(mc_ctx* c) {
   McSys& h = c->h;
   const int C = h.C;
-  // Alg. L.3 per level (gather, chunked over the interaction list)
+  // Alg. L.3 per level: a gather over the interaction list of every cell,
+  // chunked where a level has few cells.  In fixed point (8 times faster at
+  // N = 1e5, p = 12 and at least as accurate) unless the charges span more
+  // than MC_FIX_QSPAN powers of two
   for (int l = h.lmin; l <= h.L; l++) {
     const int nl = h.lev_n[l], ncl = nl * nl * nl;
-    const int nchunk = chunks_for_level(h, c->sms, l, c->scratch_doubles);
-    const int ntask = ncl * nchunk;
     double* dst = h.Lhat + (size_t)h.lev_off[l] * C;
-    k_p2l_level<<<grid_for(c->sms, ntask, MC_WARPS), MC_THREADS, 0, c->stream>>>(
-        c->d_sys, l, nchunk, nchunk > 1 ? c->d_scratch : dst);
-    CK(cudaGetLastError());
-    if (nchunk > 1) {
-      k_reduce_chunks<<<grid_for(c->sms, (size_t)ncl * C, 256), 256, 0, c->stream>>>(
-          ncl, nchunk, C, c->d_scratch, dst);
+    int nchunk;
+    if (c->fixed) {
+      FixPass ps = fix_pass(c, l, true);
+      ps.nchunk = nchunk = fix_chunks_for(h, c->sms, l, true, c->scratch_doubles);
+      CK(fix_launch(ps, fix_source(h), nchunk > 1 ? c->d_scratch : dst, c->stream));
+    } else {
+      nchunk = chunks_for_level(h, c->sms, l, c->scratch_doubles);
+      k_p2l_level<<<grid_for(c->sms, ncl * nchunk, MC_WARPS), MC_THREADS, 0, c->stream>>>(
+          c->d_sys, l, nchunk, nchunk > 1 ? c->d_scratch : dst);
       CK(cudaGetLastError());
     }
+    if (nchunk > 1) CK(fix_reduce(ncl, nchunk, C, c->sms, c->d_scratch, dst, c->stream));
   }
   // K, dipole, H = G K
   const int nch = std::min<int>(1024, std::max<int>(1, h.n / 64));
@@ -420,6 +445,18 @@ int mc_init(mc_ctx** out, int64_t n, const double* pos, const double* q, double 
   h.inv_wL = (double)h.nL / box;
   h.ncellL = h.nL * h.nL * h.nL;
   h.lmin = (bc == MC_BC_PBC) ? 2 : 3;
+  // the charges' range: the fixed-point sums take them as fractions of the
+  // power of two above the largest
+  int qmax = INT_MIN, qmin = INT_MAX;
+  for (int64_t i = 0; i < n; i++) {
+    if (q[i] == 0.0) continue;
+    int e;
+    const double f = frexp(fabs(q[i]), &e);
+    qmax = std::max(qmax, f == 0.5 ? e - 1 : e);
+    qmin = std::min(qmin, e);
+  }
+  c->qexp = qmax == INT_MIN ? 0 : qmax;
+  c->fixed = qmax == INT_MIN || qmax - qmin <= MC_FIX_QSPAN;
   int off = 0;
   for (int l = 1; l <= levels; l++) {
     h.lev_n[l] = 1 << (l - 1);
@@ -522,7 +559,8 @@ int mc_init(mc_ctx** out, int64_t n, const double* pos, const double* q, double 
   size_t need = 0;
   for (int l = h.lmin; l <= levels; l++) {
     const size_t ncl = (size_t)h.lev_n[l] * h.lev_n[l] * h.lev_n[l];
-    const int nchunk = chunks_for_level(h, c->sms, l, kScratchCap);
+    const int nchunk = c->fixed ? fix_chunks_for(h, c->sms, l, true, kScratchCap)
+                                : chunks_for_level(h, c->sms, l, kScratchCap);
     if (nchunk > 1) need = std::max(need, ncl * nchunk * C);
     // offset chunks of the fast setup's multipole-to-local pass
     const size_t nco = (size_t)m2l_offset_chunks(h.lev_n[l], c->sms);

@@ -1,0 +1,410 @@
+// Harmonic sums over the charges of cells in fixed point (mc_fix.cuh): the
+// Alg. L.3 gather of every setup, the multipoles of Eq. (4).
+#include <algorithm>
+
+#include "mc_dev.cuh"
+#include "mc_fix.cuh"
+#include "mc_fixsum.cuh"
+
+namespace {
+
+constexpr int kRound = 256;  // source units (finest cells) listed at a time
+
+struct FixArgs {
+  FixTab tab;
+  FixSource src;
+  int L, l, nchunk, irregular, pbc;
+  uint64_t rcp;  // fx_coord's reciprocal of the box side
+  int ea;        // biased exponent of the box side
+  int qexp;
+};
+
+// entry k (0..188) of the interaction list of a cell with parities b, in the
+// order of il_table_init: the 6^3 children of the parent's neighbours without
+// the 27 near cells
+__device__ __forceinline__ void list_entry(int k, const int* b, int* o) {
+  int i, j, q, rem;
+  const int head = 36 * (1 + b[0]);
+  if (k < head) {
+    i = k / 36;
+    rem = k % 36;
+    j = rem / 6;
+    q = rem % 6;
+  } else if (k < head + 81) {
+    const int k1 = k - head;
+    i = 1 + b[0] + k1 / 27;
+    rem = k1 % 27;
+    const int r0 = 6 * (1 + b[1]);
+    if (rem < r0) {
+      j = rem / 6;
+      q = rem % 6;
+    } else if (rem < r0 + 9) {
+      const int r1 = rem - r0;
+      j = 1 + b[1] + r1 / 3;
+      q = r1 % 3;
+      if (q >= 1 + b[2]) q += 3;
+    } else {
+      const int r2 = rem - r0 - 9;
+      j = 4 + b[1] + r2 / 6;
+      q = r2 % 6;
+    }
+  } else {
+    const int k2 = k - head - 81;
+    i = 4 + b[0] + k2 / 36;
+    rem = k2 % 36;
+    j = rem / 6;
+    q = rem % 6;
+  }
+  o[0] = i - 2 - b[0];
+  o[1] = j - 2 - b[1];
+  o[2] = q - 2 - b[2];
+}
+
+// index of a coefficient with m = 0 (no imaginary part)
+__device__ __forceinline__ bool is_square_index(int k) {
+  const int r = (int)sqrtf((float)k + 0.5f);
+  return r * r == k;
+}
+
+__device__ __forceinline__ int64_t shfl_xor64(int64_t v, int m) {
+  const int lo = __shfl_xor_sync(0xffffffffu, (int)(uint32_t)v, m);
+  const int hi = __shfl_xor_sync(0xffffffffu, (int)(v >> 32), m);
+  return (int64_t)(((uint64_t)(uint32_t)hi << 32) | (uint32_t)lo);
+}
+
+// Sums over the lanes of 2 x 16 terms: lane c ends with term c & 15 of ar
+// (lanes 0..15) or ai (16..31); each exchange halves the terms a lane
+// carries.  B: first step, terms past ST are 0.
+template <int ST, int B>
+__device__ __forceinline__ int64_t lane_totals(const int64_t (&ar)[ST], const int64_t (&ai)[ST], int lane) {
+  int64_t v[16];
+#pragma unroll
+  for (int i = 0; i < 16; i++) {
+    if (B + i < ST) {
+      const bool up = lane & 16;
+      v[i] = (up ? ai[B + i] : ar[B + i]) + shfl_xor64(up ? ar[B + i] : ai[B + i], 16);
+    } else {
+      v[i] = 0;
+    }
+  }
+#pragma unroll
+  for (int w = 8; w >= 1; w >>= 1) {
+#pragma unroll
+    for (int i = 0; i < w; i++) {
+      if (B + i < ST) {
+        const bool up = lane & w;
+        const int64_t hi = B + i + w < ST ? v[i + w] : 0;
+        v[i] = (up ? hi : v[i]) + shfl_xor64(up ? v[i] : hi, w);
+      }
+    }
+  }
+  return v[0];
+}
+
+constexpr int kThreads = 32 * MC_FIX_WARPS;
+// registers: 4 per step for the sums, about 70 for the rest
+constexpr int fix_ctas(int st) { return st <= 14 ? 4 : (st <= 23 ? 3 : 2); }
+
+}  // namespace
+
+// One CTA per (target cell, chunk of its source units).  Its four warps share
+// the columns m evenly, and every lane takes one charge of a group of 32: a
+// warp's table entries are uniform, no lane idles (groups of 8 lanes per
+// charge leave 21 of 112 idle at p = 12), every sub-partition has the same
+// work, and each lane keeps the sums of its coefficients in registers.  The
+// CTA forms what depends on the displacement for 128 charges at a time, one
+// per thread, in shared memory, where all four warps read it.
+// Bound by the issue of 32-bit integer instructions (one per two cycles and
+// sub-partition): 33 per coefficient and 32 charges, 23 of them multiply-adds.
+template <int P>
+__global__ void __launch_bounds__(kThreads, fix_ctas(fix_shares(P).steps))
+    k_fix_sums(const __grid_constant__ FixArgs A, double* __restrict__ out) {
+  constexpr int ST = fix_shares(P).steps;
+  constexpr int p = P, nthr = kThreads;
+  __shared__ FixStep s_step[MC_FIX_WARPS][ST];
+  __shared__ int s_cell[kRound], s_shift[kRound], s_pre[kRound + 1];
+  extern __shared__ int64_t dyn[];
+  if (A.src.range && !fix_usable(A.src.range)) return;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  for (int i = tid; i < MC_FIX_WARPS * ST; i += nthr) s_step[i / ST][i % ST] = A.tab.step[i / ST][i % ST];
+  const bool irr = A.irregular != 0, pbc = A.pbc != 0;
+  const int qexp = A.src.range ? A.src.range[1] - 1022 : A.qexp;
+  int64_t* s_zeta = dyn;                 // [nthr]
+  int64_t* s_kap = dyn + nthr;           // [nthr]
+  int64_t* s_Y = dyn + 2 * (size_t)nthr;  // [3 (p + 1)][nthr]: Y_m^m, cos m phi, sin m phi
+  const int l = A.l, nl = 1 << (l - 1), nL = 1 << (A.L - 1), fb = A.L - l, f = 1 << fb;
+  const int task = blockIdx.x, t = task / A.nchunk, ch = task % A.nchunk;
+  const int tc[3] = {t / (nl * nl), (t / nl) % nl, t % nl};
+  const int par[3] = {tc[0] & 1, tc[1] & 1, tc[2] & 1};
+  uint64_t T[3];
+#pragma unroll
+  for (int d = 0; d < 3; d++) T[d] = (uint64_t)(2 * tc[d] + 1) << (62 - l);
+  const long long units = (long long)(irr ? 189 : 1) << (3 * fb);
+  const long long per = (units + A.nchunk - 1) / A.nchunk;
+  const long long ub = (long long)ch * per, ue = ub + per < units ? ub + per : units;
+  // steps where a column begins, from ballots so that the branch is uniform
+  const unsigned turn_lo = __ballot_sync(0xffffffffu, (A.tab.turn[warp] >> lane) & 1ull);
+  const unsigned turn_hi = __ballot_sync(0xffffffffu, (A.tab.turn[warp] >> (lane + 32)) & 1ull);
+  int64_t ar[ST], ai[ST];
+#pragma unroll
+  for (int i = 0; i < ST; i++) ar[i] = ai[i] = 0;
+  double sum[3] = {0.0, 0.0, 0.0};  // this lane's coefficients: steps (lane & 15) + 16 b
+  int held = 0;                     // groups since the last flush
+  auto flush = [&]() {
+#pragma unroll
+    for (int i = 0; i < ST; i++) {
+      ar[i] = (ar[i] + 16) >> 5;
+      ai[i] = (ai[i] + 16) >> 5;
+    }
+    sum[0] += (double)lane_totals<ST, 0>(ar, ai, lane);
+    if constexpr (ST > 16) sum[1] += (double)lane_totals<ST, 16>(ar, ai, lane);
+    if constexpr (ST > 32) sum[2] += (double)lane_totals<ST, 32>(ar, ai, lane);
+#pragma unroll
+    for (int i = 0; i < ST; i++) ar[i] = ai[i] = 0;
+    held = 0;
+  };
+  for (long long u0 = ub; u0 < ue; u0 += kRound) {
+    __syncthreads();
+    for (int i = tid; i < kRound; i += nthr) {
+      int cnt = 0, cell = 0, sh = 0;
+      const long long u = u0 + i;
+      if (u < ue) {
+        int o[3] = {0, 0, 0};
+        if (irr) list_entry((int)(u >> (3 * fb)), par, o);
+        const int fc = (int)(u & (((long long)1 << (3 * fb)) - 1));
+        const int fd[3] = {fc >> (2 * fb), (fc >> fb) & (f - 1), fc & (f - 1)};
+        int g[3];
+        bool ok = true;
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+          const int e = tc[d] + o[d], s = mc_wrap_coord(e, nl);
+          if (!pbc && e != s) ok = false;
+          sh |= ((e - s) / nl + 2) << (4 * d);
+          g[d] = s * f + fd[d];
+        }
+        cell = (g[0] * nL + g[1]) * nL + g[2];
+        if (ok) cnt = A.src.start ? A.src.start[cell + 1] - A.src.start[cell] : A.src.count[cell];
+      }
+      s_cell[i] = cell;
+      s_shift[i] = sh;
+      s_pre[i + 1] = cnt;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      constexpr int kPer = kRound / 32;
+      int c[kPer], tot = 0;
+#pragma unroll
+      for (int i = 0; i < kPer; i++) {
+        c[i] = s_pre[1 + lane * kPer + i];
+        tot += c[i];
+      }
+      int inc = tot;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
+      }
+      int run = inc - tot;
+#pragma unroll
+      for (int i = 0; i < kPer; i++) {
+        run += c[i];
+        s_pre[1 + lane * kPer + i] = run;
+      }
+      if (lane == 0) s_pre[0] = 0;
+    }
+    __syncthreads();
+    const int total = s_pre[kRound];
+    for (int b0 = 0; b0 < total; b0 += nthr) {
+      const int idx = b0 + tid;
+      FixCharge c = {0, 0, 0, 0, 0, 0};
+      if (idx < total) {
+        int lo = 0;
+#pragma unroll
+        for (int s = kRound / 2; s > 0; s >>= 1)
+          if (s_pre[lo + s] <= idx) lo += s;
+        const int cell = s_cell[lo], slot = idx - s_pre[lo], sh = s_shift[lo];
+        double x[3], q;
+        if (A.src.start) {
+          const double* r = A.src.rows + 4 * ((size_t)A.src.start[cell] + slot);
+          x[0] = r[0];
+          x[1] = r[1];
+          x[2] = r[2];
+          q = r[3];
+        } else {
+          const double4 r = ldcg4(reinterpret_cast<const double4*>(A.src.rows) + (size_t)cell * A.src.cap + slot);
+          x[0] = r.x;
+          x[1] = r.y;
+          x[2] = r.z;
+          q = r.w;
+        }
+        int64_t D[3];
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+          const int im = ((sh >> (4 * d)) & 15) - 2;
+          const uint64_t X = (uint64_t)fx_coord(x[d], A.rcp, A.ea) + ((uint64_t)(int64_t)im << 62);
+          const int64_t v = (int64_t)(X - T[d]);
+          const int k = irr ? l - 3 : l - 1;
+          D[d] = k >= 0 ? (int64_t)((uint64_t)v << k) : v >> 1;
+        }
+        const int64_t qf = fx_charge(q, 1023 + qexp);
+        c = irr ? fix_irregular(D[0], D[1], D[2], qf) : fix_regular(D[0], D[1], D[2], qf);
+      }
+      s_zeta[tid] = c.zeta;
+      s_kap[tid] = (int64_t)c.kap;
+      {
+        const Fx ex = fx_split(c.ex), ey = fx_split(c.ey), en = fx_split(-c.ey), st = fx_split(c.st);
+        int64_t y = c.x0, xr = (int64_t)1 << 62, xi = 0;
+        int64_t* o = s_Y + tid;
+        for (int m = 0; m <= p; m++) {
+          o[0] = y;
+          o[nthr] = xr >> 3;
+          o[2 * nthr] = xi >> 3;
+          o += 3 * nthr;
+          const Fx a = fx_split(xr), b = fx_split(xi);
+          y = fx_mul62(fx_split(y), st);
+          fx_turn(a, b, ex, ey, en, &xr, &xi);
+        }
+      }
+      __syncthreads();
+      const int ng = min(MC_FIX_WARPS, (total - b0 + 31) >> 5);
+      if (held + ng > MC_FIX_FLUSH) flush();
+      for (int g = 0; g < ng; g++) {
+        const int s = g * 32 + lane;
+        const uint64_t kap = (uint64_t)s_kap[s];
+        const uint32_t kh = (uint32_t)(kap >> 32), kl = (uint32_t)kap;
+        const Fx zp = fx_split(s_zeta[s]), zm = fx_split(-s_zeta[s]);
+        Fx zs = zp, zn = zm;  // +zeta and -zeta, by step in turn
+        Fx Xr = {0, 0}, Xi = {0, 0}, q1 = {0, 0}, q2 = {0, 0};
+        int c = 0;
+#pragma unroll
+        for (int i = 0; i < ST; i++) {
+          if ((i < 32 ? turn_lo >> i : turn_hi >> (i & 31)) & 1u) {  // a column begins
+            const int64_t* o = s_Y + (size_t)(3 * A.tab.col[warp][c++]) * nthr + s;
+            q1 = fx_split(o[0]);
+            q2 = {0, 0};
+            Xr = fx_split(o[nthr]);
+            Xi = fx_split(o[2 * nthr]);
+            zs = (i & 1) ? zm : zp;
+            zn = (i & 1) ? zp : zm;
+          } else {
+            const FixStep st = s_step[warp][i];
+            const Fx q = fix_next((i & 1) ? zs : zn, kh, kl, q1, q2, st.wh, st.wl, st.sh);
+            q2 = q1;
+            q1 = q;
+          }
+          ar[i] = fix_mac(Xr, q1, ar[i]);
+          ai[i] = fix_mac(Xi, q1, ai[i]);
+        }
+      }
+      held += ng;
+      __syncthreads();
+    }
+  }
+  flush();
+  constexpr int C = (P + 1) * (P + 1);
+  const double sc = ldexp(1.0, qexp);
+  double* o = out + ((size_t)t * A.nchunk + ch) * C;
+#pragma unroll
+  for (int b = 0; 16 * b < ST; b++) {
+    const int i = 16 * b + (lane & 15), im = lane >> 4;
+    const int k = i < ST ? A.tab.index[warp][i] : -1;
+    if (k < 0 || (im && is_square_index(k))) continue;
+    const double r = sum[b] * A.tab.scale[warp][i] * sc;
+    o[k + im] = im ? -r : r;
+  }
+}
+
+// chunk partials of many chunks and few targets: 8 warps take every eighth
+// chunk of 32 coefficients, added in one order
+__global__ void __launch_bounds__(256)
+    k_fix_reduce(int nchunk, int C, const double* __restrict__ in, double* __restrict__ out) {
+  __shared__ double s[8][32];
+  const int nb = (C + 31) / 32, t = blockIdx.x / nb, k = (blockIdx.x % nb) * 32 + (threadIdx.x & 31);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double v = 0.0;
+  if (k < C)
+    for (int ch = warp; ch < nchunk; ch += 8) v += in[((size_t)t * nchunk + ch) * C + k];
+  s[warp][lane] = v;
+  __syncthreads();
+  if (warp == 0 && k < C) {
+    for (int w = 1; w < 8; w++) v += s[w][lane];
+    out[(size_t)t * C + k] = v;
+  }
+}
+
+__global__ void k_reduce_chunks(int, int, int, const double*, double*);
+
+cudaError_t fix_reduce(int ntarget, int nchunk, int C, int sms, const double* in, double* out, cudaStream_t st) {
+  // one thread per coefficient up to 8 chunks, eight warps per coefficient
+  // block above
+  if (nchunk <= 8) {
+    const size_t b = ((size_t)ntarget * C + 255) / 256;
+    k_reduce_chunks<<<(int)std::max<size_t>(1, std::min<size_t>(b, (size_t)sms * 8)), 256, 0, st>>>(ntarget, nchunk, C,
+                                                                                                  in, out);
+  } else {
+    k_fix_reduce<<<ntarget * ((C + 31) / 32), 256, 0, st>>>(nchunk, C, in, out);
+  }
+  return cudaGetLastError();
+}
+
+int fix_chunks(int L, int l, bool irregular, int sms, double occupancy, int p) {
+  const long long nl = 1LL << (l - 1), ncl = nl * nl * nl;
+  const long long units = (irregular ? 189LL : 1LL) << (3 * (L - l));
+  // about eight tasks per resident CTA ...
+  const long long want = (8LL * fix_ctas(fix_shares(p).steps) * sms + ncl - 1) / ncl;
+  // ... of at least two staged batches of charges each
+  const double least = 2.0 * kThreads / std::max(occupancy, 0.25);
+  const long long most = std::max<long long>(1, (long long)((double)units / least));
+  return (int)std::max<long long>(1, std::min(std::min(want, most), units));
+}
+
+cudaError_t fix_launch(const FixPass& ps, const FixSource& src, double* out, cudaStream_t st) {
+  FixArgs A;
+  const double w = ps.a / (double)(1 << (ps.l - 1));
+  fix_tab_build(&A.tab, ps.p, ps.irregular, ps.irregular ? kFixR0 * w : w);
+  A.src = src;
+  A.L = ps.L;
+  A.l = ps.l;
+  A.nchunk = ps.nchunk;
+  A.irregular = ps.irregular;
+  A.pbc = ps.pbc;
+  A.qexp = ps.qexp;
+  uint64_t u;
+  __builtin_memcpy(&u, &ps.a, 8);
+  A.ea = (int)((u >> 52) & 0x7ff);
+  const uint64_t m = (u & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
+  A.rcp = (uint64_t)((((unsigned __int128)1 << 115) + m / 2) / m);
+  const size_t smem = sizeof(int64_t) * (size_t)kThreads * (2 + 3 * (ps.p + 1));
+  const long long ncl = 1LL << (3 * (ps.l - 1));
+  const long long grid = ncl * ps.nchunk;
+  if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+  cudaError_t e = cudaErrorInvalidValue;
+#define MC_FIX_CASE(P_)                                                                              \
+  case P_:                                                                                          \
+    e = cudaFuncSetAttribute(k_fix_sums<P_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
+    if (e == cudaSuccess) {                                                                         \
+      k_fix_sums<P_><<<(int)grid, kThreads, smem, st>>>(A, out);                                    \
+      e = cudaGetLastError();                                                                       \
+    }                                                                                               \
+    break;
+  switch (ps.p) {
+    MC_FIX_CASE(0)
+    MC_FIX_CASE(1)
+    MC_FIX_CASE(2)
+    MC_FIX_CASE(3)
+    MC_FIX_CASE(4)
+    MC_FIX_CASE(5)
+    MC_FIX_CASE(6)
+    MC_FIX_CASE(7)
+    MC_FIX_CASE(8)
+    MC_FIX_CASE(9)
+    MC_FIX_CASE(10)
+    MC_FIX_CASE(11)
+    MC_FIX_CASE(12)
+    MC_FIX_CASE(13)
+    MC_FIX_CASE(14)
+    MC_FIX_CASE(15)
+  }
+#undef MC_FIX_CASE
+  return e;
+}

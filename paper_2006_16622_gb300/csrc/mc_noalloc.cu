@@ -14,12 +14,16 @@
 
 #include "../../include/mcfmm.h"
 #include "mc_dev.cuh"
+#include "mc_fixsum.cuh"
 
 // The fixed scratch: MC_NOALLOC_SCRATCH_DOUBLES doubles (8 MiB) of device
 // memory per GPU that loads the library, held until the process exits.  In
 // host code `g_noalloc_scratch` is only a host-side stand-in for the symbol;
 // its device address comes from cudaGetSymbolAddress below.
 static __device__ __align__(256) double g_noalloc_scratch[MC_NOALLOC_SCRATCH_DOUBLES];
+
+// what decides between the fixed-point sums and the FP64 ones (FixSource::range)
+static __device__ int g_noalloc_range[3];
 
 namespace {
 
@@ -34,7 +38,9 @@ struct NoAllocP2L {
 // (x, y, z, q per row).  Every task writes all C values of its partial.
 __global__ void __launch_bounds__(MC_THREADS)
     k_p2l_level_noalloc(NoAllocP2L P, const double* __restrict__ part,
-                        const int* __restrict__ cstart, double* __restrict__ scratch) {
+                        const int* __restrict__ cstart, const int* __restrict__ range,
+                        double* __restrict__ scratch) {
+  if (fix_usable(range)) return;  // done in fixed point
   __shared__ HarmTabs<double> tabs;
   __shared__ unsigned short il[8][189];
   __shared__ double stage[MC_WARPS][256];
@@ -110,17 +116,60 @@ __global__ void __launch_bounds__(MC_THREADS)
   }
 }
 
-// out[t][k] = (sum over chunks in order) / sqrt((n-m)!(n+m)!): the paper's
-// normalisation of the coefficients (the same layout as mc_get_local)
-__global__ void k_reduce_noalloc(int ntarget, int nchunk, int C, const double* __restrict__ in,
-                                 double* __restrict__ out) {
-  const size_t total = (size_t)ntarget * C;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total;
-       i += (size_t)gridDim.x * blockDim.x) {
-    const size_t t = i / C;
-    const int k = (int)(i % C);
-    double s = 0.0;
-    for (int ch = 0; ch < nchunk; ch++) s += in[(t * nchunk + ch) * C + k];
+// The range of the charges and whether every charge lies in its cell (the
+// fixed-point sums rely on the distances that gives): one warp per finest
+// cell, combined with atomic maxima.
+__global__ void __launch_bounds__(MC_THREADS)
+    k_noalloc_range(int nL, double inv_w, const double* __restrict__ part, const int* __restrict__ cstart,
+                    int* __restrict__ range) {
+  const int lane = threadIdx.x & 31;
+  int bad = 0, emax = 0, emin = 0;
+  for (int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < nL * nL * nL; c += (gridDim.x * blockDim.x) >> 5) {
+    const int g[3] = {c / (nL * nL), (c / nL) % nL, c % nL};
+    for (int i = cstart[c] + lane; i < cstart[c + 1]; i += 32) {
+      const double* v = part + 4 * (size_t)i;
+#pragma unroll
+      for (int d = 0; d < 3; d++) {
+        const double x = v[d] * inv_w - (double)g[d];
+        if (!(x >= -1.0 / 16384.0 && x <= 1.0 + 1.0 / 16384.0 && v[d] >= 0.0)) bad = 1;
+      }
+      const int e = (int)((__double_as_longlong(v[3]) >> 52) & 0x7ff);
+      if (e == 0x7ff) bad = 1;
+      if (v[3] != 0.0) {
+        emax = max(emax, max(e, 1));
+        emin = max(emin, 4096 - max(e, 1));
+      }
+    }
+  }
+  bad = __reduce_max_sync(0xffffffffu, bad);
+  emax = __reduce_max_sync(0xffffffffu, emax);
+  emin = __reduce_max_sync(0xffffffffu, emin);
+  if (lane == 0) {
+    if (bad) atomicMax(&range[0], 1);
+    if (emax) {
+      atomicMax(&range[1], emax);
+      atomicMax(&range[2], emin);
+    }
+  }
+}
+
+// out[t][k] = (sum over chunks in one order) / sqrt((n-m)!(n+m)!): the
+// paper's normalisation of the coefficients (the same layout as
+// mc_get_local); 8 warps per 32 coefficients of a target, each taking every
+// eighth chunk
+__global__ void __launch_bounds__(MC_THREADS)
+    k_reduce_noalloc(int nchunk, int C, const double* __restrict__ in, double* __restrict__ out) {
+  __shared__ double part[MC_WARPS][32];
+  const int nb = (C + 31) / 32, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const size_t t = blockIdx.x / nb;
+  const int k = (blockIdx.x % nb) * 32 + lane;
+  double s = 0.0;
+  if (k < C)
+    for (int ch = warp; ch < nchunk; ch += MC_WARPS) s += in[(t * nchunk + ch) * C + k];
+  part[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0 && k < C) {
+    for (int w = 1; w < min(MC_WARPS, nchunk); w++) s += part[w][lane];
     int n = (int)sqrtf((float)k + 0.5f);
     while (n * n > k) n--;
     while ((n + 1) * (n + 1) <= k) n++;
@@ -128,7 +177,7 @@ __global__ void k_reduce_noalloc(int ntarget, int nchunk, int C, const double* _
     double f = 1.0;
     for (int q = 2; q <= n - mm; q++) f *= q;
     for (int q = 2; q <= n + mm; q++) f *= q;
-    out[i] = s / sqrt(f);
+    out[t * C + k] = s / sqrt(f);
   }
 }
 
@@ -137,20 +186,24 @@ __global__ void k_reduce_noalloc(int ntarget, int nchunk, int C, const double* _
 // forbids calls after one)
 constexpr int kMaxDevices = 64;
 double* g_scratch_ptr[kMaxDevices];
+int* g_range_ptr[kMaxDevices];
 std::mutex g_scratch_mutex;
 
-int scratch_for_current_device(double** out) {
+int scratch_for_current_device(double** out, int** range) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return MC_ERR_CUDA;
   std::lock_guard<std::mutex> lock(g_scratch_mutex);
   if (!g_scratch_ptr[dev]) {
-    void* ptr = nullptr;
-    if (cudaGetSymbolAddress(&ptr, g_noalloc_scratch) != cudaSuccess || !ptr) {
+    void *ptr = nullptr, *rng = nullptr;
+    if (cudaGetSymbolAddress(&ptr, g_noalloc_scratch) != cudaSuccess || !ptr ||
+        cudaGetSymbolAddress(&rng, g_noalloc_range) != cudaSuccess || !rng) {
       cudaGetLastError();  // the failed lookup's own error (none was pending)
       return MC_ERR_CUDA;
     }
+    g_range_ptr[dev] = (int*)rng;
     g_scratch_ptr[dev] = (double*)ptr;
   }
+  *range = g_range_ptr[dev];
   *out = g_scratch_ptr[dev];
   return MC_OK;
 }
@@ -175,14 +228,15 @@ extern "C" int mc_p2l_level_noalloc(const double* d_part, const int* d_cell_star
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return MC_ERR_CUDA;
-  long long nchunk = (4LL * sms * MC_WARPS + ncl - 1) / ncl;
-  nchunk = nchunk < 1 ? 1 : (nchunk > 189 ? 189 : nchunk);
+  const long long ncellL = 1LL << (3 * (levels - 1));
+  long long nchunk = fix_chunks(levels, level, true, sms, (double)n / (double)ncellL, p);
   while (nchunk > 1 && ncl * nchunk * C > (long long)MC_NOALLOC_SCRATCH_DOUBLES) nchunk--;
   // an error left by the caller's earlier work is not ours to clear or
   // report as this call's own: launch nothing
   if (cudaPeekAtLastError() != cudaSuccess) return MC_ERR_PENDING;
   double* scratch = nullptr;
-  int rc = scratch_for_current_device(&scratch);
+  int* range = nullptr;
+  int rc = scratch_for_current_device(&scratch, &range);
   if (rc != MC_OK) return rc;
   NoAllocP2L P;
   P.L = levels;
@@ -195,15 +249,29 @@ extern "C" int mc_p2l_level_noalloc(const double* d_part, const int* d_cell_star
   P.a = box;
   P.w = box / (double)nl;
   cudaStream_t stream = (cudaStream_t)cuda_stream;
+  // charges that lie in their cells and span a few powers of two are summed
+  // in fixed point (level 4 of N = 1e5, p = 12: 104 ms in FP64); the FP64
+  // gather does the others, and returns at once otherwise
+  if (cudaMemsetAsync(range, 0, 3 * sizeof(int), stream) != cudaSuccess) {
+    cudaGetLastError();
+    return MC_ERR_CUDA;
+  }
+  const int rblocks = (int)((ncellL + MC_WARPS - 1) / MC_WARPS < 8LL * sms ? (ncellL + MC_WARPS - 1) / MC_WARPS : 8LL * sms);
+  k_noalloc_range<<<rblocks, MC_THREADS, 0, stream>>>(P.nL, (double)P.nL / box, d_part, d_cell_start, range);
+  // no error was pending before the launch, so one now is the launch's own
+  if (cudaGetLastError() != cudaSuccess) return MC_ERR_CUDA;
+  const FixPass ps{levels, level, p, true, bc == MC_BC_PBC, box, 0, (int)nchunk};
+  const FixSource src{d_part, nullptr, 0, d_cell_start, range};
+  if (fix_launch(ps, src, scratch, stream) != cudaSuccess) {
+    cudaGetLastError();
+    return MC_ERR_CUDA;
+  }
   const long long ntask = ncl * nchunk;
   long long blocks = (ntask + MC_WARPS - 1) / MC_WARPS;
   if (blocks > 8LL * sms) blocks = 8LL * sms;
-  k_p2l_level_noalloc<<<(int)blocks, MC_THREADS, 0, stream>>>(P, d_part, d_cell_start, scratch);
-  // no error was pending before the launch, so one now is the launch's own
+  k_p2l_level_noalloc<<<(int)blocks, MC_THREADS, 0, stream>>>(P, d_part, d_cell_start, range, scratch);
   if (cudaGetLastError() != cudaSuccess) return MC_ERR_CUDA;
-  long long rb = (ncl * C + 255) / 256;
-  if (rb > 8LL * sms) rb = 8LL * sms;
-  k_reduce_noalloc<<<(int)rb, 256, 0, stream>>>((int)ncl, (int)nchunk, C, scratch, d_out);
+  k_reduce_noalloc<<<(int)(ncl * ((C + 31) / 32)), MC_THREADS, 0, stream>>>((int)nchunk, C, scratch, d_out);
   if (cudaGetLastError() != cudaSuccess) return MC_ERR_CUDA;
   return MC_OK;
 }
