@@ -17,6 +17,7 @@
 #include "../../include/mcfmm.h"
 #include "mc_dev.cuh"
 #include "mc_fixsum.cuh"
+#include "mc_m2l.cuh"
 
 // kernels defined in the other translation units
 cudaError_t mc_launch_chain(const McSys* d_sys, const RunParams& rp, int prec, int var, int nCTA,
@@ -64,7 +65,10 @@ struct mc_ctx {
   unsigned long long* d_prof;  // MC_PROF_COUNTERS timers when profiling is on, else null
   int schedule;                // MC_SCHEDULE_*
   double* d_mpole;             // per-level multipoles (fast setup), allocated on first use
-  double* d_otab;              // offset harmonics table (fast setup)
+  double* d_otab;              // offset harmonics table (FP64 fast setup)
+  const void* m2l_table;       // this order's matrices (shared, see m2l_table_get)
+  long long* d_mfix;           // a level's multipoles as integers, their units
+  int* d_mexp;
   bool fixed;                  // charges within the span of the fixed-point sums
   int qexp;                    // |q| <= 2^qexp
   std::vector<void*> allocs;
@@ -281,9 +285,74 @@ int run_setup_mm(mc_ctx* c) {
   return setup_far(c);
 }
 
-int run_setup_fmm(mc_ctx* c) {
+// The matrices of the fixed-point translations depend on p only: one table
+// per (device, p), built when a context first needs it, shared by the
+// contexts of every thread and stream (complete before it is handed out, and
+// never written again), freed with the last context that uses it.
+struct M2LTable {
+  void* ptr;
+  int users;
+};
+std::map<std::pair<int, int>, M2LTable> g_m2l_tables;
+std::mutex g_m2l_mutex;
+
+int m2l_table_get(mc_ctx* c) {
+  if (c->m2l_table) return MC_OK;
+  std::lock_guard<std::mutex> lock(g_m2l_mutex);
+  const std::pair<int, int> key{c->dev, c->h.p};
+  auto it = g_m2l_tables.find(key);
+  if (it == g_m2l_tables.end()) {
+    const int per = (2 * c->h.p + 1) * (2 * c->h.p + 2) / 2;
+    void* t = nullptr;
+    double* otab = nullptr;
+    if (cudaMalloc(&t, m2l_table_bytes(c->h.p)) != cudaSuccess ||
+        cudaMalloc((void**)&otab, sizeof(double) * 2 * 343 * (size_t)per) != cudaSuccess) {
+      cudaGetLastError();
+      cudaFree(t);
+      return MC_ERR_NOMEM;
+    }
+    const bool ok = m2l_build_table(c->h.p, c->sms, t, otab, c->stream) == cudaSuccess &&
+                    cudaStreamSynchronize(c->stream) == cudaSuccess;
+    cudaFree(otab);
+    if (!ok) {
+      cudaFree(t);
+      return MC_ERR_CUDA;
+    }
+    it = g_m2l_tables.insert({key, M2LTable{t, 0}}).first;
+  }
+  it->second.users++;
+  c->m2l_table = it->second.ptr;
+  return MC_OK;
+}
+
+void m2l_table_release(mc_ctx* c) {
+  if (!c->m2l_table) return;
+  std::lock_guard<std::mutex> lock(g_m2l_mutex);
+  auto it = g_m2l_tables.find({c->dev, c->h.p});
+  if (it != g_m2l_tables.end() && --it->second.users == 0) {
+    cudaFree(it->second.ptr);
+    g_m2l_tables.erase(it);
+  }
+  c->m2l_table = nullptr;
+}
+
+// multipole-to-local over every level: in fixed point, or in FP64 for charges
+// too uneven for it
+int m2l_levels(mc_ctx* c) {
   McSys& h = c->h;
   const int C = h.C, p = h.p;
+  if (c->fixed) {
+    int rc = m2l_table_get(c);
+    if (rc != MC_OK) return rc;
+    if (!c->d_mfix && dalloc(c, (void**)&c->d_mfix, sizeof(long long) * (size_t)h.ncellL * C) != MC_OK)
+      return MC_ERR_NOMEM;
+    if (!c->d_mexp && dalloc(c, (void**)&c->d_mexp, sizeof(int) * (size_t)h.ncellL) != MC_OK) return MC_ERR_NOMEM;
+    for (int l = h.lmin; l <= h.L; l++)
+      CK(m2l_fix_level(p, l, h.lev_w[l], h.bc == MC_BC_PBC, c->sms, c->m2l_table,
+                       c->d_mpole + (size_t)h.lev_off[l] * C, c->d_mfix, c->d_mexp,
+                       h.Lhat + (size_t)h.lev_off[l] * C, c->d_scratch, c->scratch_doubles, c->stream));
+    return MC_OK;
+  }
   const int per = (2 * p + 1) * (2 * p + 2) / 2;
   if (!c->d_otab) {
     if (dalloc(c, (void**)&c->d_otab, sizeof(double) * 2 * 343 * (size_t)per) != MC_OK)
@@ -291,13 +360,19 @@ int run_setup_fmm(mc_ctx* c) {
     k_offset_table<<<grid_for(c->sms, 343 * (size_t)per, 256), 256, 0, c->stream>>>(p, c->d_otab);
     CK(cudaGetLastError());
   }
-  int rc = p2m_levels(c);
-  if (rc != MC_OK) return rc;
   for (int l = h.lmin; l <= h.L; l++) {
     CK(m2l_launch(c->d_sys, p, l, h.lev_n[l], c->sms, c->d_mpole + (size_t)h.lev_off[l] * C,
                   c->d_otab, h.Lhat + (size_t)h.lev_off[l] * C, c->d_scratch, c->scratch_doubles,
                   c->stream));
   }
+  return MC_OK;
+}
+
+int run_setup_fmm(mc_ctx* c) {
+  McSys& h = c->h;
+  int rc = p2m_levels(c);
+  if (rc == MC_OK) rc = m2l_levels(c);
+  if (rc != MC_OK) return rc;
   const int nch = std::min<int>(1024, std::max<int>(1, h.n / 64));
   k_box_multipole<<<grid_for(c->sms, nch, MC_WARPS), MC_THREADS, 0, c->stream>>>(c->d_sys, nch,
                                                                                 c->d_scratch);
@@ -400,6 +475,7 @@ void mc_destroy(mc_ctx* c) {
   if (!c) return;
   cudaSetDevice(c->dev);
   cudaStreamSynchronize(c->stream);
+  m2l_table_release(c);
   for (void* p : c->allocs) cudaFree(p);
   delete c;
 }
@@ -563,7 +639,7 @@ int mc_init(mc_ctx** out, int64_t n, const double* pos, const double* q, double 
                                 : chunks_for_level(h, c->sms, l, kScratchCap);
     if (nchunk > 1) need = std::max(need, ncl * nchunk * C);
     // offset chunks of the fast setup's multipole-to-local pass
-    const size_t nco = (size_t)m2l_offset_chunks(h.lev_n[l], c->sms);
+    const size_t nco = (size_t)(c->fixed ? m2l_chunks(h.lev_n[l], c->sms) : m2l_offset_chunks(h.lev_n[l], c->sms));
     if (nco > 1) need = std::max(need, std::min(ncl * nco * C, kScratchCap));
   }
   need = std::max(need, (size_t)1024 * (C + 3));

@@ -1,0 +1,469 @@
+// Multipole-to-local translations of the fast setup (Sec. 3.2, last
+// paragraph) in fixed point on the integer pipe.
+//
+// With multipoles and expansions in units of their cell (Mhat = M w^-n,
+// Lhat = L w^(j+1), paper normalisation) every offset o of an interaction
+// list has one matrix T_o of size C x C, |T| <= 1/2, whose rows sum to at
+// most 137 over all 189 offsets.  Two things make it cheap here:
+//   * integer multiply-adds of 32 x 32 + 64 bits issue every 2 cycles and
+//     FP64 ones every 64, so a product of two 57-bit numbers (28-bit low
+//     parts, the product of those, below 2^-57, left out) takes 6 cycles, and
+//     sums are exact;
+//   * in the real layout a reflection x -> -x (y, z) only changes signs:
+//     T_(s o) = X_s T_o X_s with X_s diagonal, +-1, so that the up to eight
+//     offsets that differ in signs share one product:
+//       sum_s T_(s o) M_s = sum_c T_o[r][c] Mt_d[c],  d = class(r) ^ class(c),
+//       Mt_d = sum_s (-1)^(s . d) M_s
+//     (class: the parities of a coefficient under the three reflections; Mt
+//     a Walsh-Hadamard transform of eight cells' multipoles).  189 products
+//     per cell become 56.
+// A CTA takes 32 target cells of one parity class, one per lane; warp k
+// computes the rows of class k, so that a lane needs one Mt value per column
+// and warp, and the matrix entries are the same for all lanes.
+#include <math.h>
+
+#include <algorithm>
+
+#include "mc_dev.cuh"
+#include "mc_fix.cuh"
+#include "mc_fixsum.cuh"
+#include "mc_m2l.cuh"
+
+namespace {
+
+constexpr int kTile = 16;     // columns staged at a time
+constexpr int kOrbits = 56;   // offsets up to signs: {0..3}^3 without {0, 1}^3
+constexpr int kMaxRows = (MC_PMAX + 1) * (MC_PMAX + 1) + 8;
+constexpr int kBitsT = 57, kBitsM = 54, kLimb = 28;
+
+struct M2LLayout {  // rows by class, every class padded to an even number
+  int start[8], count[8], rows;
+  short index[kMaxRows];  // real-layout index of a row, -1: padding
+};
+
+// parities under x -> -x (bit 2), y -> -y (bit 1), z -> -z (bit 0)
+int class_of(int n, int m, int im) { return (((m + im) & 1) << 2) | (im << 1) | ((n + m) & 1); }
+
+M2LLayout m2l_layout(int p) {
+  M2LLayout L;
+  L.rows = 0;
+  for (int c = 0; c < 8; c++) {
+    L.start[c] = L.rows;
+    for (int n = 0; n <= p; n++)
+      for (int m = 0; m <= n; m++)
+        for (int im = 0; im < (m ? 2 : 1); im++)
+          if (class_of(n, m, im) == c) L.index[L.rows++] = (short)(n * n + (m ? 2 * m - 1 : 0) + im);
+    L.count[c] = L.rows - L.start[c];
+    if (L.rows & 1) L.index[L.rows++] = -1;
+  }
+  return L;
+}
+
+struct M2LArgs {
+  int l, nl, h, pbc, p, nco, per_o;
+  int start[8], count[8], rows;
+  unsigned char ccol[kMaxRows];  // class of a column
+  unsigned char orbit[kOrbits];  // |ox| | |oy| << 2 | |oz| << 4
+  short index[kMaxRows];
+  double scale[kMaxRows];
+};
+
+__device__ __forceinline__ void decode(int k, int* n, int* m, int* im) {
+  int r = (int)sqrtf((float)k + 0.5f);
+  while (r * r > k) r--;
+  while ((r + 1) * (r + 1) <= k) r++;
+  *n = r;
+  const int rem = k - r * r;
+  *m = (rem + 1) / 2;
+  *im = (rem > 0 && (rem & 1) == 0) ? 1 : 0;
+}
+
+struct TableArgs {
+  int p, rows;
+  unsigned char orbit[kOrbits];
+  short index[kMaxRows];
+};
+
+// T_o[row][col] from the scaled irregular harmonics of the integer offsets
+// (k_offset_table); entry (orbit, col, row)
+__global__ void k_m2l_tables(const __grid_constant__ TableArgs A, const double* __restrict__ otab, int2* __restrict__ T) {
+  const int p = A.p, C = (p + 1) * (p + 1), cpad = (C + kTile - 1) / kTile * kTile;
+  const int per = (2 * p + 1) * (2 * p + 2) / 2;
+  const long long total = (long long)kOrbits * cpad * A.rows;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+    const int r = (int)(i % A.rows), col = (int)(i / A.rows % cpad), ob = A.orbit[i / A.rows / cpad];
+    double v = 0.0;
+    if (A.index[r] >= 0 && col < C) {
+      int j, k, rim, n, m, cim;
+      decode(A.index[r], &j, &k, &rim);
+      decode(col, &n, &m, &cim);
+      const double* t0 = otab + 2 * (size_t)((((ob & 3) + 3) * 7 + ((ob >> 2) & 3) + 3) * 7 + ((ob >> 4) & 3) + 3) * per;
+      const int l = j + n;
+      t0 += l * (l + 1);
+      const int d = m - k, ad = d < 0 ? -d : d;
+      const double sg = (min(k, m) & 1) ? -1.0 : 1.0;
+      const double ar = sg * t0[2 * ad], ai = (d < 0 ? -sg : sg) * t0[2 * ad + 1];
+      const double br = t0[2 * (m + k)], bi = t0[2 * (m + k) + 1];
+      if (m == 0) {
+        v = rim ? ai : ar;
+      } else {
+        v = rim ? (cim ? ar - br : ai - bi) : (cim ? -(ai + bi) : ar + br);
+      }
+      if (n & 1) v = -v;
+      double f = 1.0, g = 1.0;
+      for (int q = 2; q <= j - k; q++) f *= q;
+      for (int q = 2; q <= j + k; q++) f *= q;
+      for (int q = 2; q <= n - m; q++) g *= q;
+      for (int q = 2; q <= n + m; q++) g *= q;
+      v /= sqrt(f) * sqrt(g);
+    }
+    const long long w = __double2ll_rn(ldexp(v, kBitsT));
+    const int lo = ((int)w << (32 - kLimb)) >> (32 - kLimb);
+    T[i] = make_int2((int)((w - lo) >> kLimb), lo);
+  }
+}
+
+struct ConvArgs {
+  int nl, C;
+  double scale[kMaxRows];  // sqrt((n-m)!(n+m)!) w^-n
+};
+
+// one level's multipoles (scaled layout, by cell) as integers of kBitsM bits
+// in units of a power of two per cell, stored by column; cells ordered by
+// parity class, then by halved coordinates (consecutive lanes of a translation
+// read consecutive cells)
+__global__ void __launch_bounds__(256)
+    k_m2l_convert(const __grid_constant__ ConvArgs A, const double* __restrict__ K, long long* __restrict__ M,
+                  int* __restrict__ E) {
+  extern __shared__ long long tile[];  // [32][C + 1]
+  const int C = A.C, nl = A.nl, h = nl >> 1, h3 = h * h * h, ncl = nl * nl * nl;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, base = blockIdx.x * 32;
+  for (int c = warp; c < 32; c += 8) {
+    const int pos = base + c;
+    if (pos >= ncl) break;
+    const int cls = pos / h3, r = pos % h3;
+    const int i = 2 * (r / (h * h)) + ((cls >> 2) & 1), j = 2 * ((r / h) % h) + ((cls >> 1) & 1), k = 2 * (r % h) + (cls & 1);
+    const double* src = K + (size_t)((i * nl + j) * nl + k) * C;
+    double v[8];
+    int e = -4096;
+#pragma unroll
+    for (int u = 0; u < 8; u++) {
+      const int col = lane + 32 * u;
+      v[u] = col < C ? src[col] * A.scale[col] : 0.0;
+      if (v[u] != 0.0) e = max(e, (int)((__double_as_longlong(v[u]) >> 52) & 0x7ff) - 1022);
+    }
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) E[pos] = e;
+#pragma unroll
+    for (int u = 0; u < 8; u++) {
+      const int col = lane + 32 * u;
+      if (col < C) tile[c * (C + 1) + col] = e == -4096 ? 0ll : __double2ll_rn(ldexp(v[u], kBitsM - e));
+    }
+  }
+  __syncthreads();
+  if (base + lane < ncl)
+    for (int col = warp; col < C; col += 8) M[(size_t)col * ncl + base + lane] = tile[lane * (C + 1) + col];
+}
+
+__device__ __forceinline__ void cta_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
+
+struct M2LTask {
+  int cls, oc;  // target class, orbit chunk; this lane's target (clamped):
+  int I[3], b[3];
+  bool valid;
+  int ecta;
+};
+
+// halved coordinate and parity of coordinate 2 I + b + o on an axis with h
+// halves (wrapped, or -1 outside)
+__device__ __forceinline__ int half_of(int I, int b, int o, int h, bool pbc, int* par) {
+  const int e = b + o;
+  *par = e & 1;
+  const int v = I + ((e - *par) >> 1);
+  return pbc ? mc_wrap_coord(v, h) : (v < 0 || v >= h ? -1 : v);
+}
+
+// position (class-major) of the cell at offset o from this lane's target
+__device__ __forceinline__ int cell_at(const M2LTask& k, int ox, int oy, int oz, int h, bool pbc) {
+  int p0, p1, p2;
+  const int a = half_of(k.I[0], k.b[0], ox, h, pbc, &p0), b = half_of(k.I[1], k.b[1], oy, h, pbc, &p1),
+            c = half_of(k.I[2], k.b[2], oz, h, pbc, &p2);
+  if (a < 0 || b < 0 || c < 0) return -1;
+  return ((((p0 << 2 | p1 << 1 | p2) * h + a) * h) + b) * h + c;
+}
+
+// One CTA's task, as the warp that owns class w of NR rows sees it: every
+// warp stages its part of the next tile's Mt and table columns while it
+// computes the current one.
+template <int NR>
+__device__ __forceinline__ void m2l_task(const M2LArgs& A, const int2* __restrict__ T, const long long* __restrict__ M,
+                                         const int* __restrict__ E, double* __restrict__ out, const M2LTask& k,
+                                         int2* sT, int2* sM, int w, int lane) {
+  const int C = (A.p + 1) * (A.p + 1), tiles = (C + kTile - 1) / kTile, h = A.h, ncl = A.nl * A.nl * A.nl;
+  const int ob = k.oc * A.per_o, oe = min(kOrbits, ob + A.per_o);
+  const int steps = (oe - ob) * tiles, tsz = kTile * A.rows;
+  long long hh[NR > 0 ? NR : 1], x[NR > 0 ? NR : 1];
+#pragma unroll
+  for (int r = 0; r < NR; r++) hh[r] = x[r] = 0;
+  int cell[8], sh[8];
+  long long v[2][8];
+  auto load = [&](int s) {  // this thread's two columns of tile s
+    const int o = ob + s / tiles, tile = s % tiles;
+    if (tile == 0) {
+      const int a[3] = {A.orbit[o] & 3, (A.orbit[o] >> 2) & 3, (A.orbit[o] >> 4) & 3};
+#pragma unroll
+      for (int g = 0; g < 8; g++) {
+        bool ok = k.valid;
+        int of[3];
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+          const int neg = (g >> (2 - d)) & 1;
+          if ((a[d] == 0 && neg) || (a[d] == 3 && neg != k.b[d])) ok = false;
+          of[d] = neg ? -a[d] : a[d];
+        }
+        cell[g] = ok ? cell_at(k, of[0], of[1], of[2], h, A.pbc != 0) : -1;
+        sh[g] = cell[g] >= 0 ? min(63, k.ecta - E[cell[g]]) : 63;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      const int col = tile * kTile + 2 * w + u;
+#pragma unroll
+      for (int g = 0; g < 8; g++) v[u][g] = (cell[g] >= 0 && col < C) ? __ldg(&M[(size_t)col * ncl + cell[g]]) : 0ll;
+    }
+    const char* src = reinterpret_cast<const char*>(T + ((size_t)o * tiles + tile) * tsz);
+    char* dst = reinterpret_cast<char*>(sT + (s & 1) * tsz);
+    for (int i = 16 * (32 * w + lane); i < tsz * (int)sizeof(int2); i += 16 * 256) cp_async16(dst + i, src + i);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  auto store = [&](int s) {
+    int2* dst = sM + (size_t)(s & 1) * kTile * 8 * 32;
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+#pragma unroll
+      for (int g = 0; g < 8; g++) v[u][g] >>= sh[g];
+#pragma unroll
+      for (int b = 1; b < 8; b <<= 1)
+#pragma unroll
+        for (int g = 0; g < 8; g++)
+          if (!(g & b)) {
+            const long long lo = v[u][g], hi = v[u][g | b];
+            v[u][g] = lo + hi;
+            v[u][g | b] = lo - hi;
+          }
+      // transform index d = (x, y, z) bits (4, 2, 1) of the member signs
+#pragma unroll
+      for (int d = 0; d < 8; d++) {
+        const long long t = v[u][d];
+        const int l = ((int)t << (32 - kLimb)) >> (32 - kLimb);
+        dst[((2 * w + u) * 8 + d) * 32 + lane] = make_int2((int)((t - l) >> kLimb), l);
+      }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+  };
+  load(0);
+  store(0);
+  cta_sync();
+  int held = 0;
+  for (int s = 0; s < steps; s++) {
+    if (s + 1 < steps) load(s + 1);
+    if constexpr (NR > 0) {
+      const int tile = s % tiles;
+      const int2* t0 = sT + (s & 1) * tsz + A.start[w];
+      const int2* m0 = sM + (size_t)(s & 1) * kTile * 8 * 32 + lane;
+#pragma unroll 1
+      for (int c = 0; c < kTile; c++) {
+        const int d = w ^ A.ccol[tile * kTile + c];
+        const int2 m = m0[(c * 8 + d) * 32];
+        const int4* t = reinterpret_cast<const int4*>(t0 + c * A.rows);
+#pragma unroll
+        for (int r = 0; r < NR; r += 2) {
+          const int4 q = t[r / 2];
+          hh[r] = fx_wide(q.x, m.x, hh[r]);
+          x[r] = fx_wide(q.x, m.y, x[r]);
+          x[r] = fx_wide(q.y, m.x, x[r]);
+          if (r + 1 < NR) {
+            hh[r + 1] = fx_wide(q.z, m.x, hh[r + 1]);
+            x[r + 1] = fx_wide(q.z, m.y, x[r + 1]);
+            x[r + 1] = fx_wide(q.w, m.x, x[r + 1]);
+          }
+        }
+      }
+      // 64 columns of cross products stay below 2^63: carry them over
+      if (++held == 64 / kTile) {
+        held = 0;
+#pragma unroll
+        for (int r = 0; r < NR; r++) {
+          hh[r] += x[r] >> kLimb;
+          x[r] &= (1ll << kLimb) - 1;
+        }
+      }
+    }
+    if (s + 1 < steps) store(s + 1);
+    cta_sync();
+  }
+  if constexpr (NR > 0) {
+    if (k.valid) {
+      const int i = 2 * k.I[0] + k.b[0], j = 2 * k.I[1] + k.b[1], kk = 2 * k.I[2] + k.b[2];
+      double* o = out + ((size_t)((i * A.nl + j) * A.nl + kk) * A.nco + k.oc) * C;
+      const double unit = ldexp(1.0, k.ecta);
+#pragma unroll
+      for (int r = 0; r < NR; r++) {
+        hh[r] += x[r] >> kLimb;
+        x[r] &= (1ll << kLimb) - 1;
+        const double sum = (double)hh[r] + (double)x[r] * (1.0 / (double)(1 << kLimb));
+        o[A.index[A.start[w] + r]] = sum * A.scale[A.start[w] + r] * unit;
+      }
+    }
+  }
+}
+
+}  // namespace
+
+__global__ void __launch_bounds__(256, 1)
+    k_m2l_fix(const __grid_constant__ M2LArgs A, const int2* __restrict__ T, const long long* __restrict__ M,
+              const int* __restrict__ E, double* __restrict__ out) {
+  extern __shared__ int4 dyn4[];
+  __shared__ int s_emax;
+  int2* sT = reinterpret_cast<int2*>(dyn4);
+  int2* sM = sT + 2 * kTile * A.rows;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int h = A.h, h3 = h * h * h, chunks = (h3 + 31) / 32;
+  M2LTask k;
+  k.oc = blockIdx.x % A.nco;
+  const int tk = blockIdx.x / A.nco;
+  k.cls = tk / chunks;
+  const int ii = (tk % chunks) * 32 + lane;
+  k.valid = ii < h3;
+  const int r = min(ii, h3 - 1);
+  k.I[0] = r / (h * h);
+  k.I[1] = (r / h) % h;
+  k.I[2] = r % h;
+#pragma unroll
+  for (int d = 0; d < 3; d++) k.b[d] = (k.cls >> (2 - d)) & 1;
+  // unit of the sums: the largest unit of the cells in these targets' lists
+  if (threadIdx.x == 0) s_emax = -4096;
+  __syncthreads();
+  int e = -4096;
+  for (int q = w; q < 216; q += 8) {
+    const int ox = q / 36 - 2 - k.b[0], oy = (q / 6) % 6 - 2 - k.b[1], oz = q % 6 - 2 - k.b[2];
+    if (ox >= -1 && ox <= 1 && oy >= -1 && oy <= 1 && oz >= -1 && oz <= 1) continue;
+    const int c = cell_at(k, ox, oy, oz, h, A.pbc != 0);
+    if (c >= 0 && k.valid) e = max(e, E[c]);
+  }
+  e = __reduce_max_sync(0xffffffffu, e);
+  if (lane == 0) atomicMax(&s_emax, e);
+  __syncthreads();
+  k.ecta = s_emax;
+  switch (A.count[w]) {
+    case 1: m2l_task<1>(A, T, M, E, out, k, sT, sM, w, lane); break;
+    case 3: m2l_task<3>(A, T, M, E, out, k, sT, sM, w, lane); break;
+    case 6: m2l_task<6>(A, T, M, E, out, k, sT, sM, w, lane); break;
+    case 10: m2l_task<10>(A, T, M, E, out, k, sT, sM, w, lane); break;
+    case 15: m2l_task<15>(A, T, M, E, out, k, sT, sM, w, lane); break;
+    case 21: m2l_task<21>(A, T, M, E, out, k, sT, sM, w, lane); break;
+    case 28: m2l_task<28>(A, T, M, E, out, k, sT, sM, w, lane); break;
+    case 36: m2l_task<36>(A, T, M, E, out, k, sT, sM, w, lane); break;
+    default: m2l_task<0>(A, T, M, E, out, k, sT, sM, w, lane); break;
+  }
+}
+
+__global__ void k_offset_table(int p, double* __restrict__ out);
+
+size_t m2l_table_bytes(int p) {
+  const int C = (p + 1) * (p + 1);
+  return sizeof(int2) * (size_t)kOrbits * ((C + kTile - 1) / kTile * kTile) * m2l_layout(p).rows;
+}
+
+static void orbits(unsigned char* o) {
+  int n = 0;
+  for (int x = 0; x < 4; x++)
+    for (int y = 0; y < 4; y++)
+      for (int z = 0; z < 4; z++)
+        if (std::max(x, std::max(y, z)) > 1) o[n++] = (unsigned char)(x | y << 2 | z << 4);
+}
+
+cudaError_t m2l_build_table(int p, int sms, void* table, double* otab, cudaStream_t st) {
+  const int per = (2 * p + 1) * (2 * p + 2) / 2;
+  k_offset_table<<<std::max(1, std::min(sms * 8, (343 * per + 255) / 256)), 256, 0, st>>>(p, otab);
+  TableArgs A;
+  const M2LLayout L = m2l_layout(p);
+  A.p = p;
+  A.rows = L.rows;
+  std::copy(L.index, L.index + L.rows, A.index);
+  orbits(A.orbit);
+  k_m2l_tables<<<sms * 8, 256, 0, st>>>(A, otab, (int2*)table);
+  return cudaGetLastError();
+}
+
+static double sfac(int n, int m) {
+  double f = 1.0, g = 1.0;
+  for (int q = 2; q <= n - m; q++) f *= q;
+  for (int q = 2; q <= n + m; q++) g *= q;
+  return sqrt(f) * sqrt(g);
+}
+
+int m2l_chunks(int nl, int sms) {
+  const int h = nl / 2, tasks = 8 * ((h * h * h + 31) / 32);
+  // at least six tasks per SM (one CTA each), so that the last wave is short
+  return std::max(1, std::min(kOrbits, (6 * sms + tasks - 1) / tasks));
+}
+
+cudaError_t m2l_fix_level(int p, int l, double w, bool pbc, int sms, const void* table, const double* K, long long* M,
+                          int* E, double* Lout, double* scratch, size_t scratch_doubles, cudaStream_t st) {
+  const int C = (p + 1) * (p + 1), nl = 1 << (l - 1), h = nl / 2, ncl = nl * nl * nl;
+  const M2LLayout L = m2l_layout(p);
+  ConvArgs V;
+  V.nl = nl;
+  V.C = C;
+  M2LArgs A;
+  A.l = l;
+  A.nl = nl;
+  A.h = h;
+  A.pbc = pbc;
+  A.p = p;
+  A.nco = m2l_chunks(nl, sms);
+  while (A.nco > 1 && (size_t)ncl * A.nco * C > scratch_doubles) A.nco--;
+  A.per_o = (kOrbits + A.nco - 1) / A.nco;
+  A.nco = (kOrbits + A.per_o - 1) / A.per_o;
+  A.rows = L.rows;
+  for (int c = 0; c < 8; c++) {
+    A.start[c] = L.start[c];
+    A.count[c] = L.count[c];
+  }
+  orbits(A.orbit);
+  std::fill(A.ccol, A.ccol + kMaxRows, 0);
+  for (int n = 0; n <= p; n++) {
+    const double wn = pow(w, -(double)n);
+    for (int m = 0; m <= n; m++)
+      for (int im = 0; im < (m ? 2 : 1); im++) {
+        const int k = n * n + (m ? 2 * m - 1 : 0) + im;
+        A.ccol[k] = (unsigned char)class_of(n, m, im);
+        V.scale[k] = sfac(n, m) * wn;
+      }
+  }
+  for (int r = 0; r < L.rows; r++) {
+    A.index[r] = L.index[r];
+    A.scale[r] = 0.0;
+    if (L.index[r] < 0) continue;
+    int n = (int)sqrt((double)L.index[r] + 0.5);
+    const int rem = L.index[r] - n * n, m = (rem + 1) / 2;
+    A.scale[r] = sfac(n, m) * pow(w, -(double)(n + 1)) * ldexp(1.0, 2 * kLimb - kBitsT - kBitsM);
+  }
+  const size_t csm = sizeof(long long) * 32 * (C + 1);
+  cudaError_t e = cudaFuncSetAttribute(k_m2l_convert, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm);
+  if (e != cudaSuccess) return e;
+  k_m2l_convert<<<(ncl + 31) / 32, 256, csm, st>>>(V, K, M, E);
+  const size_t smem = sizeof(int2) * 2 * ((size_t)kTile * L.rows + kTile * 8 * 32);
+  e = cudaFuncSetAttribute(k_m2l_fix, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const int chunks = (h * h * h + 31) / 32;
+  k_m2l_fix<<<8 * chunks * A.nco, 256, smem, st>>>(A, (const int2*)table, M, E, A.nco > 1 ? scratch : Lout);
+  e = cudaGetLastError();
+  if (e == cudaSuccess && A.nco > 1) e = fix_reduce(ncl, A.nco, C, sms, scratch, Lout, st);
+  return e;
+}
