@@ -5,10 +5,11 @@
 // Lhat = L w^(j+1), paper normalisation) every offset o of an interaction
 // list has one matrix T_o of size C x C, |T| <= 1/2, whose rows sum to at
 // most 137 over all 189 offsets.  Two things make it cheap here:
-//   * integer multiply-adds of 32 x 32 + 64 bits issue every 2 cycles and
-//     FP64 ones every 64, so a product of two 57-bit numbers (28-bit low
-//     parts, the product of those, below 2^-57, left out) takes 6 cycles, and
-//     sums are exact;
+//   * numbers of 57 and 54 bits as an integer high part and a 28-bit low part
+//     kept as a float: the product of the high parts is one 32 x 32 + 64-bit
+//     multiply-add (exact sums, ~5 cycles) and the two cross products are
+//     single-precision ones (1.2 cycles each; they start at 2^-28 of the
+//     product), 7.4 cycles where one FP64 multiply-add takes 64;
 //   * in the real layout a reflection x -> -x (y, z) only changes signs:
 //     T_(s o) = X_s T_o X_s with X_s diagonal, +-1, so that the up to eight
 //     offsets that differ in signs share one product:
@@ -17,9 +18,13 @@
 //     (class: the parities of a coefficient under the three reflections; Mt
 //     a Walsh-Hadamard transform of eight cells' multipoles).  189 products
 //     per cell become 56.
-// A CTA takes 32 target cells of one parity class, one per lane; warp k
-// computes the rows of class k, so that a lane needs one Mt value per column
-// and warp, and the matrix entries are the same for all lanes.
+// A CTA takes 32 target cells of one parity class; warp k computes the rows of
+// class k, so that all its products take their Mt from one transform index
+// per column.  Half of the lanes take half of the rows, each lane two targets:
+// a matrix entry and a transform value are loaded for several products each
+// (one target per lane loads an entry per product, which returns 32 lanes
+// even where all are the same: 8 cycles of the SM's shared memory for the 7.4
+// of its four sub-partitions' arithmetic).
 #include <math.h>
 
 #include <algorithm>
@@ -31,13 +36,19 @@
 
 namespace {
 
-constexpr int kTile = 16;     // columns staged at a time
+constexpr int kTile = 8;      // columns staged at a time
 constexpr int kOrbits = 56;   // offsets up to signs: {0..3}^3 without {0, 1}^3
-constexpr int kMaxRows = (MC_PMAX + 1) * (MC_PMAX + 1) + 8;
+constexpr int kMaxRows = (MC_PMAX + 1) * (MC_PMAX + 1) + 32;
 constexpr int kBitsT = 57, kBitsM = 54, kLimb = 28;
 
-struct M2LLayout {  // rows by class, every class padded to an even number
-  int start[8], count[8], rows;
+// tiles of the columns: at least two, so that an orbit's cells are known a
+// step before its first tile is loaded
+__host__ __device__ __forceinline__ int tiles_of(int C) { return C <= kTile ? 2 : (C + kTile - 1) / kTile; }
+
+// Rows by class; a class is two halves of `half` rows (the rows of the lower
+// and upper 16 lanes), each padded to an even number.
+struct M2LLayout {
+  int start[8], half[8], rows;
   short index[kMaxRows];  // real-layout index of a row, -1: padding
 };
 
@@ -48,20 +59,26 @@ M2LLayout m2l_layout(int p) {
   M2LLayout L;
   L.rows = 0;
   for (int c = 0; c < 8; c++) {
-    L.start[c] = L.rows;
+    short rows[kMaxRows];
+    int cnt = 0;
     for (int n = 0; n <= p; n++)
       for (int m = 0; m <= n; m++)
         for (int im = 0; im < (m ? 2 : 1); im++)
-          if (class_of(n, m, im) == c) L.index[L.rows++] = (short)(n * n + (m ? 2 * m - 1 : 0) + im);
-    L.count[c] = L.rows - L.start[c];
-    if (L.rows & 1) L.index[L.rows++] = -1;
+          if (class_of(n, m, im) == c) rows[cnt++] = (short)(n * n + (m ? 2 * m - 1 : 0) + im);
+    const int half = (cnt + 1) / 2, pad = (half + 1) / 2 * 2;
+    L.start[c] = L.rows;
+    L.half[c] = half;
+    for (int i = 0; i < 2 * pad; i++) {
+      const int r = (i / pad) * half + i % pad;
+      L.index[L.rows++] = i % pad < half && r < cnt ? rows[r] : (short)-1;
+    }
   }
   return L;
 }
 
 struct M2LArgs {
   int l, nl, h, pbc, p, nco, per_o;
-  int start[8], count[8], rows;
+  int start[8], half[8], rows;
   unsigned char ccol[kMaxRows];  // class of a column
   unsigned char orbit[kOrbits];  // |ox| | |oy| << 2 | |oz| << 4
   short index[kMaxRows];
@@ -78,6 +95,12 @@ __device__ __forceinline__ void decode(int k, int* n, int* m, int* im) {
   *im = (rem > 0 && (rem & 1) == 0) ? 1 : 0;
 }
 
+// v as h 2^28 + l: h, and l 2^-28 as a float
+__device__ __forceinline__ int2 limbs(long long v) {
+  const int l = ((int)v << (32 - kLimb)) >> (32 - kLimb);
+  return make_int2((int)((v - l) >> kLimb), __float_as_int((float)l * (1.0f / (float)(1 << kLimb))));
+}
+
 struct TableArgs {
   int p, rows;
   unsigned char orbit[kOrbits];
@@ -87,7 +110,7 @@ struct TableArgs {
 // T_o[row][col] from the scaled irregular harmonics of the integer offsets
 // (k_offset_table); entry (orbit, col, row)
 __global__ void k_m2l_tables(const __grid_constant__ TableArgs A, const double* __restrict__ otab, int2* __restrict__ T) {
-  const int p = A.p, C = (p + 1) * (p + 1), cpad = (C + kTile - 1) / kTile * kTile;
+  const int p = A.p, C = (p + 1) * (p + 1), cpad = tiles_of(C) * kTile;
   const int per = (2 * p + 1) * (2 * p + 2) / 2;
   const long long total = (long long)kOrbits * cpad * A.rows;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
@@ -118,8 +141,7 @@ __global__ void k_m2l_tables(const __grid_constant__ TableArgs A, const double* 
       v /= sqrt(f) * sqrt(g);
     }
     const long long w = __double2ll_rn(ldexp(v, kBitsT));
-    const int lo = ((int)w << (32 - kLimb)) >> (32 - kLimb);
-    T[i] = make_int2((int)((w - lo) >> kLimb), lo);
+    T[i] = limbs(w);
   }
 }
 
@@ -171,9 +193,29 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
 }
 
+// warp w's class: the two warps of a sub-partition (w, w + 4) take opposite
+// classes, whose rows add up to nearly a quarter of all (28 + 15 and 3 x 42 of
+// 169 at p = 12)
+__device__ __forceinline__ int class_of_warp(int w) { return w < 4 ? w : 11 - w; }
+
+// 8 bytes, or zeros
+__device__ __forceinline__ void cp_async8(void* dst, const void* src, bool valid) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  const int n = valid ? 8 : 0;
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+}
+
+struct M2LShared {
+  int2* T;        // [2][kTile rows]: table columns
+  int2* Mt;       // [2][kTile][8][32]: transform values
+  long long* raw; // [kTile][8][32]: the members' multipoles on their way there
+  int* cell;      // [2][8][32]: members' cells of an orbit (-1: none), by lane
+  int* shift;     // [2][8][32]: shifts to the task's unit
+};
+
 struct M2LTask {
-  int cls, oc;  // target class, orbit chunk; this lane's target (clamped):
-  int I[3], b[3];
+  int cls, oc;  // target class, orbit chunk
+  int I[3], b[3];  // the target this thread stages (clamped): halved coordinates, parities
   bool valid;
   int ecta;
 };
@@ -197,126 +239,159 @@ __device__ __forceinline__ int cell_at(const M2LTask& k, int ox, int oy, int oz,
 }
 
 // One CTA's task, as the warp that owns class w of NR rows sees it: every
-// warp stages its part of the next tile's Mt and table columns while it
-// computes the current one.
-template <int NR>
+// thread stages its target's part of the next tile's Mt and of the table
+// columns while its warp computes the current ones.
+template <int NR>  // rows of half a class
 __device__ __forceinline__ void m2l_task(const M2LArgs& A, const int2* __restrict__ T, const long long* __restrict__ M,
                                          const int* __restrict__ E, double* __restrict__ out, const M2LTask& k,
-                                         int2* sT, int2* sM, int w, int lane) {
-  const int C = (A.p + 1) * (A.p + 1), tiles = (C + kTile - 1) / kTile, h = A.h, ncl = A.nl * A.nl * A.nl;
+                                         const M2LShared& S, int t0, int w, int lane) {
+  constexpr int NT = 2;
+  const int C = (A.p + 1) * (A.p + 1), tiles = tiles_of(C), h = A.h, ncl = A.nl * A.nl * A.nl;
   const int ob = k.oc * A.per_o, oe = min(kOrbits, ob + A.per_o);
   const int steps = (oe - ob) * tiles, tsz = kTile * A.rows;
-  long long hh[NR > 0 ? NR : 1], x[NR > 0 ? NR : 1];
+  const int tid = 32 * w + lane, cls = class_of_warp(w);
+  long long hh[NR > 0 ? NR : 1][NT];
+  float x[NR > 0 ? NR : 1][NT];
 #pragma unroll
-  for (int r = 0; r < NR; r++) hh[r] = x[r] = 0;
-  int cell[8], sh[8];
-  long long v[2][8];
-  auto load = [&](int s) {  // this thread's two columns of tile s
-    const int o = ob + s / tiles, tile = s % tiles;
-    if (tile == 0) {
-      const int a[3] = {A.orbit[o] & 3, (A.orbit[o] >> 2) & 3, (A.orbit[o] >> 4) & 3};
+  for (int r = 0; r < NR; r++)
 #pragma unroll
-      for (int g = 0; g < 8; g++) {
-        bool ok = k.valid;
-        int of[3];
-#pragma unroll
-        for (int d = 0; d < 3; d++) {
-          const int neg = (g >> (2 - d)) & 1;
-          if ((a[d] == 0 && neg) || (a[d] == 3 && neg != k.b[d])) ok = false;
-          of[d] = neg ? -a[d] : a[d];
-        }
-        cell[g] = ok ? cell_at(k, of[0], of[1], of[2], h, A.pbc != 0) : -1;
-        sh[g] = cell[g] >= 0 ? min(63, k.ecta - E[cell[g]]) : 63;
-      }
+    for (int t = 0; t < NT; t++) {
+      hh[r][t] = 0;
+      x[r][t] = 0.0f;
     }
+  int lo = ob, lt = 0;  // orbit and tile to load next
+  // member w (signs of its offset: bits x 4, y 2, z 1) of an orbit
+  auto members = [&](int o) {
+    int of[3];
+    bool ok = k.valid;
 #pragma unroll
-    for (int u = 0; u < 2; u++) {
-      const int col = tile * kTile + 2 * w + u;
-#pragma unroll
-      for (int g = 0; g < 8; g++) v[u][g] = (cell[g] >= 0 && col < C) ? __ldg(&M[(size_t)col * ncl + cell[g]]) : 0ll;
+    for (int d = 0; d < 3; d++) {
+      const int a = (A.orbit[o] >> (2 * d)) & 3, neg = (w >> (2 - d)) & 1;
+      if ((a == 0 && neg) || (a == 3 && neg != k.b[d])) ok = false;
+      of[d] = neg ? -a : a;
     }
-    const char* src = reinterpret_cast<const char*>(T + ((size_t)o * tiles + tile) * tsz);
-    char* dst = reinterpret_cast<char*>(sT + (s & 1) * tsz);
-    for (int i = 16 * (32 * w + lane); i < tsz * (int)sizeof(int2); i += 16 * 256) cp_async16(dst + i, src + i);
+    const int c = ok ? cell_at(k, of[0], of[1], of[2], h, A.pbc != 0) : -1;
+    const int i = ((o & 1) * 8 + w) * 32 + lane;
+    S.cell[i] = c;
+    S.shift[i] = c >= 0 ? min(63, k.ecta - E[c]) : 0;
+  };
+  // column w of the next tile: its lane's target's members, and the table
+  auto load = [&](int s) {
+    const int col = lt * kTile + w;
+    const long long* Mc = M + (size_t)min(col, C - 1) * ncl;
+    const int* cl = S.cell + (lo & 1) * 256 + lane;
+#pragma unroll
+    for (int g = 0; g < 8; g++) {
+      const int c = cl[32 * g];
+      cp_async8(&S.raw[(w * 8 + g) * 32 + lane], &Mc[max(c, 0)], c >= 0 && col < C);
+    }
+    const char* src = reinterpret_cast<const char*>(T + ((size_t)lo * tiles + lt) * tsz);
+    char* dst = reinterpret_cast<char*>(S.T + (s & 1) * tsz);
+    for (int i = 16 * tid; i < tsz * (int)sizeof(int2); i += 16 * 256) cp_async16(dst + i, src + i);
     asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  auto store = [&](int s) {
-    int2* dst = sM + (size_t)(s & 1) * kTile * 8 * 32;
-#pragma unroll
-    for (int u = 0; u < 2; u++) {
-#pragma unroll
-      for (int g = 0; g < 8; g++) v[u][g] >>= sh[g];
-#pragma unroll
-      for (int b = 1; b < 8; b <<= 1)
-#pragma unroll
-        for (int g = 0; g < 8; g++)
-          if (!(g & b)) {
-            const long long lo = v[u][g], hi = v[u][g | b];
-            v[u][g] = lo + hi;
-            v[u][g | b] = lo - hi;
-          }
-      // transform index d = (x, y, z) bits (4, 2, 1) of the member signs
-#pragma unroll
-      for (int d = 0; d < 8; d++) {
-        const long long t = v[u][d];
-        const int l = ((int)t << (32 - kLimb)) >> (32 - kLimb);
-        dst[((2 * w + u) * 8 + d) * 32 + lane] = make_int2((int)((t - l) >> kLimb), l);
-      }
+    if (++lt == tiles) {
+      lt = 0;
+      lo++;
+    } else if (lt == tiles - 1 && lo + 1 < oe) {
+      members(lo + 1);  // read from the step after next on
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
   };
+  int so = ob, stl = 0;  // orbit and tile to transform next
+  auto store = [&](int s) {
+    // (each thread reads back what it copied itself)
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    int2* dst = S.Mt + (size_t)((s & 1) * kTile + w) * 8 * 32 + lane;
+    const int* sh = S.shift + (so & 1) * 256 + lane;
+    long long v[8];
+#pragma unroll
+    for (int g = 0; g < 8; g++) v[g] = S.raw[(w * 8 + g) * 32 + lane] >> sh[32 * g];
+#pragma unroll
+    for (int b = 1; b < 8; b <<= 1)
+#pragma unroll
+      for (int g = 0; g < 8; g++)
+        if (!(g & b)) {
+          const long long p = v[g], q = v[g | b];
+          v[g] = p + q;
+          v[g | b] = p - q;
+        }
+    // transform index d = (x, y, z) bits (4, 2, 1) of the member signs
+#pragma unroll
+    for (int d = 0; d < 8; d++) dst[d * 32] = limbs(v[d]);
+    if (++stl == tiles) {
+      stl = 0;
+      so++;
+    }
+  };
+  // the cross products' large part, carried over every 64 columns
+  auto carry = [&]() {
+#pragma unroll
+    for (int r = 0; r < NR; r++)
+#pragma unroll
+      for (int t = 0; t < NT; t++) {
+        // multiples of 2^11, read off the last bits of the sum with 3 2^33
+        // (|x| < 2^35; a conversion to 64 bits would use the FP64 pipe)
+        const float f = x[r][t] + 25769803776.0f;
+        hh[r][t] = fx_wide(__float_as_int(f) - 0x50C00000, 2048, hh[r][t]);
+        x[r][t] -= f - 25769803776.0f;
+      }
+  };
+  members(ob);
+  cta_sync();
   load(0);
   store(0);
   cta_sync();
-  int held = 0;
+  int tile = 0;
   for (int s = 0; s < steps; s++) {
     if (s + 1 < steps) load(s + 1);
     if constexpr (NR > 0) {
-      const int tile = s % tiles;
-      const int2* t0 = sT + (s & 1) * tsz + A.start[w];
-      const int2* m0 = sM + (size_t)(s & 1) * kTile * 8 * 32 + lane;
-#pragma unroll 1
+      const int2* tt = S.T + (s & 1) * tsz + A.start[cls] + (lane >> 4) * ((NR + 1) / 2 * 2);
+      const int2* m0 = S.Mt + (size_t)(s & 1) * kTile * 8 * 32 + (lane & 15);
+#pragma unroll 2
       for (int c = 0; c < kTile; c++) {
-        const int d = w ^ A.ccol[tile * kTile + c];
-        const int2 m = m0[(c * 8 + d) * 32];
-        const int4* t = reinterpret_cast<const int4*>(t0 + c * A.rows);
+        const int d = cls ^ A.ccol[tile * kTile + c];
+        int mh[NT];
+        float ml[NT], mf[NT];
 #pragma unroll
-        for (int r = 0; r < NR; r += 2) {
-          const int4 q = t[r / 2];
-          hh[r] = fx_wide(q.x, m.x, hh[r]);
-          x[r] = fx_wide(q.x, m.y, x[r]);
-          x[r] = fx_wide(q.y, m.x, x[r]);
-          if (r + 1 < NR) {
-            hh[r + 1] = fx_wide(q.z, m.x, hh[r + 1]);
-            x[r + 1] = fx_wide(q.z, m.y, x[r + 1]);
-            x[r + 1] = fx_wide(q.w, m.x, x[r + 1]);
+        for (int t = 0; t < NT; t++) {
+          const int2 m = m0[(c * 8 + d) * 32 + 16 * t];
+          mh[t] = m.x;
+          ml[t] = __int_as_float(m.y);
+          mf[t] = (float)m.x;
+        }
+        const int4* tr = reinterpret_cast<const int4*>(tt + c * A.rows);
+#pragma unroll
+        for (int r = 0; r < NR; r++) {
+          const int4 q = tr[r / 2];
+          const int th = r & 1 ? q.z : q.x;
+          const float tl = __int_as_float(r & 1 ? q.w : q.y), tf = (float)th;
+#pragma unroll
+          for (int t = 0; t < NT; t++) {
+            hh[r][t] = fx_wide(th, mh[t], hh[r][t]);
+            x[r][t] = fmaf(tf, ml[t], x[r][t]);
+            x[r][t] = fmaf(tl, mf[t], x[r][t]);
           }
         }
       }
-      // 64 columns of cross products stay below 2^63: carry them over
-      if (++held == 64 / kTile) {
-        held = 0;
-#pragma unroll
-        for (int r = 0; r < NR; r++) {
-          hh[r] += x[r] >> kLimb;
-          x[r] &= (1ll << kLimb) - 1;
-        }
-      }
+      if (++tile == tiles) tile = 0;
+      if ((s & (64 / kTile - 1)) == 64 / kTile - 1) carry();
     }
     if (s + 1 < steps) store(s + 1);
     cta_sync();
   }
   if constexpr (NR > 0) {
-    if (k.valid) {
-      const int i = 2 * k.I[0] + k.b[0], j = 2 * k.I[1] + k.b[1], kk = 2 * k.I[2] + k.b[2];
+    const double unit = ldexp(1.0, k.ecta);
+    const int h3 = h * h * h;
+#pragma unroll
+    for (int t = 0; t < NT; t++) {
+      const int ii = t0 + 16 * t + (lane & 15);
+      if (ii >= h3) continue;
+      const int i = 2 * (ii / (h * h)) + k.b[0], j = 2 * ((ii / h) % h) + k.b[1], kk = 2 * (ii % h) + k.b[2];
       double* o = out + ((size_t)((i * A.nl + j) * A.nl + kk) * A.nco + k.oc) * C;
-      const double unit = ldexp(1.0, k.ecta);
 #pragma unroll
       for (int r = 0; r < NR; r++) {
-        hh[r] += x[r] >> kLimb;
-        x[r] &= (1ll << kLimb) - 1;
-        const double sum = (double)hh[r] + (double)x[r] * (1.0 / (double)(1 << kLimb));
-        o[A.index[A.start[w] + r]] = sum * A.scale[A.start[w] + r] * unit;
+        const int row = A.start[cls] + (lane >> 4) * ((NR + 1) / 2 * 2) + r;
+        const double sum = (double)hh[r][t] + (double)x[r][t];
+        if (A.index[row] >= 0) o[A.index[row]] = sum * A.scale[row] * unit;
       }
     }
   }
@@ -324,20 +399,25 @@ __device__ __forceinline__ void m2l_task(const M2LArgs& A, const int2* __restric
 
 }  // namespace
 
-__global__ void __launch_bounds__(256, 1)
+__global__ void __launch_bounds__(256, 2)
     k_m2l_fix(const __grid_constant__ M2LArgs A, const int2* __restrict__ T, const long long* __restrict__ M,
               const int* __restrict__ E, double* __restrict__ out) {
   extern __shared__ int4 dyn4[];
   __shared__ int s_emax;
-  int2* sT = reinterpret_cast<int2*>(dyn4);
-  int2* sM = sT + 2 * kTile * A.rows;
+  constexpr int kTargets = 32;
+  M2LShared S;
+  S.T = reinterpret_cast<int2*>(dyn4);
+  S.Mt = S.T + 2 * kTile * A.rows;
+  S.raw = reinterpret_cast<long long*>(S.Mt + 2 * kTile * 8 * 32);
+  S.cell = reinterpret_cast<int*>(S.raw + kTile * 8 * 32);
+  S.shift = S.cell + 2 * 8 * 32;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int h = A.h, h3 = h * h * h, chunks = (h3 + 31) / 32;
+  const int h = A.h, h3 = h * h * h, chunks = (h3 + kTargets - 1) / kTargets;
   M2LTask k;
   k.oc = blockIdx.x % A.nco;
   const int tk = blockIdx.x / A.nco;
   k.cls = tk / chunks;
-  const int ii = (tk % chunks) * 32 + lane;
+  const int t0 = (tk % chunks) * kTargets, ii = t0 + threadIdx.x % kTargets;
   k.valid = ii < h3;
   const int r = min(ii, h3 - 1);
   k.I[0] = r / (h * h);
@@ -349,7 +429,7 @@ __global__ void __launch_bounds__(256, 1)
   if (threadIdx.x == 0) s_emax = -4096;
   __syncthreads();
   int e = -4096;
-  for (int q = w; q < 216; q += 8) {
+  for (int q = threadIdx.x / kTargets; q < 216; q += 256 / kTargets) {
     const int ox = q / 36 - 2 - k.b[0], oy = (q / 6) % 6 - 2 - k.b[1], oz = q % 6 - 2 - k.b[2];
     if (ox >= -1 && ox <= 1 && oy >= -1 && oy <= 1 && oz >= -1 && oz <= 1) continue;
     const int c = cell_at(k, ox, oy, oz, h, A.pbc != 0);
@@ -359,24 +439,28 @@ __global__ void __launch_bounds__(256, 1)
   if (lane == 0) atomicMax(&s_emax, e);
   __syncthreads();
   k.ecta = s_emax;
-  switch (A.count[w]) {
-    case 1: m2l_task<1>(A, T, M, E, out, k, sT, sM, w, lane); break;
-    case 3: m2l_task<3>(A, T, M, E, out, k, sT, sM, w, lane); break;
-    case 6: m2l_task<6>(A, T, M, E, out, k, sT, sM, w, lane); break;
-    case 10: m2l_task<10>(A, T, M, E, out, k, sT, sM, w, lane); break;
-    case 15: m2l_task<15>(A, T, M, E, out, k, sT, sM, w, lane); break;
-    case 21: m2l_task<21>(A, T, M, E, out, k, sT, sM, w, lane); break;
-    case 28: m2l_task<28>(A, T, M, E, out, k, sT, sM, w, lane); break;
-    case 36: m2l_task<36>(A, T, M, E, out, k, sT, sM, w, lane); break;
-    default: m2l_task<0>(A, T, M, E, out, k, sT, sM, w, lane); break;
+  // half of 1, 3, 6, 10, 15, 21, 28, 36 rows
+#define MC_M2L_ROWS(NR_) \
+  case NR_: m2l_task<NR_>(A, T, M, E, out, k, S, t0, w, lane); break;
+  switch (A.half[class_of_warp(w)]) {
+    MC_M2L_ROWS(1)
+    MC_M2L_ROWS(2)
+    MC_M2L_ROWS(3)
+    MC_M2L_ROWS(5)
+    MC_M2L_ROWS(8)
+    MC_M2L_ROWS(11)
+    MC_M2L_ROWS(14)
+    MC_M2L_ROWS(18)
+    MC_M2L_ROWS(0)
   }
+#undef MC_M2L_ROWS
 }
 
 __global__ void k_offset_table(int p, double* __restrict__ out);
 
 size_t m2l_table_bytes(int p) {
   const int C = (p + 1) * (p + 1);
-  return sizeof(int2) * (size_t)kOrbits * ((C + kTile - 1) / kTile * kTile) * m2l_layout(p).rows;
+  return sizeof(int2) * (size_t)kOrbits * tiles_of(C) * kTile * m2l_layout(p).rows;
 }
 
 static void orbits(unsigned char* o) {
@@ -409,8 +493,8 @@ static double sfac(int n, int m) {
 
 int m2l_chunks(int nl, int sms) {
   const int h = nl / 2, tasks = 8 * ((h * h * h + 31) / 32);
-  // at least six tasks per SM (one CTA each), so that the last wave is short
-  return std::max(1, std::min(kOrbits, (6 * sms + tasks - 1) / tasks));
+  // at least twelve tasks per SM (two at a time), so that the last wave is short
+  return std::max(1, std::min(kOrbits, (12 * sms + tasks - 1) / tasks));
 }
 
 cudaError_t m2l_fix_level(int p, int l, double w, bool pbc, int sms, const void* table, const double* K, long long* M,
@@ -433,7 +517,7 @@ cudaError_t m2l_fix_level(int p, int l, double w, bool pbc, int sms, const void*
   A.rows = L.rows;
   for (int c = 0; c < 8; c++) {
     A.start[c] = L.start[c];
-    A.count[c] = L.count[c];
+    A.half[c] = L.half[c];
   }
   orbits(A.orbit);
   std::fill(A.ccol, A.ccol + kMaxRows, 0);
@@ -458,10 +542,10 @@ cudaError_t m2l_fix_level(int p, int l, double w, bool pbc, int sms, const void*
   cudaError_t e = cudaFuncSetAttribute(k_m2l_convert, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm);
   if (e != cudaSuccess) return e;
   k_m2l_convert<<<(ncl + 31) / 32, 256, csm, st>>>(V, K, M, E);
-  const size_t smem = sizeof(int2) * 2 * ((size_t)kTile * L.rows + kTile * 8 * 32);
+  const int chunks = (h * h * h + 31) / 32;
+  const size_t smem = sizeof(int2) * (2 * (size_t)kTile * L.rows + 3 * kTile * 8 * 32) + sizeof(int) * 4 * 8 * 32;
   e = cudaFuncSetAttribute(k_m2l_fix, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const int chunks = (h * h * h + 31) / 32;
   k_m2l_fix<<<8 * chunks * A.nco, 256, smem, st>>>(A, (const int2*)table, M, E, A.nco > 1 ? scratch : Lout);
   e = cudaGetLastError();
   if (e == cudaSuccess && A.nco > 1) e = fix_reduce(ncl, A.nco, C, sms, scratch, Lout, st);
