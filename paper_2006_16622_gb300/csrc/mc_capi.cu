@@ -37,9 +37,13 @@ __global__ void k_max_int(int, const int*, int*);
 __global__ void k_p2l_level(const McSys*, int, int, double*);
 __global__ void k_reduce_chunks(int, int, int, const double*, double*);
 __global__ void k_box_multipole(const McSys*, int, double*);
-__global__ void k_far_finish(const McSys*, int, const double*);
 __global__ void k_energy_particles(const McSys*, double*);
 __global__ void k_energy_finish(const McSys*, int, const double*, double*);
+__global__ void k_far_apply(const McSys*, const double*);
+cudaError_t m2m_table(int, double*, cudaStream_t);
+cudaError_t m2m_level(int, int, double, const double*, const double*, double*, cudaStream_t);
+__global__ void k_energy_dot(size_t, int, const double*, const double*, double*);
+__global__ void k_energy_sum(const McSys*, int, int, const double*, double*);
 __global__ void k_lattice_sums(int, double*);
 __global__ void k_far_operator(int, double, const double*, double*);
 __global__ void k_p2m_level(const McSys*, int, int, double*);
@@ -65,6 +69,7 @@ struct mc_ctx {
   unsigned long long* d_prof;  // MC_PROF_COUNTERS timers when profiling is on, else null
   int schedule;                // MC_SCHEDULE_*
   double* d_mpole;             // per-level multipoles (fast setup), allocated on first use
+  double* d_m2m;               // children-to-cell matrix of this order
   double* d_otab;              // offset harmonics table (FP64 fast setup)
   const void* m2l_table;       // this order's matrices (shared, see m2l_table_get)
   long long* d_mfix;           // a level's multipoles as integers, their units
@@ -113,7 +118,7 @@ FixSource fix_source(const McSys& h) {
 }
 FixPass fix_pass(const mc_ctx* c, int l, bool irregular) {
   const McSys& h = c->h;
-  return FixPass{h.L, l, h.p, irregular, h.bc == MC_BC_PBC, h.a, c->qexp, 1};
+  return FixPass{h.L, l, h.p, irregular, h.bc == MC_BC_PBC, h.a, c->qexp, 1, nullptr};
 }
 // chunks of one fixed-point pass, as many as the scratch holds
 int fix_chunks_for(const McSys& h, int sms, int l, bool irregular, size_t max_doubles) {
@@ -194,6 +199,40 @@ int launch_chain(mc_ctx* c, RunParams& rp) {
   return MC_OK;
 }
 
+// sums of one fixed-point pass over level l into dst (C per cell)
+int fix_level(mc_ctx* c, int l, bool irregular, double* dst) {
+  const McSys& h = c->h;
+  const int ncl = 1 << (3 * (l - 1));
+  FixPass ps = fix_pass(c, l, irregular);
+  ps.nchunk = fix_chunks_for(h, c->sms, l, irregular, c->scratch_doubles);
+  CK(fix_launch(ps, fix_source(h), ps.nchunk > 1 ? c->d_scratch : dst, c->stream));
+  if (ps.nchunk > 1) CK(fix_reduce(ncl, ps.nchunk, h.C, c->sms, c->d_scratch, dst, c->stream));
+  return MC_OK;
+}
+
+// H = G K, and the dipole, of a box multipole that is in place (kh null) or in
+// kh with the dipole behind it
+int far_apply(mc_ctx* c, const double* kh) {
+  k_far_apply<<<(c->h.C + 31) / 32, 256, 0, c->stream>>>(c->d_sys, kh);
+  CK(cudaGetLastError());
+  return MC_OK;
+}
+
+// chunks of the box multipole's sum over the charges: four charges per warp
+// step, at least four steps
+int box_chunks(const McSys& h, int sms) { return std::min(8 * sms, std::max(1, h.n / 16)); }
+
+// the box multipole K and the dipole from the charges, and H = G K
+int setup_far(mc_ctx* c) {
+  const int nch = box_chunks(c->h, c->sms), n = c->h.C + 3;
+  double* kh = c->d_scratch + (size_t)nch * n;
+  k_box_multipole<<<grid_for(c->sms, nch, MC_WARPS), MC_THREADS, 0, c->stream>>>(c->d_sys, nch,
+                                                                                c->d_scratch);
+  CK(cudaGetLastError());
+  CK(fix_reduce(1, nch, n, c->sms, c->d_scratch, kh, c->stream));
+  return far_apply(c, kh);
+}
+
 int run_setup(mc_ctx* c) {
   McSys& h = c->h;
   const int C = h.C;
@@ -204,69 +243,46 @@ int run_setup(mc_ctx* c) {
   for (int l = h.lmin; l <= h.L; l++) {
     const int nl = h.lev_n[l], ncl = nl * nl * nl;
     double* dst = h.Lhat + (size_t)h.lev_off[l] * C;
-    int nchunk;
     if (c->fixed) {
-      FixPass ps = fix_pass(c, l, true);
-      ps.nchunk = nchunk = fix_chunks_for(h, c->sms, l, true, c->scratch_doubles);
-      CK(fix_launch(ps, fix_source(h), nchunk > 1 ? c->d_scratch : dst, c->stream));
-    } else {
-      nchunk = chunks_for_level(h, c->sms, l, c->scratch_doubles);
-      k_p2l_level<<<grid_for(c->sms, ncl * nchunk, MC_WARPS), MC_THREADS, 0, c->stream>>>(
-          c->d_sys, l, nchunk, nchunk > 1 ? c->d_scratch : dst);
-      CK(cudaGetLastError());
+      const int rc = fix_level(c, l, true, dst);
+      if (rc != MC_OK) return rc;
+      continue;
     }
+    const int nchunk = chunks_for_level(h, c->sms, l, c->scratch_doubles);
+    k_p2l_level<<<grid_for(c->sms, ncl * nchunk, MC_WARPS), MC_THREADS, 0, c->stream>>>(
+        c->d_sys, l, nchunk, nchunk > 1 ? c->d_scratch : dst);
+    CK(cudaGetLastError());
     if (nchunk > 1) CK(fix_reduce(ncl, nchunk, C, c->sms, c->d_scratch, dst, c->stream));
   }
-  // K, dipole, H = G K
-  const int nch = std::min<int>(1024, std::max<int>(1, h.n / 64));
-  k_box_multipole<<<grid_for(c->sms, nch, MC_WARPS), MC_THREADS, 0, c->stream>>>(c->d_sys, nch,
-                                                                                c->d_scratch);
-  CK(cudaGetLastError());
-  k_far_finish<<<1, 256, 0, c->stream>>>(c->d_sys, nch, c->d_scratch);
-  CK(cudaGetLastError());
-  return MC_OK;
+  return setup_far(c);
 }
 
-// FMM-variant initialisation (fast mode): multipoles of every level, then
-// multipole-to-local over the interaction lists
-// per-level multipoles (Eq. 4) of every cell into d_mpole (allocated on
-// first use): the fast setup's first pass and Alg. M.3
+// Multipoles (Eq. 4) of every cell into d_mpole (allocated on first use): the
+// fast setup's first pass and Alg. M.3.  The finest level's from the charges,
+// the others' from their children, and with periodic boundaries (lmin = 2)
+// the box multipole K likewise, then the dipole and H = G K.
 int p2m_levels(mc_ctx* c) {
   McSys& h = c->h;
   const int C = h.C;
   if (!c->d_mpole &&
       dalloc(c, (void**)&c->d_mpole, sizeof(double) * (size_t)std::max(1, h.ncell_total) * C) != MC_OK)
     return MC_ERR_NOMEM;
-  for (int l = h.lmin; l <= h.L; l++) {
-    const int nl = h.lev_n[l], ncl = nl * nl * nl;
-    const int f = 1 << (h.L - l);
-    double* M = c->d_mpole + (size_t)h.lev_off[l] * C;
-    long long nchunk = std::min<long long>((long long)f * f * f,
-                                           std::max<long long>(1, (4LL * c->sms * MC_WARPS + ncl - 1) / ncl));
-    if (nchunk > 1 && (size_t)(ncl * nchunk * C) > c->scratch_doubles)
-      nchunk = std::max<long long>(1, (long long)(c->scratch_doubles / ((size_t)ncl * C)));
-    const long long ntask = (long long)ncl * nchunk;
-    k_p2m_level<<<grid_for(c->sms, (size_t)ntask, MC_WARPS), MC_THREADS, 0, c->stream>>>(
-        c->d_sys, l, (int)nchunk, nchunk > 1 ? c->d_scratch : M);
-    CK(cudaGetLastError());
-    if (nchunk > 1) {
-      k_reduce_chunks<<<grid_for(c->sms, (size_t)ncl * C, 256), 256, 0, c->stream>>>(
-          ncl, (int)nchunk, C, c->d_scratch, M);
-      CK(cudaGetLastError());
-    }
+  if (!c->d_m2m) {
+    if (dalloc(c, (void**)&c->d_m2m, sizeof(double) * (size_t)C * C) != MC_OK) return MC_ERR_NOMEM;
+    CK(m2m_table(h.p, c->d_m2m, c->stream));
   }
-  return MC_OK;
-}
-
-// the box multipole K, dipole and H = G K
-int setup_far(mc_ctx* c) {
-  const int nch = std::min<int>(1024, std::max<int>(1, c->h.n / 64));
-  k_box_multipole<<<grid_for(c->sms, nch, MC_WARPS), MC_THREADS, 0, c->stream>>>(c->d_sys, nch,
-                                                                                c->d_scratch);
-  CK(cudaGetLastError());
-  k_far_finish<<<1, 256, 0, c->stream>>>(c->d_sys, nch, c->d_scratch);
-  CK(cudaGetLastError());
-  return MC_OK;
+  if (h.L >= h.lmin) {
+    // finest cells hold one unit each, so one task (warp) per cell
+    double* M = c->d_mpole + (size_t)h.lev_off[h.L] * C;
+    k_p2m_level<<<grid_for(c->sms, (size_t)h.ncellL, MC_WARPS), MC_THREADS, 0, c->stream>>>(c->d_sys, h.L, 1, M);
+    CK(cudaGetLastError());
+  }
+  for (int l = h.L - 1; l >= h.lmin; l--)
+    CK(m2m_level(h.p, h.lev_n[l], h.lev_w[l + 1], c->d_m2m, c->d_mpole + (size_t)h.lev_off[l + 1] * C,
+                 c->d_mpole + (size_t)h.lev_off[l] * C, c->stream));
+  if (h.bc != MC_BC_PBC || h.p < 1) return setup_far(c);
+  CK(m2m_level(h.p, 1, h.lev_w[2], c->d_m2m, c->d_mpole + (size_t)h.lev_off[2] * C, h.Khat, c->stream));
+  return far_apply(c, nullptr);
 }
 
 // the state of one method on the device: method 0 (local) or 1 (multipole)
@@ -281,8 +297,7 @@ int set_method(mc_ctx* c, int method) {
 int run_setup_mm(mc_ctx* c) {
   int rc = p2m_levels(c);
   if (rc != MC_OK) return rc;
-  if ((rc = set_method(c, 1)) != MC_OK) return rc;
-  return setup_far(c);
+  return set_method(c, 1);
 }
 
 // The matrices of the fixed-point translations depend on p only: one table
@@ -369,20 +384,45 @@ int m2l_levels(mc_ctx* c) {
 }
 
 int run_setup_fmm(mc_ctx* c) {
-  McSys& h = c->h;
-  int rc = p2m_levels(c);
-  if (rc == MC_OK) rc = m2l_levels(c);
-  if (rc != MC_OK) return rc;
-  const int nch = std::min<int>(1024, std::max<int>(1, h.n / 64));
-  k_box_multipole<<<grid_for(c->sms, nch, MC_WARPS), MC_THREADS, 0, c->stream>>>(c->d_sys, nch,
-                                                                                c->d_scratch);
-  CK(cudaGetLastError());
-  k_far_finish<<<1, 256, 0, c->stream>>>(c->d_sys, nch, c->d_scratch);
-  CK(cudaGetLastError());
-  return MC_OK;
+  const int rc = p2m_levels(c);
+  return rc == MC_OK ? m2l_levels(c) : rc;
 }
 
-int energy_into(mc_ctx* c, double* d_dst) {
+// chunks of the expansions' part of the energy on one level
+int energy_chunks(const McSys& h, int sms, int l, bool irregular) {
+  return fix_chunks(h.L, l, irregular, sms, (double)h.n / (double)h.ncellL, h.p);
+}
+
+// Total energy from the current expansions and positions into d_dst.  The
+// expansions' part is a contraction cell by cell: of the local expansions
+// with the cells' multipoles, or (multipole method) of the multipoles with
+// the Alg. L.3 sums, since sum_i q_i sum_c M_c It(r_i - R_c) over the listed
+// cells c is sum_c M_c (sum of q_i It over the charges whose lists hold c).
+// `mpole`: d_mpole holds the multipoles of the current positions.
+int energy_into(mc_ctx* c, double* d_dst, bool mpole) {
+  const McSys& h = c->h;
+  if (c->fixed && !h.lj_on) {
+    const int nb = fix_near_blocks(h.L, c->sms), nnear = 8 * nb;
+    CK(fix_near(h.L, h.bc == MC_BC_PBC, h.a, fix_source(h), nb, c->d_scratch, c->stream));
+    int nexp = 0;
+    if (h.method == 0 && mpole && c->d_mpole) {
+      nexp = 2 * c->sms;
+      k_energy_dot<<<nexp, 256, 0, c->stream>>>((size_t)h.ncell_total * h.C, h.C, c->d_mpole, h.Lhat,
+                                                c->d_scratch + nnear);
+      CK(cudaGetLastError());
+    } else {
+      for (int l = h.lmin; l <= h.L; l++) {
+        FixPass ps = fix_pass(c, l, h.method == 1);
+        ps.nchunk = energy_chunks(h, c->sms, l, h.method == 1);
+        ps.dot = (h.method == 1 ? h.Mhat : h.Lhat) + (size_t)h.lev_off[l] * h.C;
+        CK(fix_launch(ps, fix_source(h), c->d_scratch + nnear + nexp, c->stream));
+        nexp += (1 << (3 * (l - 1))) * ps.nchunk;
+      }
+    }
+    k_energy_sum<<<1, 1024, 0, c->stream>>>(c->d_sys, nnear, nexp, c->d_scratch, d_dst);
+    CK(cudaGetLastError());
+    return MC_OK;
+  }
   const int blocks = c->sms * 2;
   const int nw = blocks * MC_WARPS;
   k_energy_particles<<<blocks, MC_THREADS, 0, c->stream>>>(c->d_sys, c->d_scratch);
@@ -642,8 +682,16 @@ int mc_init(mc_ctx** out, int64_t n, const double* pos, const double* q, double 
     const size_t nco = (size_t)(c->fixed ? m2l_chunks(h.lev_n[l], c->sms) : m2l_offset_chunks(h.lev_n[l], c->sms));
     if (nco > 1) need = std::max(need, std::min(ncl * nco * C, kScratchCap));
   }
-  need = std::max(need, (size_t)1024 * (C + 3));
+  need = std::max(need, (size_t)(box_chunks(h, c->sms) + 1) * (C + 3));
   need = std::max(need, (size_t)c->sms * 2 * MC_WARPS);
+  if (c->fixed) {
+    // the energy's partials: near pairs, then the expansions of every level
+    size_t e = 8 * (size_t)fix_near_blocks(levels, c->sms) + 2 * (size_t)c->sms;
+    for (int l = h.lmin; l <= levels; l++)
+      e += ((size_t)1 << (3 * (l - 1))) *
+           std::max(energy_chunks(h, c->sms, l, false), energy_chunks(h, c->sms, l, true));
+    need = std::max(need, e);
+  }
   c->scratch_doubles = need;
   DA(c->d_scratch, sizeof(double) * need);
 
@@ -687,7 +735,7 @@ int mc_setup(mc_ctx* c, int mode) {
     if (rc == MC_OK) rc = mode == MC_SETUP_FMM ? run_setup_fmm(c) : run_setup(c);
   }
   if (rc != MC_OK) return rc;
-  rc = energy_into(c, c->h.energy);
+  rc = energy_into(c, c->h.energy, mode == MC_SETUP_FMM);
   if (rc != MC_OK) return rc;
   CK(cudaStreamSynchronize(c->stream));
   c->setup_done = 1;
@@ -799,7 +847,7 @@ int mc_run(mc_ctx* c, int64_t n_steps, uint64_t seed, double beta, double half_w
       // full FP64 re-setup from the current positions; drift = running - fresh
       double run_e = 0.0, fresh = 0.0;
       if ((rc = c->h.method ? run_setup_mm(c) : run_setup(c)) != MC_OK) break;
-      if ((rc = energy_into(c, c->d_energy_tmp)) != MC_OK) break;
+      if ((rc = energy_into(c, c->d_energy_tmp, false)) != MC_OK) break;
       if (cudaMemcpyAsync(&run_e, c->h.energy, sizeof(double), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess ||
           cudaMemcpyAsync(&fresh, c->d_energy_tmp, sizeof(double), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess ||
           cudaStreamSynchronize(c->stream) != cudaSuccess) {
@@ -855,7 +903,7 @@ int mc_energy_fresh(mc_ctx* c, double* e) {
   if (!c || !e) return MC_ERR_ARG;
   if (!c->setup_done) return MC_ERR_STATE;
   CK(cudaSetDevice(c->dev));
-  int rc = energy_into(c, c->d_energy_tmp);
+  int rc = energy_into(c, c->d_energy_tmp, false);
   if (rc != MC_OK) return rc;
   CK(cudaStreamSynchronize(c->stream));
   CK(cudaMemcpy(e, c->d_energy_tmp, sizeof(double), cudaMemcpyDeviceToHost));

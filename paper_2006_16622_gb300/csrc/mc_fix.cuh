@@ -31,9 +31,11 @@
 #define MC_FIX_WARPS 4   // warps that share the columns
 #define MC_FIX_STEPS 34  // most recurrence steps of one warp (p = 15)
 // groups of 32 charges between two flushes of a lane's sums: one term is at
-// most 2^57, so 56 stay below 2^63, and after the shift by 5 the sum over
-// the 32 lanes does too
-#define MC_FIX_FLUSH 56
+// most 2^58, so 28 stay below 2^63, and after the shift by 5 the sum over
+// the 32 lanes does too (a bit more for the terms would double the flushes,
+// 3 % of the kernel)
+#define MC_FIX_FLUSH 28
+#define MC_FIX_PHASE 2  // cos m phi, sin m phi enter the terms as multiples of 2^-60
 
 // value h 2^32 + l with signed l, so that every partial product is a signed
 // 32 x 32 one
@@ -80,23 +82,36 @@ __host__ __device__ __forceinline__ int64_t fx_addhi(int64_t t, int64_t acc) {
 }
 constexpr int64_t kFxHalf = 0x80000000LL;
 
-// a b / 2^64, rounded; the product of the low parts (below 2^-2 of the last
-// bit) left out
-__host__ __device__ __forceinline__ int64_t fx_mul(Fx a, Fx b) {
-  const int64_t t = fx_wide(a.h, b.l, fx_wide(a.l, b.h, kFxHalf));
-  return fx_addhi(t, fx_wide(a.h, b.h, 0));
+// ((h 2^32 + t) / 2^32) 2^s, s < 32: the bits below the high product's last
+// one come from the cross product (a plain shift would fill zeros in: the
+// values would be good to 2^-59 instead of 2^-61)
+__host__ __device__ __forceinline__ int64_t fx_shl(int64_t t, int64_t h, int s) {
+  const int64_t r = fx_addhi(t, h);
+#ifdef __CUDA_ARCH__
+  const uint32_t lo = __funnelshift_l((uint32_t)t, (uint32_t)r, s);
+  const uint32_t hi = __funnelshift_l((uint32_t)r, (uint32_t)((uint64_t)r >> 32), s);
+  return (int64_t)(((uint64_t)hi << 32) | lo);
+#else
+  return (int64_t)(((uint64_t)r << s) | ((uint64_t)(uint32_t)t >> (32 - s)));
+#endif
+}
+// a b / 2^(64 - s), 0 < s < 32; the product of the low parts (below 2^-2 of
+// the last bit before the shift) left out
+__host__ __device__ __forceinline__ int64_t fx_mul(Fx a, Fx b, int s) {
+  const int64_t t = fx_wide(a.h, b.l, fx_wide(a.l, b.h, 0));
+  return fx_shl(t, fx_wide(a.h, b.h, 0), s);
 }
 // a b / 2^32 for a 31-bit a
 __host__ __device__ __forceinline__ int64_t fx_mulint(int32_t a, Fx b) {
   return fx_addhi(fx_wide(a, b.l, kFxHalf), fx_wide(a, b.h, 0));
 }
 // a b / 2^62, and a c - b d, a d + b c over 2^62: one step of the powers of
-// st and of e^{i phi} (rounded at 2^-60)
+// st and of e^{i phi}
 __host__ __device__ __forceinline__ int64_t fx_mul62(Fx a, Fx b) {
-  return (int64_t)((uint64_t)fx_mul(a, b) << 2);
+  return fx_mul(a, b, 2);
 }
 __host__ __device__ __forceinline__ void fx_turn(Fx a, Fx b, Fx c, Fx d, Fx dn, int64_t* re, int64_t* im) {
-  int64_t t = fx_wide(a.l, c.h, kFxHalf), u = fx_wide(a.l, d.h, kFxHalf);
+  int64_t t = fx_wide(a.l, c.h, 0), u = fx_wide(a.l, d.h, 0);
   t = fx_wide(a.h, c.l, t);
   u = fx_wide(a.h, d.l, u);
   t = fx_wide(b.l, dn.h, t);
@@ -104,8 +119,8 @@ __host__ __device__ __forceinline__ void fx_turn(Fx a, Fx b, Fx c, Fx d, Fx dn, 
   t = fx_wide(b.h, dn.l, t);
   u = fx_wide(b.h, c.l, u);
   const int64_t r = fx_wide(b.h, dn.h, fx_wide(a.h, c.h, 0)), i = fx_wide(b.h, c.h, fx_wide(a.h, d.h, 0));
-  *re = (int64_t)((uint64_t)fx_addhi(t, r) << 2);
-  *im = (int64_t)((uint64_t)fx_addhi(u, i) << 2);
+  *re = fx_shl(t, r, 2);
+  *im = fx_shl(u, i, 2);
 }
 
 // x / a in units of 2^-62 for 0 <= x <= a: rcp = 2^115 / (mantissa of a),
@@ -231,18 +246,16 @@ __host__ __device__ __forceinline__ FixCharge fix_irregular(int64_t dx, int64_t 
   const uint64_t phi = (uint64_t)(((unsigned __int128)y2 * (uint64_t)r2) >> 64);
 #endif
   const int64_t d = (int64_t)(kFixC80 - ((phi << 24) | (plo >> 40)));  // e r0^2 2^80
-  const int64_t e = (int64_t)((uint64_t)fx_mul(fx_split(d), fx_split(kFixCinv)) << 4);  // 2^80, below 2^60
+  const int64_t e = fx_mul(fx_split(d), fx_split(kFixCinv), 4);  // 2^80, below 2^60
   const int32_t eh = (int32_t)(e >> 32);
   const int64_t c = (e >> 1) + ((3 * (((int64_t)eh * eh) >> 16)) >> 3);
   const int64_t rho = ((int64_t)yi << 32) + (fx_mulint(yi, fx_split(c)) >> 16);
   FixCharge f;
   const Fx rs = fx_split(rho);
-  const int64_t k60 = fx_mul(rs, rs);  // kappa (2^60)
-  f.kap = (uint64_t)k60 << 3;
-  const Fx g = fx_split((int64_t)((uint64_t)fx_mul(fx_split((int64_t)((uint64_t)k60 << 2)), fx_split(kFixR0inv)) << 2));
-  // g: kappa / r0 (2^61)
-  f.zeta = (int64_t)((uint64_t)fx_mul(fx_split(dz), g) << 3);
-  f.st = (int64_t)((uint64_t)fx_mul(fx_split(fix_polar(dx, dy, &f)), g) << 3);
+  f.kap = (uint64_t)fx_mul(rs, rs, 3);
+  const Fx g = fx_split(fx_mul(fx_split((int64_t)(f.kap >> 1)), fx_split(kFixR0inv), 2));  // kappa / r0 (2^61)
+  f.zeta = fx_mul(fx_split(dz), g, 3);
+  f.st = fx_mul(fx_split(fix_polar(dx, dy, &f)), g, 3);
   f.x0 = fx_mul62(fx_split(q), rs);
   return f;
 }
@@ -270,16 +283,15 @@ __host__ __device__ __forceinline__ Fx fix_next(Fx zs, uint32_t kh, uint32_t kl,
   const uint64_t kw = fx_wideu(kh, wh, s >> 32);
 #endif
   const Fx k = fx_split((int64_t)kw);
-  int64_t t = fx_wide(zs.l, q1.h, kFxHalf);
+  int64_t t = fx_wide(zs.l, q1.h, 0);
   t = fx_wide(zs.h, q1.l, t);
   t = fx_wide(k.l, q2.h, t);
   t = fx_wide(k.h, q2.l, t);
   int64_t r = fx_wide(zs.h, q1.h, 0);
   r = fx_wide(k.h, q2.h, r);
-  r = fx_addhi(t, r);
-  return fx_split((int64_t)((uint64_t)r << sh));
+  return fx_split(fx_shl(t, r, sh));
 }
-// acc + x y (phase x 2^59, y 2^62: terms of 2^57)
+// acc + x y (phase x 2^60, y 2^62: terms of 2^58)
 __host__ __device__ __forceinline__ int64_t fix_mac(Fx x, Fx q, int64_t acc) {
   int64_t t = fx_wide(x.l, q.h, kFxHalf);
   t = fx_wide(x.h, q.l, t);
@@ -319,7 +331,7 @@ constexpr FixShares fix_shares(int p) {
 }
 
 // Tables of one launch: per warp and step the recurrence constants and the
-// value of the step's sum in the scaled layout (times 2^-52); unused steps
+// value of the step's sum in the scaled layout (times 2^-53); unused steps
 // have scale 0 and index -1.
 struct FixStep {
   uint32_t wh, wl;
@@ -385,7 +397,7 @@ inline void fix_tab_build(FixTab* T, int p, bool irregular, double R) {
         }
       }
       const long double sign = (i & 2) ? -1.0L : 1.0L;
-      T->scale[k][t] = (double)(head * rad * sign * prod / (long double)(1ull << sigma) / 4503599627370496.0L);
+      T->scale[k][t] = (double)(head * rad * sign * prod / (long double)(1ull << sigma) / 9007199254740992.0L);
       T->index[k][t] = (short)(n * n + (m ? 2 * m - 1 : 0));
     }
   }

@@ -17,6 +17,7 @@ struct FixArgs {
   uint64_t rcp;  // fx_coord's reciprocal of the box side
   int ea;        // biased exponent of the box side
   int qexp;
+  const double* dot;
 };
 
 // entry k (0..188) of the interaction list of a cell with parities b, in the
@@ -257,8 +258,8 @@ __global__ void __launch_bounds__(kThreads, fix_ctas(fix_shares(P).steps))
         int64_t* o = s_Y + tid;
         for (int m = 0; m <= p; m++) {
           o[0] = y;
-          o[nthr] = xr >> 3;
-          o[2 * nthr] = xi >> 3;
+          o[nthr] = xr >> MC_FIX_PHASE;
+          o[2 * nthr] = xi >> MC_FIX_PHASE;
           o += 3 * nthr;
           const Fx a = fx_split(xr), b = fx_split(xi);
           y = fx_mul62(fx_split(y), st);
@@ -304,13 +305,26 @@ __global__ void __launch_bounds__(kThreads, fix_ctas(fix_shares(P).steps))
   constexpr int C = (P + 1) * (P + 1);
   const double sc = ldexp(1.0, qexp);
   double* o = out + ((size_t)t * A.nchunk + ch) * C;
+  double contracted = 0.0;
 #pragma unroll
   for (int b = 0; 16 * b < ST; b++) {
     const int i = 16 * b + (lane & 15), im = lane >> 4;
     const int k = i < ST ? A.tab.index[warp][i] : -1;
     if (k < 0 || (im && is_square_index(k))) continue;
-    const double r = sum[b] * A.tab.scale[warp][i] * sc;
-    o[k + im] = im ? -r : r;
+    double r = sum[b] * A.tab.scale[warp][i] * sc;
+    if (im) r = -r;
+    if (A.dot) {
+      contracted += (is_square_index(k) ? 1.0 : 2.0) * r * A.dot[(size_t)t * C + k + im];
+    } else {
+      o[k + im] = r;
+    }
+  }
+  if (A.dot) {
+    __shared__ double part[MC_FIX_WARPS];
+    contracted = warp_sum(contracted);
+    if (lane == 0) part[warp] = contracted;
+    __syncthreads();
+    if (tid == 0) out[blockIdx.x] = (part[0] + part[1]) + (part[2] + part[3]);
   }
 }
 
@@ -330,6 +344,138 @@ __global__ void __launch_bounds__(256)
     for (int w = 1; w < 8; w++) v += s[w][lane];
     out[(size_t)t * C + k] = v;
   }
+}
+
+// ------------------------------------------------------ near pairs (energy)
+// q_i q_j / r_ij over the pairs of a cell with itself and with 13 of its 26
+// neighbours (the other 13 see the pair from their side).  One warp per
+// (cell, neighbour): a lane per charge of the cell, the neighbour's charges
+// staged in shared memory and read by all lanes.  Differences are exact
+// 64-bit integers; 1/r comes from a single-precision estimate and one
+// third-order step in integers on the difference shifted up to full length,
+// good to 2^-60, so only the last multiply-add is an FP64 instruction (one
+// against 15 of a pair in FP64 at 64 cycles each).
+struct NearArgs {
+  FixSource src;
+  int L, pbc;
+  uint64_t rcp;
+  int ea;
+  double unit;  // 1 / (four finest cells)
+};
+
+// 1/|(x, y, z)| for a difference in units of 2^-62 (times the caller's unit)
+__device__ __forceinline__ double near_rinv(int64_t dx, int64_t dy, int64_t dz) {
+  const uint64_t m = (uint64_t)(dx < 0 ? -dx : dx) | (uint64_t)(dy < 0 ? -dy : dy) | (uint64_t)(dz < 0 ? -dz : dz);
+  if (m == 0) return __builtin_huge_val();
+  const int k = __clzll((long long)m) - 2;
+  const Fx x = fx_split((int64_t)((uint64_t)dx << k)), y = fx_split((int64_t)((uint64_t)dy << k)),
+           z = fx_split((int64_t)((uint64_t)dz << k));
+  const int64_t n2 = fx_norm(x, y, z);  // 2^60, in [1/4, 3)
+  const float yf = rsqrtf((float)(int32_t)(n2 >> 32) * 3.7252902984619140625e-9f);
+  const int32_t yi = (int32_t)(yf * 536870912.0f);  // 2^29
+  const uint64_t y2 = (uint64_t)((int64_t)yi * yi);
+  const uint64_t plo = y2 * (uint64_t)n2, phi = __umul64hi(y2, (uint64_t)n2);
+  const int64_t e = -(int64_t)((phi << 26) | (plo >> 38));  // 1 - y^2 n2 (2^80)
+  const int32_t eh = (int32_t)(e >> 32);
+  const int64_t c = (e >> 1) + ((3 * (((int64_t)eh * eh) >> 16)) >> 3);
+  const uint64_t r = (uint64_t)(((int64_t)yi << 32) + (fx_mulint(yi, fx_split(c)) >> 16));  // 2^61, in (0.57, 2]
+  // to a double: 53 leading bits, rounded; value r 2^(k - 61)
+  const int s = __clzll((long long)r);  // 1, 2 or 3
+  const uint64_t f = (r << s) + (1ull << 10);  // below 2^10: rounded up to the next power of two
+  const uint64_t top = f < (1ull << 10) ? (1ull << 63) : f;
+  const int ex = 1023 + 63 - s - 61 + k + (f < (1ull << 10) ? 1 : 0);
+  return __longlong_as_double((long long)(((uint64_t)ex << 52) | ((top >> 11) & 0xFFFFFFFFFFFFFull)));
+}
+
+__global__ void __launch_bounds__(256)
+    k_fix_near(const __grid_constant__ NearArgs A, double* __restrict__ out) {
+  __shared__ int64_t s_x[8][32][4];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nL = 1 << (A.L - 1), cap = A.src.cap;
+  const long long tasks = 14LL * nL * nL * nL;
+  const double4* rows = reinterpret_cast<const double4*>(A.src.rows);
+  double total = 0.0;
+  for (long long task = (long long)blockIdx.x * 8 + warp; task < tasks; task += (long long)gridDim.x * 8) {
+    const int cell = (int)(task / 14), o = (int)(task % 14);  // o = 0: the cell itself
+    const int c[3] = {cell / (nL * nL), (cell / nL) % nL, cell % nL};
+    const int k = 13 + o;
+    int e[3] = {c[0] + k / 9 - 1, c[1] + (k / 3) % 3 - 1, c[2] + k % 3 - 1};
+    int src[3], im[3];
+    bool ok = true;
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+      src[d] = mc_wrap_coord(e[d], nL);
+      im[d] = (e[d] - src[d]) / nL;
+      if (!A.pbc && im[d]) ok = false;
+    }
+    if (!ok) continue;
+    const int other = (src[0] * nL + src[1]) * nL + src[2];
+    const int ni = A.src.count[cell], nj = A.src.count[other];
+    for (int i0 = 0; i0 < ni; i0 += 32) {
+      const int i = i0 + lane;
+      int64_t xi[3] = {0, 0, 0};
+      double qi = 0.0, acc = 0.0;
+      if (i < ni) {
+        const double4 r = ldcg4(&rows[(size_t)cell * cap + i]);
+        xi[0] = fx_coord(r.x, A.rcp, A.ea);
+        xi[1] = fx_coord(r.y, A.rcp, A.ea);
+        xi[2] = fx_coord(r.z, A.rcp, A.ea);
+        qi = r.w;
+      }
+      for (int j0 = 0; j0 < nj; j0 += 32) {
+        if (o == 0 && j0 > i0) break;  // pairs i > j
+        __syncwarp();
+        if (j0 + lane < nj) {
+          const double4 r = ldcg4(&rows[(size_t)other * cap + j0 + lane]);
+          int64_t* x = s_x[warp][lane];
+          x[0] = fx_coord(r.x, A.rcp, A.ea) + (int64_t)((uint64_t)(int64_t)im[0] << 62);
+          x[1] = fx_coord(r.y, A.rcp, A.ea) + (int64_t)((uint64_t)(int64_t)im[1] << 62);
+          x[2] = fx_coord(r.z, A.rcp, A.ea) + (int64_t)((uint64_t)(int64_t)im[2] << 62);
+          x[3] = __double_as_longlong(r.w);
+        }
+        __syncwarp();
+        const int jn = min(32, nj - j0);
+        for (int j = 0; j < jn; j++) {
+          const int64_t* x = s_x[warp][j];
+          if (i >= ni || (o == 0 && j0 + j >= i)) continue;
+          int64_t d[3];
+#pragma unroll
+          for (int a = 0; a < 3; a++) {
+            const int64_t v = (int64_t)((uint64_t)xi[a] - (uint64_t)x[a]);
+            d[a] = A.L >= 3 ? (int64_t)((uint64_t)v << (A.L - 3)) : v >> 1;
+          }
+          acc += __longlong_as_double(x[3]) * near_rinv(d[0], d[1], d[2]);
+        }
+      }
+      total += qi * acc;
+    }
+  }
+  total = warp_sum(total);
+  if (lane == 0) out[(size_t)blockIdx.x * 8 + warp] = total * A.unit;
+}
+
+int fix_near_blocks(int L, int sms) {
+  const long long b = (14LL << (3 * (L - 1))) / 8 + 1;
+  return (int)std::min<long long>(b, 8LL * sms);
+}
+
+static void box_scale(double a, uint64_t* rcp, int* ea) {
+  uint64_t u;
+  __builtin_memcpy(&u, &a, 8);
+  *ea = (int)((u >> 52) & 0x7ff);
+  const uint64_t m = (u & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
+  *rcp = (uint64_t)((((unsigned __int128)1 << 115) + m / 2) / m);
+}
+
+cudaError_t fix_near(int L, bool pbc, double a, const FixSource& src, int blocks, double* out, cudaStream_t st) {
+  NearArgs A;
+  A.src = src;
+  A.L = L;
+  A.pbc = pbc;
+  box_scale(a, &A.rcp, &A.ea);
+  A.unit = (double)(1 << (L - 1)) / (4.0 * a);
+  k_fix_near<<<blocks, 256, 0, st>>>(A, out);
+  return cudaGetLastError();
 }
 
 __global__ void k_reduce_chunks(int, int, int, const double*, double*);
@@ -369,11 +515,8 @@ cudaError_t fix_launch(const FixPass& ps, const FixSource& src, double* out, cud
   A.irregular = ps.irregular;
   A.pbc = ps.pbc;
   A.qexp = ps.qexp;
-  uint64_t u;
-  __builtin_memcpy(&u, &ps.a, 8);
-  A.ea = (int)((u >> 52) & 0x7ff);
-  const uint64_t m = (u & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
-  A.rcp = (uint64_t)((((unsigned __int128)1 << 115) + m / 2) / m);
+  A.dot = ps.dot;
+  box_scale(ps.a, &A.rcp, &A.ea);
   const size_t smem = sizeof(int64_t) * (size_t)kThreads * (2 + 3 * (ps.p + 1));
   const long long ncl = 1LL << (3 * (ps.l - 1));
   const long long grid = ncl * ps.nchunk;

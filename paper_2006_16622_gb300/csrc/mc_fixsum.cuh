@@ -19,18 +19,26 @@ struct FixSource {
 
 // One pass over level l (1 = the box): irregular sums over the interaction
 // list of every cell, or regular sums over the cell's own charges.  Chunk ch
-// of cell t goes to out[(t * nchunk + ch) * C] in the scaled layout.
+// of cell t goes to out[(t * nchunk + ch) * C] in the scaled layout; with
+// `dot` (the level's other expansions, C per cell) only its contraction
+// sum_k W_k S_k dot_k (W = 1 for m = 0, else 2) goes to out[t * nchunk + ch].
 struct FixPass {
   int L, l, p;
   bool irregular, pbc;
   double a;     // box side
   int qexp;     // charges are at most 2^qexp in size
   int nchunk;   // chunks of the source units (finest cells) per target
+  const double* dot;
 };
 // chunks per target that keep every SM busy without tasks too short to pay
 // for themselves (occupancy: mean charges of a finest cell)
 int fix_chunks(int L, int l, bool irregular, int sms, double occupancy, int p);
 cudaError_t fix_launch(const FixPass& ps, const FixSource& src, double* out, cudaStream_t st);
+// Direct part of the energy: 1/r over the pairs of charges within near cells
+// (every pair and image once), one partial per warp of the returned number
+// of blocks of 256 threads
+int fix_near_blocks(int L, int sms);
+cudaError_t fix_near(int L, bool pbc, double a, const FixSource& src, int blocks, double* out, cudaStream_t st);
 // charges of this span of exponents (largest minus smallest) keep the
 // fixed-point sums at least as accurate as FP64 ones
 #define MC_FIX_QSPAN 6

@@ -262,29 +262,206 @@ __global__ void __launch_bounds__(MC_THREADS)
   }
 }
 
-// Khat, dipole from the chunk partials (fixed order), then Hhat = G Khat
-__global__ void k_far_finish(const McSys* __restrict__ sysp, int nchunk,
-                             const double* __restrict__ in) {
+__device__ __forceinline__ void rt_single(int l, int mu, double x, double y, double z, double* re, double* im);
+__device__ __forceinline__ void rl_decode(int k, int* n, int* m, int* im);
+
+// Khat and the dipole from kh (C + 3 values; kh null: Khat is in place and its
+// n = 1 terms are the dipole about the box centre), then Hhat = G Khat: 32
+// rows per block, every warp an eighth of the columns
+__global__ void __launch_bounds__(256) k_far_apply(const McSys* __restrict__ sysp, const double* __restrict__ kh) {
   const McSys& S = *sysp;
-  const int C = S.C;
-  __shared__ double kh[256 + 3];
-  for (int k = threadIdx.x; k < C + 3; k += blockDim.x) {
-    double s = 0.0;
-    for (int ch = 0; ch < nchunk; ch++) s += in[(size_t)ch * (C + 3) + k];
-    kh[k] = s;
+  __shared__ double part[8][32];
+  const int C = S.C, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, k = blockIdx.x * 32 + lane;
+  const double* K = kh ? kh : S.Khat;
+  double h = 0.0;
+  if (S.bc == 0 && k < C)
+    for (int c = warp; c < C; c += 8) h += S.G[(size_t)c * C + k] * K[c];
+  part[warp][lane] = h;
+  __syncthreads();
+  if (warp == 0 && k < C) {
+    for (int w = 1; w < 8; w++) h += part[w][lane];
+    S.Hhat[k] = h;
+    if (kh) S.Khat[k] = kh[k];
+  }
+  if (blockIdx.x == 0 && threadIdx.x < 3) {
+    const int d = threadIdx.x;
+    S.dipv[d] = kh ? kh[C + d] : (d == 0 ? 2.0 * K[2] : d == 1 ? -2.0 * K[3] : K[1]) + 0.5 * S.a * K[0];
+  }
+}
+
+// ------------------------------------------------- multipoles of upper levels
+// A cell's multipole from its eight children's (the addition theorem of the
+// scaled regular harmonics, the same truncated set exactly):
+//   K_j^k = sum_{n <= j} sum_m conj Rt_{j-n}^{k-m}(child centre - centre) K_n^m.
+// In the real layout the matrices of the eight offsets (+-1/2 of a child)
+// differ in signs only, so the children go through one product after a
+// Walsh-Hadamard transform (class: parities of a coefficient under the three
+// reflections).  FP64: one product per eight children is little work.
+__device__ __forceinline__ int rl_class(int k) {
+  int r = (int)sqrtf((float)k + 0.5f);
+  while (r * r > k) r--;
+  while ((r + 1) * (r + 1) <= k) r++;
+  const int rem = k - r * r, m = (rem + 1) / 2, im = (rem > 0 && (rem & 1) == 0) ? 1 : 0;
+  return (((m + im) & 1) << 2) | (im << 1) | ((r + m) & 1);
+}
+
+// matrix of the offset (1/2, 1/2, 1/2) at unit child width, T[col * C + row]
+__global__ void k_m2m_table(int p, double* __restrict__ T) {
+  const int C = (p + 1) * (p + 1);
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < C * C; i += gridDim.x * blockDim.x) {
+    const int row = i % C, col = i / C;
+    int j, k, rim, n, m, cim;
+    rl_decode(row, &j, &k, &rim);
+    rl_decode(col, &n, &m, &cim);
+    double v = 0.0;
+    if (n <= j) {
+      // the order -m of a set Z with Z^-m = (-1)^m conj Z^m joins that of m
+      auto a = [&](int mu, double* re, double* im) {
+        const int ab = abs(mu), l = j - n;
+        *re = *im = 0.0;
+        if (ab > l) return;
+        rt_single(l, ab, 0.5, 0.5, 0.5, re, im);
+        *im = -*im;  // conj
+        if (mu < 0) {
+          const double sg = (ab & 1) ? -1.0 : 1.0;
+          *re *= sg;
+          *im *= -sg;
+        }
+      };
+      double pr, pi, qr = 0.0, qi = 0.0;
+      a(k - m, &pr, &pi);
+      if (m > 0) {
+        a(k + m, &qr, &qi);
+        if (m & 1) {
+          qr = -qr;
+          qi = -qi;
+        }
+      }
+      // (p + i pi)(x + i y) + (q + i qi)(x - i y)
+      v = !rim ? (!cim ? pr + qr : -pi + qi) : (!cim ? pi + qi : pr - qr);
+    }
+    T[(size_t)col * C + row] = v;
+  }
+}
+
+#define MC_M2M_CELLS 4
+__global__ void __launch_bounds__(256)
+    k_m2m_level(int p, int nl, double wc, const double* __restrict__ T, const double* __restrict__ child,
+                double* __restrict__ out) {
+  extern __shared__ double mt[];  // [MC_M2M_CELLS][8][C]
+  __shared__ unsigned char cls[(MC_PMAX + 1) * (MC_PMAX + 1)];
+  const int C = (p + 1) * (p + 1), ncl = nl * nl * nl, nc = 2 * nl;
+  for (int k = threadIdx.x; k < C; k += blockDim.x) cls[k] = (unsigned char)rl_class(k);
+  for (int i = threadIdx.x; i < MC_M2M_CELLS * C; i += blockDim.x) {
+    const int t = blockIdx.x * MC_M2M_CELLS + i / C, col = i % C;
+    double v[8];
+    int n = (int)sqrtf((float)col + 0.5f);
+    double sc = 1.0;
+    for (int q = 0; q < n; q++) sc /= wc;
+#pragma unroll
+    for (int g = 0; g < 8; g++) {  // signs of the child's offset: bits x 4, y 2, z 1
+      const int cx = 2 * (t / (nl * nl)) + !(g & 4), cy = 2 * ((t / nl) % nl) + !(g & 2), cz = 2 * (t % nl) + !(g & 1);
+      v[g] = t < ncl ? child[(size_t)((cx * nc + cy) * nc + cz) * C + col] * sc : 0.0;
+    }
+#pragma unroll
+    for (int b = 1; b < 8; b <<= 1)
+#pragma unroll
+      for (int g = 0; g < 8; g++)
+        if (!(g & b)) {
+          const double x = v[g], y = v[g | b];
+          v[g] = x + y;
+          v[g | b] = x - y;
+        }
+#pragma unroll
+    for (int d = 0; d < 8; d++) mt[((i / C) * 8 + d) * C + col] = v[d];
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < C; k += blockDim.x) {
-    S.Khat[k] = kh[k];
-    double h = 0.0;
-    if (S.bc == 0)
-      for (int c = 0; c < C; c++) h += S.G[(size_t)c * C + k] * kh[c];
-    S.Hhat[k] = h;
+  const int r = threadIdx.x;
+  if (r >= C) return;
+  const int j = (int)sqrtf((float)r + 0.5f), cr = cls[r];
+  double acc[MC_M2M_CELLS] = {};
+  for (int c = 0; c < (j + 1) * (j + 1); c++) {
+    const double t = T[(size_t)c * C + r];
+    const int d = cr ^ cls[c];
+#pragma unroll
+    for (int q = 0; q < MC_M2M_CELLS; q++) acc[q] = fma(t, mt[(q * 8 + d) * C + c], acc[q]);
   }
-  if (threadIdx.x < 3) S.dipv[threadIdx.x] = kh[C + threadIdx.x];
+  double sc = 1.0;
+  for (int q = 0; q < j; q++) sc *= wc;
+#pragma unroll
+  for (int q = 0; q < MC_M2M_CELLS; q++) {
+    const int t = blockIdx.x * MC_M2M_CELLS + q;
+    if (t < ncl) out[(size_t)t * C + r] = acc[q] * sc;
+  }
+}
+
+cudaError_t m2m_table(int p, double* T, cudaStream_t st) {
+  const int C = (p + 1) * (p + 1);
+  k_m2m_table<<<(C * C + 255) / 256, 256, 0, st>>>(p, T);
+  return cudaGetLastError();
+}
+// the multipoles of the level with nl cells per axis from those of its
+// children (child cell width wc)
+cudaError_t m2m_level(int p, int nl, double wc, const double* T, const double* child, double* out, cudaStream_t st) {
+  const int C = (p + 1) * (p + 1), ncl = nl * nl * nl;
+  const int smem = (int)sizeof(double) * MC_M2M_CELLS * 8 * C;
+  cudaError_t e = cudaFuncSetAttribute(k_m2m_level, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  k_m2m_level<<<(ncl + MC_M2M_CELLS - 1) / MC_M2M_CELLS, 256, smem, st>>>(p, nl, wc, T, child, out);
+  return cudaGetLastError();
 }
 
 // ------------------------------------------------------------ total energy
+// The level expansions' part, sum_i q_i Psi(r_i) = sum over cells of
+// sum_k W_k Mhat_k Lhat_k, where the multipoles of every level are at hand;
+// one partial per block
+__global__ void __launch_bounds__(256)
+    k_energy_dot(size_t total, int C, const double* __restrict__ M, const double* __restrict__ L,
+                 double* __restrict__ out) {
+  __shared__ double red[8];
+  double s = 0.0;
+  for (size_t i = blockIdx.x * (size_t)256 + threadIdx.x; i < total; i += (size_t)gridDim.x * 256) {
+    const int k = (int)(i % C), r = (int)sqrtf((float)k + 0.5f);
+    s += (r * r == k ? 1.0 : 2.0) * (M[i] * L[i]);
+  }
+  s = warp_sum(s);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; w++) s += red[w];
+    out[blockIdx.x] = s;
+  }
+}
+
+// U from the partials of the near pairs and (twice) of the expansions, and the
+// periodic terms
+__global__ void __launch_bounds__(1024)
+    k_energy_sum(const McSys* __restrict__ sysp, int nnear, int nexp, const double* __restrict__ in,
+                 double* __restrict__ dst) {
+  const McSys& S = *sysp;
+  __shared__ double red[32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double s = 0.0;
+  for (int i = threadIdx.x; i < nnear; i += 1024) s += in[i];
+  for (int i = threadIdx.x; i < nexp; i += 1024) s += 0.5 * in[nnear + i];
+  if (S.bc == 0)
+    for (int k = threadIdx.x; k < S.C; k += 1024) {
+      const int r = (int)sqrtf((float)k + 0.5f);
+      s += (r * r == k ? 0.5 : 1.0) * (S.Khat[k] * S.Hhat[k]);
+    }
+  s = warp_sum(s);
+  if (lane == 0) red[warp] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 32; w++) s += red[w];
+    if (S.bc == 0 && S.dip == 0) {
+      const double D2 = S.dipv[0] * S.dipv[0] + S.dipv[1] * S.dipv[1] + S.dipv[2] * S.dipv[2];
+      s += -2.0 * 3.141592653589793 / (3.0 * S.V) * D2;
+    }
+    dst[0] = s;
+  }
+}
+
 // U = 1/2 sum_i q_i phi_i + 1/2 sum_k W_k Khat_k Hhat_k + dipole term, where
 // phi_i sums the level expansions at r_i and the direct near-cell charges
 // other than i itself.  One warp per particle; per-warp running sums in

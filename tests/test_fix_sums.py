@@ -9,7 +9,7 @@ faces and corners of the nearest listed cells, at the furthest corner.
 
 Bound: a term's error in units of the largest value its coefficient can have
 (R0^-(n+1) or R0^n in the paper's normalisation).  Products are rounded at
-2^-57; the scale factors are doubles (2^-53 of the value); the recurrence
+2^-58; the scale factors are doubles (2^-53 of the value); the recurrence
 loses at most the ratio of a harmonic's largest value to its size at the
 start of its column (below 2^8 for p <= 15) times 2^-59.  So rms < 2^-54 and
 every term < 2^-49.
@@ -109,7 +109,7 @@ int main(int argc, char** argv) {
     const Fx ex = fx_split(c.ex), ey = fx_split(c.ey), en = fx_split(-c.ey), st = fx_split(c.st);
     int64_t y = c.x0, xr = (int64_t)1 << 62, xi = 0;
     for (int m = 0; m <= p; m++) {
-      const Fx pr = fx_split(xr >> 3), pi = fx_split(xi >> 3), zp = fx_split(c.zeta), zn = fx_split(-c.zeta);
+      const Fx pr = fx_split(xr >> MC_FIX_PHASE), pi = fx_split(xi >> MC_FIX_PHASE), zp = fx_split(c.zeta), zn = fx_split(-c.zeta);
       Fx q1 = fx_split(y), q2 = {0, 0};
       for (int n = m; n <= p; n++) {
         const int i = n - m, t = sh.first[m] + i, wi = sh.warp[m];
