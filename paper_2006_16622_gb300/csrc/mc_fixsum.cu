@@ -20,47 +20,6 @@ struct FixArgs {
   const double* dot;
 };
 
-// entry k (0..188) of the interaction list of a cell with parities b, in the
-// order of il_table_init: the 6^3 children of the parent's neighbours without
-// the 27 near cells
-__device__ __forceinline__ void list_entry(int k, const int* b, int* o) {
-  int i, j, q, rem;
-  const int head = 36 * (1 + b[0]);
-  if (k < head) {
-    i = k / 36;
-    rem = k % 36;
-    j = rem / 6;
-    q = rem % 6;
-  } else if (k < head + 81) {
-    const int k1 = k - head;
-    i = 1 + b[0] + k1 / 27;
-    rem = k1 % 27;
-    const int r0 = 6 * (1 + b[1]);
-    if (rem < r0) {
-      j = rem / 6;
-      q = rem % 6;
-    } else if (rem < r0 + 9) {
-      const int r1 = rem - r0;
-      j = 1 + b[1] + r1 / 3;
-      q = r1 % 3;
-      if (q >= 1 + b[2]) q += 3;
-    } else {
-      const int r2 = rem - r0 - 9;
-      j = 4 + b[1] + r2 / 6;
-      q = r2 % 6;
-    }
-  } else {
-    const int k2 = k - head - 81;
-    i = 4 + b[0] + k2 / 36;
-    rem = k2 % 36;
-    j = rem / 6;
-    q = rem % 6;
-  }
-  o[0] = i - 2 - b[0];
-  o[1] = j - 2 - b[1];
-  o[2] = q - 2 - b[2];
-}
-
 // index of a coefficient with m = 0 (no imaginary part)
 __device__ __forceinline__ bool is_square_index(int k) {
   const int r = (int)sqrtf((float)k + 0.5f);
@@ -171,7 +130,7 @@ __global__ void __launch_bounds__(kThreads, fix_ctas(fix_shares(P).steps))
       const long long u = u0 + i;
       if (u < ue) {
         int o[3] = {0, 0, 0};
-        if (irr) list_entry((int)(u >> (3 * fb)), par, o);
+        if (irr) il_entry((int)(u >> (3 * fb)), par, o);
         const int fc = (int)(u & (((long long)1 << (3 * fb)) - 1));
         const int fd[3] = {fc >> (2 * fb), (fc >> fb) & (f - 1), fc & (f - 1)};
         int g[3];

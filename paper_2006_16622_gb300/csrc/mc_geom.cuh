@@ -6,26 +6,58 @@
 // host tests.
 #pragma once
 
-// Interaction-list offsets (Sec. 3.1) for the 8 parity classes of a cell:
-// children of the parent's 27 neighbours span [-2-b, 3-b] per axis (b the
-// cell's parity on that axis); the 27 near offsets are removed.  Built per
-// CTA in shared memory: il[parity][k] = packed (ox+4) | (oy+4)<<4 | (oz+4)<<8.
-__device__ __forceinline__ void il_table_init(unsigned short (*il)[189]) {
-  for (int t = threadIdx.x; t < 8 * 216; t += blockDim.x) {
-    const int par = t / 216, b = t % 216;
-    const int bx = (par >> 2) & 1, by = (par >> 1) & 1, bz = par & 1;
-    const int i = b / 36, jj = (b / 6) % 6, l = b % 6;
-    const int ox = i - 2 - bx, oy = jj - 2 - by, oz = l - 2 - bz;
-    const bool inner = (ox >= -1 && ox <= 1 && oy >= -1 && oy <= 1 && oz >= -1 && oz <= 1);
-    if (inner) continue;
-    // rank of b among the non-inner entries of this parity class
-    int k = 0;
-    for (int bb = 0; bb < b; bb++) {
-      const int ii = bb / 36, j2 = (bb / 6) % 6, l2 = bb % 6;
-      const int px = ii - 2 - bx, py = j2 - 2 - by, pz = l2 - 2 - bz;
-      if (!(px >= -1 && px <= 1 && py >= -1 && py <= 1 && pz >= -1 && pz <= 1)) k++;
+// Entry k (0..188) of the interaction list (Sec. 3.1) of a cell with parities
+// b: children of the parent's 27 neighbours span [-2-b, 3-b] per axis, the 27
+// near offsets are left out.  Planes, rows and places of the 6^3 box are
+// counted without the 3^3 block that starts at 1 + b on every axis.
+__device__ __forceinline__ void il_entry(int k, const int* b, int* o) {
+  int i, j, q, rem;
+  const int head = 36 * (1 + b[0]);
+  if (k < head) {
+    i = k / 36;
+    rem = k % 36;
+    j = rem / 6;
+    q = rem % 6;
+  } else if (k < head + 81) {
+    const int k1 = k - head;
+    i = 1 + b[0] + k1 / 27;
+    rem = k1 % 27;
+    const int r0 = 6 * (1 + b[1]);
+    if (rem < r0) {
+      j = rem / 6;
+      q = rem % 6;
+    } else if (rem < r0 + 9) {
+      const int r1 = rem - r0;
+      j = 1 + b[1] + r1 / 3;
+      q = r1 % 3;
+      if (q >= 1 + b[2]) q += 3;
+    } else {
+      const int r2 = rem - r0 - 9;
+      j = 4 + b[1] + r2 / 6;
+      q = r2 % 6;
     }
-    il[par][k] = (unsigned short)((ox + 4) | ((oy + 4) << 4) | ((oz + 4) << 8));
+  } else {
+    const int k2 = k - head - 81;
+    i = 4 + b[0] + k2 / 36;
+    rem = k2 % 36;
+    j = rem / 6;
+    q = rem % 6;
+  }
+  o[0] = i - 2 - b[0];
+  o[1] = j - 2 - b[1];
+  o[2] = q - 2 - b[2];
+}
+
+// The lists of the 8 parity classes, built per CTA in shared memory:
+// il[parity][k] = packed (ox+4) | (oy+4)<<4 | (oz+4)<<8.  (Counting the entries
+// before each one instead took ~25 us at the start of every kernel.)
+__device__ __forceinline__ void il_table_init(unsigned short (*il)[189]) {
+  for (int t = threadIdx.x; t < 8 * 189; t += blockDim.x) {
+    const int par = t / 189, k = t % 189;
+    const int b[3] = {(par >> 2) & 1, (par >> 1) & 1, par & 1};
+    int o[3];
+    il_entry(k, b, o);
+    il[par][k] = (unsigned short)((o[0] + 4) | ((o[1] + 4) << 4) | ((o[2] + 4) << 8));
   }
 }
 __device__ __forceinline__ void il_unpack(unsigned short v, int* ox, int* oy, int* oz) {

@@ -19,27 +19,50 @@ struct HarmTabs {
   T iA[MC_PMAX + 1][16], iB[MC_PMAX + 1][16];  // irregular
 };
 
+// The tables' values, formed by the compiler: forming them at the start of
+// every kernel took 3 FP64 divisions a thread, ~10 us of a single proposal's 51.
+struct HarmConst {
+  double rA[MC_PMAX + 1][16], rB[MC_PMAX + 1][16], iA[MC_PMAX + 1][16], iB[MC_PMAX + 1][16];
+  double W[MC_PMAX + 1][16];                       // irregular_w_tabs
+  double P[(MC_PMAX + 1) * (MC_PMAX + 1)];
+};
+constexpr HarmConst harm_const() {
+  HarmConst h{};
+  for (int n = 1; n <= MC_PMAX; n++)
+    for (int m = 0; m < 16; m++) {
+      h.iA[n][m] = 2.0 * n - 1.0;
+      if (n <= m) {
+        h.rA[n][m] = 1.0 / (2.0 * n);
+      } else {
+        const double den = (double)(n + m) * (double)(n - m);
+        h.rA[n][m] = (2.0 * n - 1.0) / den;
+        h.rB[n][m] = 1.0 / den;
+        h.iB[n][m] = (double)(n + m - 1) * (double)(n - m - 1);
+      }
+      if (n >= m + 2)
+        h.W[n][m] = ((double)(n - 1) * (n - 1) - (double)m * m) / ((2.0 * n - 1.0) * (2.0 * n - 3.0));
+    }
+  // P_n^m = prod_{k=m+1..n} (2k - 1) at the real layout index of (n, m) (both parts)
+  for (int n = 0; n <= MC_PMAX; n++)
+    for (int m = 0; m <= n; m++) {
+      double pr = 1.0;
+      for (int j = m + 1; j <= n; j++) pr *= 2.0 * j - 1.0;
+      const int k = n * n + (m ? 2 * m - 1 : 0);
+      h.P[k] = pr;
+      if (m) h.P[k + 1] = pr;
+    }
+  return h;
+}
+static __device__ const HarmConst kHarmConst = harm_const();
+
 template <typename T>
 __device__ void harm_tabs_init(HarmTabs<T>* t) {
   for (int k = threadIdx.x; k < (MC_PMAX + 1) * 16; k += blockDim.x) {
-    int n = k / 16, m = k % 16;
-    double ra = 0, rb = 0, ia = 0, ib = 0;
-    if (n >= 1) {
-      if (n <= m) {
-        ra = 1.0 / (2.0 * n);
-        ia = 2.0 * n - 1.0;
-      } else {
-        double den = (double)(n + m) * (double)(n - m);
-        ra = (2.0 * n - 1.0) / den;
-        rb = 1.0 / den;
-        ia = 2.0 * n - 1.0;
-        ib = (double)(n + m - 1) * (double)(n - m - 1);
-      }
-    }
-    t->rA[n][m] = (T)ra;
-    t->rB[n][m] = (T)rb;
-    t->iA[n][m] = (T)ia;
-    t->iB[n][m] = (T)ib;
+    const int n = k / 16, m = k % 16;
+    t->rA[n][m] = (T)kHarmConst.rA[n][m];
+    t->rB[n][m] = (T)kHarmConst.rB[n][m];
+    t->iA[n][m] = (T)kHarmConst.iA[n][m];
+    t->iB[n][m] = (T)kHarmConst.iB[n][m];
   }
 }
 
@@ -284,21 +307,8 @@ __device__ void pair_w_tabs(const T (*W)[16], const double* P, f2 (*W2)[16], f2*
 
 template <typename T>
 __device__ void irregular_w_tabs(T (*W)[16], double* P) {
-  for (int k = threadIdx.x; k < (MC_PMAX + 1) * 16; k += blockDim.x) {
-    const int n = k / 16, m = k % 16;
-    double w = 0.0;
-    if (n >= m + 2) w = ((double)(n - 1) * (n - 1) - (double)m * m) / ((2.0 * n - 1.0) * (2.0 * n - 3.0));
-    W[n][m] = (T)w;
-  }
-  // P_n^m at the real layout index of (n, m) (both parts)
-  for (int k = threadIdx.x; k < (MC_PMAX + 1) * (MC_PMAX + 1); k += blockDim.x) {
-    int n = 0;
-    while ((n + 1) * (n + 1) <= k) n++;
-    const int m = (k == n * n) ? 0 : (k - n * n + 1) / 2;
-    double pr = 1.0;
-    for (int j = m + 1; j <= n; j++) pr *= 2.0 * j - 1.0;
-    P[k] = pr;
-  }
+  for (int k = threadIdx.x; k < (MC_PMAX + 1) * 16; k += blockDim.x) W[k / 16][k % 16] = (T)kHarmConst.W[k / 16][k % 16];
+  for (int k = threadIdx.x; k < (MC_PMAX + 1) * (MC_PMAX + 1); k += blockDim.x) P[k] = kHarmConst.P[k];
 }
 
 // Column factorisation: every scaled harmonic of column m is the diagonal
