@@ -160,6 +160,19 @@ int sync_status(mc_ctx* c) {
   return st;
 }
 
+constexpr size_t kControlBytes = 8 * 6;  // bar, status (padded), result[4]
+
+// status word and result of a single proposal, after everything on the stream
+int control_read(mc_ctx* c, double* result) {
+  unsigned long long w[6];
+  CK(cudaMemcpyAsync(w, c->h.bar, kControlBytes, cudaMemcpyDeviceToHost, c->stream));
+  CK(cudaStreamSynchronize(c->stream));
+  int st;
+  memcpy(&st, &w[1], sizeof(int));
+  if (st == MC_OK && result) memcpy(result, &w[2], sizeof(double));
+  return st;
+}
+
 int launch_chain(mc_ctx* c, RunParams& rp) {
   rp.wait_ns = c->wait_ns;
   rp.bar_missing = c->bar_missing;
@@ -168,7 +181,8 @@ int launch_chain(mc_ctx* c, RunParams& rp) {
   // single proposals and the multipole method run on the phased kernel
   const bool async = !mm && rp.mode == 0 && c->schedule == MC_SCHEDULE_ASYNC;
   rp.nf_cols = MC_NF_COLS;
-  rp.spec = (!mm && (c->schedule == MC_SCHEDULE_PHASED || c->schedule == MC_SCHEDULE_ASYNC)) ? 1 : 0;
+  // (a proposal alone needs no Alg. L.2 contributions)
+  rp.spec = (!mm && rp.mode != 1 && (c->schedule == MC_SCHEDULE_PHASED || c->schedule == MC_SCHEDULE_ASYNC)) ? 1 : 0;
   rp.chain = 0u;
   // grid: the caller's (mc_set_ctas), else every SM, except for the phased
   // FP32-eval chain of the local method, which is faster on 5/7 of the SMs
@@ -179,8 +193,7 @@ int launch_chain(mc_ctx* c, RunParams& rp) {
   int grid = c->nCTA;
   if (grid == 0)
     grid = (!mm && !async && rp.spec && c->h.prec == MC_FP32_EVAL) ? std::max(1, (5 * c->sms) / 7) : c->sms;
-  CK(cudaMemsetAsync(c->h.bar, 0, sizeof(unsigned long long), c->stream));
-  CK(cudaMemsetAsync(c->h.status, 0, sizeof(int), c->stream));
+  CK(cudaMemsetAsync(c->h.bar, 0, 2 * sizeof(unsigned long long), c->stream));  // and the status word
   if (async) {
     // counters, partial-slot ring at its "not written" pattern (all bits
     // set), the four small-level contribution buffers clear
@@ -482,6 +495,32 @@ int near_parts_auto(const McSys& h) {
   return P;
 }
 
+struct RowScale {
+  double v[(MC_PMAX + 1) * (MC_PMAX + 1)];
+};
+__global__ void k_scale_rows(size_t total, int C, const __grid_constant__ RowScale f, const double* __restrict__ in,
+                             double* __restrict__ out) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x)
+    out[i] = in[i] * f.v[i % C];
+}
+__global__ void k_pack_positions(size_t n, const double4* __restrict__ in, double* __restrict__ out) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < 3 * n; i += (size_t)gridDim.x * blockDim.x)
+    out[i] = reinterpret_cast<const double*>(in)[4 * (i / 3) + i % 3];
+}
+
+// rows of C coefficients times their factors, into a host array
+int copy_scaled(mc_ctx* c, const double* in, size_t cnt, const RowScale& f, double* out) {
+  const size_t most = c->scratch_doubles / c->h.C * c->h.C;
+  for (size_t i = 0; i < cnt; i += most) {
+    const size_t m = std::min(most, cnt - i);
+    k_scale_rows<<<grid_for(c->sms, m, 256), 256, 0, c->stream>>>(m, c->h.C, f, in + i, c->d_scratch);
+    CK(cudaGetLastError());
+    CK(cudaMemcpyAsync(out + i, c->d_scratch, sizeof(double) * m, cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+  }
+  return MC_OK;
+}
+
 int in_box(const double* x, double a) {
   for (int k = 0; k < 3; k++)
     if (!(x[k] >= 0.0 && x[k] < a)) return 0;
@@ -644,10 +683,12 @@ int mc_init(mc_ctx** out, int64_t n, const double* pos, const double* q, double 
   DA(h.partials, sizeof(double) * 4 * MC_MAX_ITEMS);
   DA(h.dK, sizeof(double) * 4 * C);
   DA(h.gK, sizeof(double) * 4 * MC_NF_COLS * C);
-  DA(h.bar, sizeof(unsigned long long));
-  DA(h.status, sizeof(int));
+  // barrier counter, status word and a single proposal's result share a block:
+  // one clear before a launch, one copy after it
+  DA(h.bar, kControlBytes);
+  h.status = reinterpret_cast<int*>(h.bar + 1);
+  h.result = reinterpret_cast<double*>(h.bar + 2);
   DA(h.stats, sizeof(long long) * 4);
-  DA(h.result, sizeof(double) * 4);
   DA(c->d_energy_tmp, sizeof(double));
   h.ls_end = h.L + 1;
   for (int l = h.lmin; l <= h.L; l++)
@@ -667,7 +708,7 @@ int mc_init(mc_ctx** out, int64_t n, const double* pos, const double* q, double 
   DCK(cudaMemsetAsync(h.G, 0, sizeof(double) * (size_t)C * C, c->stream));
   DCK(cudaMemsetAsync(h.dipv, 0, sizeof(double) * 3, c->stream));
   DCK(cudaMemsetAsync(h.energy, 0, sizeof(double), c->stream));
-  DCK(cudaMemsetAsync(h.status, 0, sizeof(int), c->stream));
+  DCK(cudaMemsetAsync(h.bar, 0, kControlBytes, c->stream));
   DCK(cudaMemsetAsync(h.stats, 0, sizeof(long long) * 4, c->stream));
   DCK(cudaMemsetAsync(h.partials, 0, sizeof(double) * 4 * MC_MAX_ITEMS, c->stream));
 
@@ -757,10 +798,7 @@ int mc_propose(mc_ctx* c, int64_t j, const double r_new[3], double* dE_out) {
   rp.rz = r_new[2];
   int rc = launch_chain(c, rp);
   if (rc != MC_OK) return rc;
-  rc = sync_status(c);
-  if (rc != MC_OK) return rc;
-  CK(cudaMemcpy(dE_out, c->h.result, sizeof(double), cudaMemcpyDeviceToHost));
-  return MC_OK;
+  return control_read(c, dE_out);
 }
 
 int mc_accept(mc_ctx* c, int64_t j, const double r_new[3], const double* dE_or_null) {
@@ -780,7 +818,7 @@ int mc_accept(mc_ctx* c, int64_t j, const double r_new[3], const double* dE_or_n
   rp.dEg = dE_or_null ? *dE_or_null : 0.0;
   int rc = launch_chain(c, rp);
   if (rc != MC_OK) return rc;
-  return sync_status(c);
+  return control_read(c, nullptr);
 }
 
 int mc_run(mc_ctx* c, int64_t n_steps, uint64_t seed, double beta, double half_width,
@@ -914,12 +952,15 @@ int mc_get_positions(mc_ctx* c, double* pos_out) {
   if (!c || !pos_out) return MC_ERR_ARG;
   CK(cudaSetDevice(c->dev));
   CK(cudaStreamSynchronize(c->stream));
-  std::vector<double4> hp(c->h.n);
-  CK(cudaMemcpy(hp.data(), c->h.ppos, sizeof(double4) * c->h.n, cudaMemcpyDeviceToHost));
-  for (int i = 0; i < c->h.n; i++) {
-    pos_out[3 * i] = hp[i].x;
-    pos_out[3 * i + 1] = hp[i].y;
-    pos_out[3 * i + 2] = hp[i].z;
+  // packed on the device, in pieces of the setup scratch: the copy goes
+  // straight into the caller's array
+  const size_t most = c->scratch_doubles / 3;
+  for (size_t i = 0; i < (size_t)c->h.n; i += most) {
+    const size_t m = std::min<size_t>(most, (size_t)c->h.n - i);
+    k_pack_positions<<<grid_for(c->sms, m, 256), 256, 0, c->stream>>>(m, c->h.ppos + i, c->d_scratch);
+    CK(cudaGetLastError());
+    CK(cudaMemcpyAsync(pos_out + 3 * i, c->d_scratch, sizeof(double) * 3 * m, cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
   }
   return MC_OK;
 }
@@ -936,12 +977,9 @@ int mc_get_local(mc_ctx* c, int level, double* out) {
   }
   CK(cudaSetDevice(c->dev));
   CK(cudaStreamSynchronize(c->stream));
-  CK(cudaMemcpy(out, c->h.Lhat + (size_t)c->h.lev_off[level] * C, sizeof(double) * cnt,
-                cudaMemcpyDeviceToHost));
-  std::vector<double> inv(C);
-  for (int k = 0; k < C; k++) inv[k] = 1.0 / scale_of(k);
-  for (size_t i = 0; i < cnt; i++) out[i] *= inv[i % C];
-  return MC_OK;
+  RowScale f;
+  for (int k = 0; k < C; k++) f.v[k] = 1.0 / scale_of(k);
+  return copy_scaled(c, c->h.Lhat + (size_t)c->h.lev_off[level] * C, cnt, f, out);
 }
 
 int mc_set_lj(mc_ctx* c, double eps, double sigma, double cutoff) {
@@ -984,12 +1022,9 @@ int mc_get_multipole(mc_ctx* c, int level, double* out) {
   }
   CK(cudaSetDevice(c->dev));
   CK(cudaStreamSynchronize(c->stream));
-  CK(cudaMemcpy(out, c->d_mpole + (size_t)c->h.lev_off[level] * C, sizeof(double) * cnt,
-                cudaMemcpyDeviceToHost));
-  std::vector<double> sc(C);
-  for (int k = 0; k < C; k++) sc[k] = scale_of(k);
-  for (size_t i = 0; i < cnt; i++) out[i] *= sc[i % C];
-  return MC_OK;
+  RowScale f;
+  for (int k = 0; k < C; k++) f.v[k] = scale_of(k);
+  return copy_scaled(c, c->d_mpole + (size_t)c->h.lev_off[level] * C, cnt, f, out);
 }
 
 int mc_get_far(mc_ctx* c, double* K, double* H) {
