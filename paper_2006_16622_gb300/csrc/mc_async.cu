@@ -675,6 +675,57 @@ __device__ __forceinline__ void async_body(const McSys* __restrict__ sysp, RunPa
                                   [&](int t2, int n, int m, bool v, bool c1, TE qv) {
                                     qsv[t2] = v ? qv : TE(0);
                                   });
+              if constexpr (sizeof(TE) == 8) {
+                // FP64: everything but the expansion's values comes before
+                // the wait.  Weights of the values: charge and sign, column
+                // factor, polynomial; the two groups of a side take three and
+                // two of the quarter's steps.  After the wait: six
+                // multiply-adds and the sum over the lanes (11 FP64
+                // instructions of ~64 cycles each on the step's critical
+                // path, 45 with the factors applied to the column sums)
+                const int hf = grp >> 1, m1 = lane & 7, len1 = p - m1 + 1;
+                const double qs = side ? g.q : -g.q, f1 = m1 ? 2.0 * qs : qs, f2 = 2.0 * qs;
+                const double c1r = f1 * D1r, c1i = -f1 * D1i, c2r = f2 * D2r, c2i = -f2 * D2i;
+                double wr[3], wi[3];
+                const double *pr[3], *pi[3];
+#pragma unroll
+                for (int i = 0; i < 3; i++) {
+                  const int t2 = qd * kQ + 3 * hf + i;
+                  int n, m;
+                  bool v;
+                  group_nm(p, t2, &n, &m, &v);
+                  v = v && t2 <= p + 1 && 3 * hf + i < kQ;
+                  double qv = 0.0;
+#pragma unroll
+                  for (int u = 0; u < 4 * kQ; u++)
+                    if (u == t2) qv = qsv[u];
+                  const bool c1 = t2 < len1;
+                  wr[i] = v ? (c1 ? c1r : c2r) * qv : 0.0;
+                  wi[i] = v && m ? (c1 ? c1i : c2i) * qv : 0.0;
+                  const int k = v ? rl_re(n, m) : 0;
+                  pr[i] = Lb + k;
+                  pi[i] = Lb + k + (v && m ? 1 : 0);
+                }
+                if (!need_state()) {
+                  fail = true;
+                  break;
+                }
+                if (prof_on && lane == 0) prof_item(rp.prof, 9, s_tpub[gi]);
+                double lr[3], li[3];
+#pragma unroll
+                for (int i = 0; i < 3; i++) {
+                  lr[i] = __ldcg(pr[i]);
+                  li[i] = __ldcg(pi[i]);
+                }
+                double acc = wr[0] * lr[0];
+                acc = fma(wi[0], li[0], acc);
+#pragma unroll
+                for (int i = 1; i < 3; i++) {
+                  acc = fma(wr[i], lr[i], acc);
+                  acc = fma(wi[i], li[i], acc);
+                }
+                partial = warp_sum(acc);
+              } else {
               // this quarter's steps t2 = qd kQ + i (columns m1 then m2 of
               // the lane), their polynomials selected out of the registers
               TE qq[kQ];
@@ -714,6 +765,7 @@ __device__ __forceinline__ void async_body(const McSys* __restrict__ sysp, RunPa
               acc = group_sum(acc);
               const TE accn = __shfl_sync(0xffffffffu, acc, 8);
               partial = g.q * to_double(accn - acc);
+              }
             }
             // on a step without a move too: decision t then implies that
             // every apply of step t-1 is complete, which the reuse of the
@@ -864,14 +916,9 @@ __device__ __forceinline__ void async_body(const McSys* __restrict__ sysp, RunPa
                   }
                 });
               }
-              if (!need_state()) {
-                fail = true;
-                break;
-              }
-              const double hk = (cb == 0 && k < C) ? __ldcg(&S.Hhat[k]) : 0.0;
               __syncwarp();
               const int cbeg = cb * csz, cend = min(C, cbeg + csz);
-              double contrib = 0.0;
+              double wst = 0.0, contrib = 0.0;
               if (k < C) {
                 double gk = 0.0;
                 if (gpre && it == lw) {
@@ -882,11 +929,20 @@ __device__ __forceinline__ void async_body(const McSys* __restrict__ sysp, RunPa
                   for (int c = cbeg; c < cend; c++) gk += __ldcg(&S.G[(size_t)c * C + k]) * st[c];
                 }
                 S.gK[(size_t)(t & 3) * MC_NF_COLS * C + (size_t)cb * C + k] = gk;
-                const double Wk = is_square(k) ? 1.0 : 2.0;
-                contrib = Wk * st[k] * (0.5 * gk + hk);
+                wst = (is_square(k) ? 1.0 : 2.0) * st[k];
+                contrib = wst * (0.5 * gk);
               }
               if (f == 0) {
                 for (int kk = lane; kk < C; kk += 32) S.dK[(size_t)(t & 3) * C + kk] = st[kk];
+              }
+              // H is the only state a far item reads, in the items of the
+              // first column chunk
+              if (cb == 0) {
+                if (!need_state()) {
+                  fail = true;
+                  break;
+                }
+                if (k < C) contrib = fma(wst, __ldcg(&S.Hhat[k]), contrib);
               }
               partial = warp_sum(contrib);
               __syncwarp();
@@ -898,7 +954,7 @@ __device__ __forceinline__ void async_body(const McSys* __restrict__ sysp, RunPa
             ptype = 1;
             const int k0 = it - iN;
             if (!idle) {
-              const NearPart np = near_part(k0, same, nNP, 2 * nNP);
+              const NearPart np = sizeof(TE) == 8 ? near_part_sides(k0, nNP) : near_part(k0, same, nNP, 2 * nNP);
               const int k = np.k, side = np.side, part = np.part, nparts = np.nparts;
               if (!item_near<TE>(S, g, off, k, side, part, nparts, pbc, lane,
                                  [&](int, int, int) {

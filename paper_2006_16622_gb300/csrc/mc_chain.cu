@@ -608,8 +608,6 @@ __device__ __forceinline__ void chain_body(const McSys* __restrict__ sysp, RunPa
         const int grp = lane >> 3;
         const double* xg = (grp & 1) ? g.rn : g.r;
         const int k = rb * 32 + lane;
-        need_state();
-        const double hk = (cb == 0 && k < C) ? __ldcg(&S.Hhat[k]) : 0.0;
         if (dk_pre) {
           const double* src = S.dKpre + (size_t)(t & 1) * C;
           for (int kk = lane; kk < C; kk += 32) st[kk] = __ldcg(&src[kk]);
@@ -629,7 +627,7 @@ __device__ __forceinline__ void chain_body(const McSys* __restrict__ sysp, RunPa
         }
         __syncwarp();
         const int cbeg = cb * csz, cend = min(C, cbeg + csz);
-        double contrib = 0.0;
+        double wst = 0.0, contrib = 0.0;
         if (k < C) {
           double gk = 0.0;
           if (gpre && it == gw) {
@@ -640,11 +638,18 @@ __device__ __forceinline__ void chain_body(const McSys* __restrict__ sysp, RunPa
             for (int c = cbeg; c < cend; c++) gk += __ldcg(&S.G[(size_t)c * C + k]) * st[c];
           }
           S.gK[(size_t)buf * MC_NF_COLS * C + (size_t)cb * C + k] = gk;
-          const double Wk = is_square(k) ? 1.0 : 2.0;
-          contrib = Wk * st[k] * (0.5 * gk + hk);
+          wst = (is_square(k) ? 1.0 : 2.0) * st[k];
+          contrib = wst * (0.5 * gk);
         }
         if (f == 0) {
           for (int kk = lane; kk < C; kk += 32) S.dK[(size_t)buf * C + kk] = st[kk];
+        }
+        // H is the only state a far item reads, in the items of the first
+        // column chunk (gK and dK were last read by the accept of step t-2,
+        // complete since barrier 1 of step t-1)
+        if (cb == 0) {
+          need_state();
+          if (k < C) contrib = fma(wst, __ldcg(&S.Hhat[k]), contrib);
         }
         partial = warp_sum(contrib);
         __syncwarp();

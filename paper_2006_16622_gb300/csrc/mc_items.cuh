@@ -227,17 +227,16 @@ __device__ __forceinline__ bool item_image(const McSys& S, const StepGeo& g, boo
   if (pbc) {
     partial += g.q * g.q / S.a * kImageConst;
     if (S.dip == 0) {
-      if (!wait()) return false;
+      // -2 pi/(3V) (|D + d|^2 - |D|^2) = -2 pi/(3V) d.(2 D + d), d = q (r' - r):
+      // one axis per lane, d before the wait
+      const int k = lane < 3 ? lane : 0;
+      const double d = lane < 3 ? g.q * (k == 0 ? g.rn[0] - g.r[0] : (k == 1 ? g.rn[1] - g.r[1] : g.rn[2] - g.r[2])) : 0.0;
       const double cdip = -2.0 * kPi / (3.0 * S.V);
-      double D2 = 0.0, Dn2 = 0.0;
-#pragma unroll
-      for (int kk = 0; kk < 3; kk++) {
-        const double D = __ldcg(&S.dipv[kk]);
-        const double Dn = D + g.q * (g.rn[kk] - g.r[kk]);
-        D2 += D * D;
-        Dn2 += Dn * Dn;
-      }
-      partial += cdip * Dn2 - cdip * D2;
+      if (!wait()) return false;
+      const double D = __ldcg(&S.dipv[k]);
+      const double v3 = d * fma(2.0, D, d);
+      const double s3 = (__shfl_sync(0xffffffffu, v3, 0) + __shfl_sync(0xffffffffu, v3, 1)) + __shfl_sync(0xffffffffu, v3, 2);
+      partial = fma(cdip, s3, partial);
     }
   }
   *partial_out = partial;
