@@ -358,6 +358,7 @@ __device__ __forceinline__ void async_body(const McSys* __restrict__ sysp, RunPa
     long long t = 0;
     bool ok = true;
     unsigned long long cumB = 0ull;  // apply items of the accepted steps so far
+    long long c_prev = clock64(), c_ema = 0;  // last decision, mean time between decisions
     // proposal 0
     {
       double uu = 0.5;
@@ -437,6 +438,15 @@ __device__ __forceinline__ void async_body(const McSys* __restrict__ sysp, RunPa
           return &part[lane + 32 * i < nSlots ? lane + 32 * i : lane];
         };
         const void* dc = t > 0 ? (const void*)&dcnt[16 * ((t - 1) & 3)] : (const void*)&part[lane];
+        // sleep through the first 5/8 of the usual time between decisions:
+        // polling that early only takes issue slots and memory bandwidth from
+        // the items (measured on GB300: N = 1e4 9.87 -> 9.42 us a step,
+        // N = 1e5 10.75 -> 10.5, NaCl 10.4 -> 10.15; 4/8 to 5.5/8 within 1 %,
+        // 6/8 oversleeps, shorter back-offs below give nothing)
+        {
+          const long long left = (c_ema * 5 >> 3) - (clock64() - c_prev);  // cycles, ~2 per ns
+          if (left > 200) __nanosleep((unsigned)(left >> 1));
+        }
         const unsigned long long t0 = mc_globaltimer();
         unsigned spins = 0;
         while (true) {
@@ -510,6 +520,11 @@ __device__ __forceinline__ void async_body(const McSys* __restrict__ sysp, RunPa
         }
       }
       __syncwarp();
+      {
+        const long long c = clock64(), d = c - c_prev;
+        c_ema += ((d < 200000 ? d : 200000) - c_ema) >> 3;
+        c_prev = c;
+      }
       // decisions within 1e-9 of the threshold (counted after publishing)
       if (dE > 0.0 && fabs(lu - t2) < 1e-9 * fmax(1.0, fabs(t2))) n_border++;
       if (!idle) cumD[t & 3] += (unsigned long long)nDs;
