@@ -233,10 +233,18 @@ __device__ __forceinline__ void async_body(const McSys* __restrict__ sysp, RunPa
   const int bstart = nLw - 1 - lw;  // first apply item of a light warp
   const size_t nsC = (size_t)S.nsmall * C;
   // counters on their own 128-byte lines (sync[16 i]): [1..4] contributions
-  // done by step mod 4, [5] K item of step s done (s + 1), [6] decisions made
+  // done by step mod 4, [5] K item of step s done (s + 1), [6..9] CTAs whose
+  // control warp has drawn the proposal of a step, by step mod 4
   unsigned long long* dcnt = S.sync + 16;      // dcnt[16 i]: step mod 4 = i
   unsigned long long* ktag = S.sync + 16 * 5;
-  unsigned long long* decdone = S.sync + 16 * 6;
+  // A CTA draws step s after its decision s - 2, and no CTA decides step s
+  // before all have drawn it: a position is loaded before the moves of its own
+  // step and of later ones are stored, and a CTA that owns no partial slots
+  // (few cells, small p) can not fall so far behind that the slots it polls
+  // are written again.  A counter is exact: step s + 4 is drawn after decision
+  // s + 2, that is after every CTA's draw of step s.
+  unsigned long long* drawn = S.sync + 16 * 6;  // drawn[16 i]: step mod 4 = i
+  auto drawn_all = [&](long long s) { return (unsigned long long)nCTA * (unsigned long long)((s >> 2) + 1); };
 
   // far operator columns kept in registers by the light warp of F item lw
   const bool gpre = nF <= nLw && csz <= MC_GPRE;
@@ -366,6 +374,7 @@ __device__ __forceinline__ void async_body(const McSys* __restrict__ sysp, RunPa
       draw(0, &j, &pf_d, &uu, &pf_pos);
       form_geo(pg, j, pf_pos.w, axis(pf_pos), pf_d, uu);
       if (rp.nsteps > 0) ok = publish(0);
+      if (lane == 0) red_release_add(drawn, 1ull);
     }
     for (; t < rp.nsteps && ok; t++) {
       const int gi = (int)(t & 3);
@@ -415,6 +424,7 @@ __device__ __forceinline__ void async_body(const McSys* __restrict__ sysp, RunPa
           ok = false;
           break;
         }
+        if (lane == 0) red_release_add(&drawn[16 * ((t + 1) & 3)], 1ull);
       }
       if (prof_on && cta == 0 && lane == 0) rp.prof[1] += mc_globaltimer() - t_pub;
       // ---- decision of step t: the partial slots of this step, log(u),
@@ -425,11 +435,12 @@ __device__ __forceinline__ void async_body(const McSys* __restrict__ sysp, RunPa
       static_assert(kRows % 4 == 0, "the poll loads rows in groups of four");
       unsigned long long bb[kRows];
       double lu = 0.0;
+      bool late;  // complete on the first poll
       const int nRows = (nSlots + 31) / 32;  // warp-uniform
       {
         // slot of row i that this lane polls (a row past the slots repeats
         // the lane's slot of row 0: loaded, never used); lane 0 also polls
-        // log u and the contribution counter of step t-1.  Each poll is one
+        // log u, the contribution counter of step t-1 and the draws of step t.  Each poll is one
         // round trip for every row at once; the back-off between polls
         // (measured on GB300: 50 ns slowed the step's items, 150-500 ns
         // gave +3-4 % over the row-by-row poll) keeps the polling loads of
@@ -443,12 +454,15 @@ __device__ __forceinline__ void async_body(const McSys* __restrict__ sysp, RunPa
         // the items (measured on GB300: N = 1e4 9.87 -> 9.42 us a step,
         // N = 1e5 10.75 -> 10.5, NaCl 10.4 -> 10.15; 4/8 to 5.5/8 within 1 %,
         // 6/8 oversleeps, shorter back-offs below give nothing)
+        // (a sleep may last twice as long as asked for: a warp that finds the
+        // step complete on its first poll takes its mean back, below)
         {
           const long long left = (c_ema * 5 >> 3) - (clock64() - c_prev);  // cycles, ~2 per ns
           if (left > 200) __nanosleep((unsigned)(left >> 1));
         }
         const unsigned long long t0 = mc_globaltimer();
         unsigned spins = 0;
+        late = true;
         while (true) {
           unsigned long long bx[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll
@@ -459,7 +473,7 @@ __device__ __forceinline__ void async_body(const McSys* __restrict__ sysp, RunPa
               bb[g4] = bb[g4 + 1] = bb[g4 + 2] = bb[g4 + 3] = 0ull;
             }
           }
-          if (lane == 0) ld_relaxed_x4(&part[MC_MAX_ITEMS - 1], dc, slot(0), slot(0), bx);
+          if (lane == 0) ld_relaxed_x4(&part[MC_MAX_ITEMS - 1], dc, &drawn[16 * gi], slot(0), bx);
           bool all = true;
 #pragma unroll
           for (int i = 0; i < kRows; i++) all = all && (lane + 32 * i >= nSlots || bb[i] != kSentinel);
@@ -467,9 +481,11 @@ __device__ __forceinline__ void async_body(const McSys* __restrict__ sysp, RunPa
             all = all && (bx[0] != kSentinel);
             lu = __longlong_as_double((long long)bx[0]);
             if (t > 0) all = all && (bx[1] >= dprev);
+            all = all && (bx[2] >= drawn_all(t));
             if (rp.bar_missing) all = false;  // failure-path test: never complete
           }
           if (__all_sync(0xffffffffu, all)) break;
+          late = false;
           __nanosleep(350);
           int bad = 0;
           if (lane == 0 && (++spins & 63u) == 0u) {
@@ -504,7 +520,6 @@ __device__ __forceinline__ void async_body(const McSys* __restrict__ sysp, RunPa
         s_acc[t & 7] = accept ? 1 : 0;
         s_cumB[t & 7] = cumB;
         flag_publish(&s_dstep, t);
-        red_release_add(decdone, 1ull);
         if (cta == 0) {
           if (rp.log_j) {
             rp.log_j[t] = g.j;
@@ -522,7 +537,7 @@ __device__ __forceinline__ void async_body(const McSys* __restrict__ sysp, RunPa
       __syncwarp();
       {
         const long long c = clock64(), d = c - c_prev;
-        c_ema += ((d < 200000 ? d : 200000) - c_ema) >> 3;
+        c_ema += late ? -(c_ema >> 4) : ((d < 200000 ? d : 200000) - c_ema) >> 3;
         c_prev = c;
       }
       // decisions within 1e-9 of the threshold (counted after publishing)
@@ -618,11 +633,9 @@ __device__ __forceinline__ void async_body(const McSys* __restrict__ sysp, RunPa
       double* part_next = S.partials + (size_t)((t + 1) & 3) * MC_MAX_ITEMS;
       bool fail = false;
       // the owner of a partial slot resets its next-step entry (last read by
-      // the decisions of step t-3, which every CTA has made)
+      // the decisions of step t-3, which every CTA made before it drew step t-1)
       auto reset_next = [&](int slot) -> bool {
-        if (t >= 3 && !counter_wait(decdone, (unsigned long long)nCTA * (unsigned long long)(t - 2), S.status,
-                                 rp.wait_ns))
-          return false;
+        if (t >= 3 && !counter_wait(&drawn[16 * ((t - 1) & 3)], drawn_all(t - 1), S.status, rp.wait_ns)) return false;
         if (lane == 0) {
           *(unsigned long long*)&part_next[slot] = kSentinel;
           if (slot == iU) *(unsigned long long*)&part_next[MC_MAX_ITEMS - 1] = kSentinel;

@@ -197,7 +197,7 @@ int launch_chain(mc_ctx* c, RunParams& rp) {
   if (async) {
     // counters, partial-slot ring at its "not written" pattern (all bits
     // set), the four small-level contribution buffers clear
-    CK(cudaMemsetAsync(c->h.sync, 0, sizeof(unsigned long long) * 128, c->stream));
+    CK(cudaMemsetAsync(c->h.sync, 0, sizeof(unsigned long long) * 160, c->stream));
     CK(cudaMemsetAsync(c->h.partials, 0xFF, sizeof(double) * 4 * MC_MAX_ITEMS, c->stream));
     if (c->h.nsmall > 0)
       CK(cudaMemsetAsync(c->h.dsmall, 0, sizeof(double) * 4 * (size_t)c->h.nsmall * c->h.C, c->stream));
@@ -699,7 +699,7 @@ int mc_init(mc_ctx** out, int64_t n, const double* pos, const double* q, double 
   h.nsmall = h.lev_off[h.ls_end > h.L ? h.L : h.ls_end] + (h.ls_end > h.L ? h.lev_n[h.L] * h.lev_n[h.L] * h.lev_n[h.L] : 0);
   if (h.ls_end <= h.lmin) h.nsmall = 0;
   DA(h.dsmall, sizeof(double) * 4 * (size_t)std::max(1, h.nsmall) * C);
-  DA(h.sync, sizeof(unsigned long long) * 128);
+  DA(h.sync, sizeof(unsigned long long) * 160);
   DA(h.dacc, sizeof(double) * 8 * (size_t)(levels - h.lmin + 1) * MC_DSLOTS * C);
   DA(h.dKpre, sizeof(double) * 4 * C);
   DCK(cudaMemsetAsync(h.dsmall, 0, sizeof(double) * 4 * (size_t)std::max(1, h.nsmall) * C, c->stream));
