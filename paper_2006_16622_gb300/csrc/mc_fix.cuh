@@ -2,10 +2,11 @@
 //   irregular  S_n^m = sum_i q_i conj It_n^m(r_i - R)   (Alg. L.3)
 //   regular    S_n^m = sum_i q_i conj Rt_n^m(r_i - R)   (Eq. 4)
 // GB300 issues one FP64 warp instruction per ~64 cycles and sub-partition,
-// but a 32 x 32 + 64 bit integer multiply-add every 2 cycles (both measured),
-// so a 62-bit product of four multiply-adds costs 8 cycles against 64 for one
-// FP64 instruction, and it keeps more bits: every quantity below is bounded
-// by 1 by construction, is held to 2^-59 .. 2^-63, and is summed exactly.
+// but a 32 x 32 + 64 bit integer multiply-add every ~4.3 cycles (both
+// measured), so a 62-bit product of three or four multiply-adds costs 13 to 17
+// cycles against 64 for one FP64 instruction, and it keeps more bits: every
+// quantity below is bounded by 1 by construction, is held to 2^-59 .. 2^-63,
+// and is summed exactly.
 //
 // Scaling.  With R0 a radius every source satisfies (r >= R0 irregular,
 // r <= R0 regular), rho = R0/r (or r/R0) <= 1, zeta = rho cos t,
@@ -48,45 +49,34 @@ __host__ __device__ __forceinline__ Fx fx_split(int64_t v) {
   r.h = (int32_t)((uint32_t)((uint64_t)v >> 32) + ((uint32_t)v >> 31));
   return r;
 }
-// a b + c: one instruction (written out, the multiply and the add of the C
-// expressions cost two to four: a step of the recurrence 102 instead of 66
-// cycles)
+// a b + c as two multiply-adds with a carry between them.  The one wide
+// instruction takes the same 4.3 cycles but wants its sum in an aligned
+// register pair: with it Alg. L.3 for 1e5 charges at L = 4 took 5.35 instead
+// of 4.74 ms (the C expressions cost half as much again)
 __host__ __device__ __forceinline__ int64_t fx_wide(int32_t a, int32_t b, int64_t c) {
 #ifdef __CUDA_ARCH__
-  int64_t r;
-  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
-  return r;
+  int32_t lo = (int32_t)c, hi = (int32_t)(c >> 32);
+  asm("mad.lo.cc.s32 %0, %2, %3, %0;\n\tmadc.hi.s32 %1, %2, %3, %1;" : "+r"(lo), "+r"(hi) : "r"(a), "r"(b));
+  return (int64_t)(((uint64_t)(uint32_t)hi << 32) | (uint32_t)lo);
 #else
   return (int64_t)((uint64_t)((int64_t)a * (int64_t)b) + (uint64_t)c);
 #endif
 }
 __host__ __device__ __forceinline__ uint64_t fx_wideu(uint32_t a, uint32_t b, uint64_t c) {
 #ifdef __CUDA_ARCH__
-  uint64_t r;
-  asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
-  return r;
+  uint32_t lo = (uint32_t)c, hi = (uint32_t)(c >> 32);
+  asm("mad.lo.cc.u32 %0, %2, %3, %0;\n\tmadc.hi.u32 %1, %2, %3, %1;" : "+r"(lo), "+r"(hi) : "r"(a), "r"(b));
+  return ((uint64_t)hi << 32) | lo;
 #else
   return (uint64_t)a * (uint64_t)b + c;
 #endif
 }
-// acc + (t >> 32), rounded by the caller's start value of t
-__host__ __device__ __forceinline__ int64_t fx_addhi(int64_t t, int64_t acc) {
-#ifdef __CUDA_ARCH__
-  // one multiply-add: the sign extension and the two adds cost three times that
-  int64_t r;
-  asm("mad.wide.s32 %0, %1, 1, %2;" : "=l"(r) : "r"((int32_t)(t >> 32)), "l"(acc));
-  return r;
-#else
-  return (int64_t)((uint64_t)acc + (uint64_t)(t >> 32));
-#endif
-}
 constexpr int64_t kFxHalf = 0x80000000LL;
 
-// ((h 2^32 + t) / 2^32) 2^s, s < 32: the bits below the high product's last
-// one come from the cross product (a plain shift would fill zeros in: the
+// (r + (low half of t) / 2^32) 2^s, s < 32, for a cross product t whose high
+// half is in r already: the bits below r's last one come from t (a plain shift would fill zeros in: the
 // values would be good to 2^-59 instead of 2^-61)
-__host__ __device__ __forceinline__ int64_t fx_shl(int64_t t, int64_t h, int s) {
-  const int64_t r = fx_addhi(t, h);
+__host__ __device__ __forceinline__ int64_t fx_shl(int64_t t, int64_t r, int s) {
 #ifdef __CUDA_ARCH__
   const uint32_t lo = __funnelshift_l((uint32_t)t, (uint32_t)r, s);
   const uint32_t hi = __funnelshift_l((uint32_t)r, (uint32_t)((uint64_t)r >> 32), s);
@@ -99,11 +89,11 @@ __host__ __device__ __forceinline__ int64_t fx_shl(int64_t t, int64_t h, int s) 
 // the last bit before the shift) left out
 __host__ __device__ __forceinline__ int64_t fx_mul(Fx a, Fx b, int s) {
   const int64_t t = fx_wide(a.h, b.l, fx_wide(a.l, b.h, 0));
-  return fx_shl(t, fx_wide(a.h, b.h, 0), s);
+  return fx_shl(t, fx_wide(a.h, b.h, t >> 32), s);
 }
 // a b / 2^32 for a 31-bit a
 __host__ __device__ __forceinline__ int64_t fx_mulint(int32_t a, Fx b) {
-  return fx_addhi(fx_wide(a, b.l, kFxHalf), fx_wide(a, b.h, 0));
+  return fx_wide(a, b.h, fx_wide(a, b.l, kFxHalf) >> 32);
 }
 // a b / 2^62, and a c - b d, a d + b c over 2^62: one step of the powers of
 // st and of e^{i phi}
@@ -118,7 +108,7 @@ __host__ __device__ __forceinline__ void fx_turn(Fx a, Fx b, Fx c, Fx d, Fx dn, 
   u = fx_wide(b.l, c.h, u);
   t = fx_wide(b.h, dn.l, t);
   u = fx_wide(b.h, c.l, u);
-  const int64_t r = fx_wide(b.h, dn.h, fx_wide(a.h, c.h, 0)), i = fx_wide(b.h, c.h, fx_wide(a.h, d.h, 0));
+  const int64_t r = fx_wide(b.h, dn.h, fx_wide(a.h, c.h, t >> 32)), i = fx_wide(b.h, c.h, fx_wide(a.h, d.h, u >> 32));
   *re = fx_shl(t, r, 2);
   *im = fx_shl(u, i, 2);
 }
@@ -287,7 +277,7 @@ __host__ __device__ __forceinline__ Fx fix_next(Fx zs, uint32_t kh, uint32_t kl,
   t = fx_wide(zs.h, q1.l, t);
   t = fx_wide(k.l, q2.h, t);
   t = fx_wide(k.h, q2.l, t);
-  int64_t r = fx_wide(zs.h, q1.h, 0);
+  int64_t r = fx_wide(zs.h, q1.h, t >> 32);
   r = fx_wide(k.h, q2.h, r);
   return fx_split(fx_shl(t, r, sh));
 }
@@ -295,8 +285,7 @@ __host__ __device__ __forceinline__ Fx fix_next(Fx zs, uint32_t kh, uint32_t kl,
 __host__ __device__ __forceinline__ int64_t fix_mac(Fx x, Fx q, int64_t acc) {
   int64_t t = fx_wide(x.l, q.h, kFxHalf);
   t = fx_wide(x.h, q.l, t);
-  acc = fx_wide(x.h, q.h, acc);
-  return fx_addhi(t, acc);
+  return acc + fx_wide(x.h, q.h, t >> 32);
 }
 
 // Steps of the longest of four shares of the columns m = 0..p (p - m + 1

@@ -187,6 +187,14 @@ __global__ void __launch_bounds__(256)
     for (int col = warp; col < C; col += 8) M[(size_t)col * ncl + base + lane] = tile[lane * (C + 1) + col];
 }
 
+// a b + c in one instruction (the carry form of the sums over charges makes
+// this kernel 1.3 times slower: 28.7 instead of 21.6 ms at level 6)
+__device__ __forceinline__ long long m2l_wide(int a, int b, long long c) {
+  long long r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+}
+
 __device__ __forceinline__ void cta_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
@@ -331,7 +339,7 @@ __device__ __forceinline__ void m2l_task(const M2LArgs& A, const int2* __restric
         // multiples of 2^11, read off the last bits of the sum with 3 2^33
         // (|x| < 2^35; a conversion to 64 bits would use the FP64 pipe)
         const float f = x[r][t] + 25769803776.0f;
-        hh[r][t] = fx_wide(__float_as_int(f) - 0x50C00000, 2048, hh[r][t]);
+        hh[r][t] = m2l_wide(__float_as_int(f) - 0x50C00000, 2048, hh[r][t]);
         x[r][t] -= f - 25769803776.0f;
       }
   };
@@ -366,7 +374,7 @@ __device__ __forceinline__ void m2l_task(const M2LArgs& A, const int2* __restric
           const float tl = __int_as_float(r & 1 ? q.w : q.y), tf = (float)th;
 #pragma unroll
           for (int t = 0; t < NT; t++) {
-            hh[r][t] = fx_wide(th, mh[t], hh[r][t]);
+            hh[r][t] = m2l_wide(th, mh[t], hh[r][t]);
             x[r][t] = fmaf(tf, ml[t], x[r][t]);
             x[r][t] = fmaf(tl, mf[t], x[r][t]);
           }
