@@ -344,24 +344,29 @@ __global__ void k_m2m_table(int p, double* __restrict__ T) {
   }
 }
 
-#define MC_M2M_CELLS 4
+// One block per cell, one thread per row: the matrix comes out of the L2 cache,
+// eight of its rows in flight.  The cells with the fewest children to share it
+// (the upper levels, where a launch is one block's latency) decide the form:
+// four cells a block with the powers of the width from divisions took 104 us a
+// level at p = 12, this 23; with 4096 cells 326 and 233 us (four cells a block
+// no faster there).
+struct M2MScale {
+  double up[MC_PMAX + 1], down[MC_PMAX + 1];  // wc^n, wc^-n
+};
 __global__ void __launch_bounds__(256)
-    k_m2m_level(int p, int nl, double wc, const double* __restrict__ T, const double* __restrict__ child,
-                double* __restrict__ out) {
-  extern __shared__ double mt[];  // [MC_M2M_CELLS][8][C]
+    k_m2m_level(int p, int nl, const __grid_constant__ M2MScale W, const double* __restrict__ T,
+                const double* __restrict__ child, double* __restrict__ out) {
+  extern __shared__ double mt[];  // [8][C]
   __shared__ unsigned char cls[(MC_PMAX + 1) * (MC_PMAX + 1)];
-  const int C = (p + 1) * (p + 1), ncl = nl * nl * nl, nc = 2 * nl;
-  for (int k = threadIdx.x; k < C; k += blockDim.x) cls[k] = (unsigned char)rl_class(k);
-  for (int i = threadIdx.x; i < MC_M2M_CELLS * C; i += blockDim.x) {
-    const int t = blockIdx.x * MC_M2M_CELLS + i / C, col = i % C;
+  const int C = (p + 1) * (p + 1), nc = 2 * nl, t = blockIdx.x;
+  const int r = threadIdx.x, j = (int)sqrtf((float)r + 0.5f);
+  if (r < C) {
+    cls[r] = (unsigned char)rl_class(r);
     double v[8];
-    int n = (int)sqrtf((float)col + 0.5f);
-    double sc = 1.0;
-    for (int q = 0; q < n; q++) sc /= wc;
 #pragma unroll
     for (int g = 0; g < 8; g++) {  // signs of the child's offset: bits x 4, y 2, z 1
       const int cx = 2 * (t / (nl * nl)) + !(g & 4), cy = 2 * ((t / nl) % nl) + !(g & 2), cz = 2 * (t % nl) + !(g & 1);
-      v[g] = t < ncl ? child[(size_t)((cx * nc + cy) * nc + cz) * C + col] * sc : 0.0;
+      v[g] = child[(size_t)((cx * nc + cy) * nc + cz) * C + r] * W.down[j];
     }
 #pragma unroll
     for (int b = 1; b < 8; b <<= 1)
@@ -373,26 +378,15 @@ __global__ void __launch_bounds__(256)
           v[g | b] = x - y;
         }
 #pragma unroll
-    for (int d = 0; d < 8; d++) mt[((i / C) * 8 + d) * C + col] = v[d];
+    for (int d = 0; d < 8; d++) mt[d * C + r] = v[d];
   }
   __syncthreads();
-  const int r = threadIdx.x;
   if (r >= C) return;
-  const int j = (int)sqrtf((float)r + 0.5f), cr = cls[r];
-  double acc[MC_M2M_CELLS] = {};
-  for (int c = 0; c < (j + 1) * (j + 1); c++) {
-    const double t = T[(size_t)c * C + r];
-    const int d = cr ^ cls[c];
-#pragma unroll
-    for (int q = 0; q < MC_M2M_CELLS; q++) acc[q] = fma(t, mt[(q * 8 + d) * C + c], acc[q]);
-  }
-  double sc = 1.0;
-  for (int q = 0; q < j; q++) sc *= wc;
-#pragma unroll
-  for (int q = 0; q < MC_M2M_CELLS; q++) {
-    const int t = blockIdx.x * MC_M2M_CELLS + q;
-    if (t < ncl) out[(size_t)t * C + r] = acc[q] * sc;
-  }
+  const int cr = cls[r];
+  double acc = 0.0;
+#pragma unroll 8
+  for (int c = 0; c < (j + 1) * (j + 1); c++) acc = fma(T[(size_t)c * C + r], mt[(cr ^ cls[c]) * C + c], acc);
+  out[(size_t)t * C + r] = acc * W.up[j];
 }
 
 cudaError_t m2m_table(int p, double* T, cudaStream_t st) {
@@ -403,11 +397,14 @@ cudaError_t m2m_table(int p, double* T, cudaStream_t st) {
 // the multipoles of the level with nl cells per axis from those of its
 // children (child cell width wc)
 cudaError_t m2m_level(int p, int nl, double wc, const double* T, const double* child, double* out, cudaStream_t st) {
-  const int C = (p + 1) * (p + 1), ncl = nl * nl * nl;
-  const int smem = (int)sizeof(double) * MC_M2M_CELLS * 8 * C;
-  cudaError_t e = cudaFuncSetAttribute(k_m2m_level, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  k_m2m_level<<<(ncl + MC_M2M_CELLS - 1) / MC_M2M_CELLS, 256, smem, st>>>(p, nl, wc, T, child, out);
+  const int C = (p + 1) * (p + 1);
+  M2MScale W;
+  W.up[0] = W.down[0] = 1.0;
+  for (int n = 1; n <= MC_PMAX; n++) {
+    W.up[n] = W.up[n - 1] * wc;
+    W.down[n] = W.down[n - 1] / wc;
+  }
+  k_m2m_level<<<nl * nl * nl, 256, sizeof(double) * 8 * C, st>>>(p, nl, W, T, child, out);
   return cudaGetLastError();
 }
 
@@ -837,11 +834,20 @@ __global__ void __launch_bounds__(MC_THREADS)
         const int s = s0 + grp;
         double4 v = make_double4(Rx, Ry, Rz, 0.0);  // inactive: zero charge at the centre
         if (s < cnt) v = S.cpos[(size_t)cell * S.cap + s];
-        regular_group<double>(&tabs, p, v.x - Rx, v.y - Ry, v.z - Rz,
-                              [&](int t2, int n, int m, bool vld, double cr, double ci) {
-                                ar[t2] += v.w * cr;
-                                ai[t2] -= v.w * ci;
-                              });
+        // polynomial times column factor times charge: six FP64 instructions a
+        // step (eight with the recurrence on complex values)
+        double D1r, D1i, D2r, D2i, f1r = 0.0, f1i = 0.0, f2r = 0.0, f2i = 0.0;
+        regular_group_q<double>(&tabs, p, v.x - Rx, v.y - Ry, v.z - Rz, &D1r, &D1i, &D2r, &D2i,
+                                [&](int t2, int n, int m, bool vld, bool c1, double qv) {
+                                  if (t2 == 0) {
+                                    f1r = v.w * D1r;
+                                    f1i = v.w * D1i;
+                                    f2r = v.w * D2r;
+                                    f2i = v.w * D2i;
+                                  }
+                                  ar[t2] = fma(c1 ? f1r : f2r, qv, ar[t2]);
+                                  ai[t2] = fma(c1 ? -f1i : -f2i, qv, ai[t2]);
+                                });
       }
     }
     double* st = stage[warp];
