@@ -74,8 +74,10 @@ constexpr int fix_ctas(int st) { return st <= 14 ? 4 : (st <= 23 ? 3 : 2); }
 // work, and each lane keeps the sums of its coefficients in registers.  The
 // CTA forms what depends on the displacement for 128 charges at a time, one
 // per thread, in shared memory, where all four warps read it.
-// Bound by the issue of 32-bit integer instructions (one per two cycles and
-// sub-partition): 33 per coefficient and 32 charges, 23 of them multiply-adds.
+// Bound by the issue of integer instructions: 99 cycles of a sub-partition per
+// coefficient and 32 charges, 78 of them for 18 multiply-adds of 64 bits.  One
+// level of N = 1e5, p = 12 takes 4.6 ms; the same sums in FP64 (64 cycles an
+// instruction) took 41 ms.
 template <int P>
 __global__ void __launch_bounds__(kThreads, fix_ctas(fix_shares(P).steps))
     k_fix_sums(const __grid_constant__ FixArgs A, double* __restrict__ out) {
@@ -309,7 +311,11 @@ __global__ void __launch_bounds__(256)
 // q_i q_j / r_ij over the pairs of a cell with itself and with 13 of its 26
 // neighbours (the other 13 see the pair from their side).  One warp per
 // (cell, neighbour): a lane per charge of the cell, the neighbour's charges
-// staged in shared memory and read by all lanes.  Differences are exact
+// staged in shared memory and read by all lanes (or, where few of the cell's
+// charges are left, by the group of lanes whose turn they are: 4.00 -> 3.20 ms
+// for 1e6 charges, 30.5 a cell, and 121 -> 70 us for 3e4, 7.3 a cell).  About
+// 220 cycles of a sub-partition for 32 pairs, 64 of them (in parallel) the FP64
+// multiply-add.  Differences are exact
 // 64-bit integers; 1/r comes from a single-precision estimate and one
 // third-order step in integers on the difference shifted up to full length,
 // good to 2^-60, so only the last multiply-add is an FP64 instruction (one
@@ -371,7 +377,10 @@ __global__ void __launch_bounds__(256)
     const int other = (src[0] * nL + src[1]) * nL + src[2];
     const int ni = A.src.count[cell], nj = A.src.count[other];
     for (int i0 = 0; i0 < ni; i0 += 32) {
-      const int i = i0 + lane;
+      // fewer than 17 particles left: 2 to 32 groups of lanes share the other
+      // cell's particles (at 30.5 a cell a second pass has five on average)
+      const int sh = ni - i0 > 16 ? 5 : 32 - __clz(ni - i0 - 1);
+      const int i = i0 + (lane & ((1 << sh) - 1));
       int64_t xi[3] = {0, 0, 0};
       double qi = 0.0, acc = 0.0;
       if (i < ni) {
@@ -394,7 +403,7 @@ __global__ void __launch_bounds__(256)
         }
         __syncwarp();
         const int jn = min(32, nj - j0);
-        for (int j = 0; j < jn; j++) {
+        for (int j = lane >> sh; j < jn; j += 32 >> sh) {
           const int64_t* x = s_x[warp][j];
           if (i >= ni || (o == 0 && j0 + j >= i)) continue;
           int64_t d[3];
