@@ -602,16 +602,18 @@ int mc_init(mc_ctx** out, int64_t n, const double* pos, const double* q, double 
   h.lmin = (bc == MC_BC_PBC) ? 2 : 3;
   // the charges' range: the fixed-point sums take them as fractions of the
   // power of two above the largest
-  int qmax = INT_MIN, qmin = INT_MAX;
+  double qhi = 0.0, qlo = INFINITY;
   for (int64_t i = 0; i < n; i++) {
-    if (q[i] == 0.0) continue;
-    int e;
-    const double f = frexp(fabs(q[i]), &e);
-    qmax = std::max(qmax, f == 0.5 ? e - 1 : e);
-    qmin = std::min(qmin, e);
+    const double v = fabs(q[i]);
+    qhi = std::max(qhi, v);
+    qlo = std::min(qlo, v > 0.0 ? v : INFINITY);
   }
-  c->qexp = qmax == INT_MIN ? 0 : qmax;
-  c->fixed = qmax == INT_MIN || qmax - qmin <= MC_FIX_QSPAN;
+  int elo = 0;
+  if (qhi > 0.0) {
+    if (frexp(qhi, &c->qexp) == 0.5) c->qexp--;
+    frexp(qlo, &elo);
+  }
+  c->fixed = qhi == 0.0 || c->qexp - elo <= MC_FIX_QSPAN;
   int off = 0;
   for (int l = 1; l <= levels; l++) {
     h.lev_n[l] = 1 << (l - 1);
