@@ -46,7 +46,7 @@ __global__ void k_energy_dot(size_t, int, const double*, const double*, double*)
 __global__ void k_energy_sum(const McSys*, int, int, const double*, double*);
 __global__ void k_lattice_sums(int, double*);
 __global__ void k_far_operator(int, double, const double*, double*);
-__global__ void k_p2m_level(const McSys*, int, int, double*);
+__global__ void k_p2m_finest(const McSys*, double*);
 __global__ void k_offset_table(int, double*);
 cudaError_t m2l_launch(const McSys*, int, int, int, int, const double*, const double*, double*, double*,
                        size_t, cudaStream_t);
@@ -120,10 +120,10 @@ FixPass fix_pass(const mc_ctx* c, int l, bool irregular) {
   const McSys& h = c->h;
   return FixPass{h.L, l, h.p, irregular, h.bc == MC_BC_PBC, h.a, c->qexp, 1, nullptr};
 }
-// chunks of one fixed-point pass, as many as the scratch holds
-int fix_chunks_for(const McSys& h, int sms, int l, bool irregular, size_t max_doubles) {
+// chunks of one Alg. L.3 pass, as many as the scratch holds
+int fix_chunks_for(const McSys& h, int sms, int l, size_t max_doubles) {
   const size_t ncl = (size_t)1 << (3 * (l - 1));
-  const int n = fix_chunks(h.L, l, irregular, sms, (double)h.n / (double)h.ncellL, h.p);
+  const int n = fix_chunks(h.L, l, true, sms, (double)h.n / (double)h.ncellL, h.p);
   const size_t most = max_doubles / (ncl * h.C);
   return (int)std::max<size_t>(1, std::min<size_t>((size_t)n, most));
 }
@@ -212,12 +212,12 @@ int launch_chain(mc_ctx* c, RunParams& rp) {
   return MC_OK;
 }
 
-// sums of one fixed-point pass over level l into dst (C per cell)
-int fix_level(mc_ctx* c, int l, bool irregular, double* dst) {
+// Alg. L.3 of level l in fixed point into dst (C per cell)
+int fix_level(mc_ctx* c, int l, double* dst) {
   const McSys& h = c->h;
   const int ncl = 1 << (3 * (l - 1));
-  FixPass ps = fix_pass(c, l, irregular);
-  ps.nchunk = fix_chunks_for(h, c->sms, l, irregular, c->scratch_doubles);
+  FixPass ps = fix_pass(c, l, true);
+  ps.nchunk = fix_chunks_for(h, c->sms, l, c->scratch_doubles);
   CK(fix_launch(ps, fix_source(h), ps.nchunk > 1 ? c->d_scratch : dst, c->stream));
   if (ps.nchunk > 1) CK(fix_reduce(ncl, ps.nchunk, h.C, c->sms, c->d_scratch, dst, c->stream));
   return MC_OK;
@@ -250,14 +250,14 @@ int run_setup(mc_ctx* c) {
   McSys& h = c->h;
   const int C = h.C;
   // Alg. L.3 per level: a gather over the interaction list of every cell,
-  // chunked where a level has few cells.  In fixed point (8 times faster at
-  // N = 1e5, p = 12 and at least as accurate) unless the charges span more
-  // than MC_FIX_QSPAN powers of two
+  // chunked where a level has few cells.  In fixed point (4.6 ms a
+  // level at N = 1e5, p = 12 instead of 41 in FP64, and at least as accurate)
+  // unless the charges span more than MC_FIX_QSPAN powers of two
   for (int l = h.lmin; l <= h.L; l++) {
     const int nl = h.lev_n[l], ncl = nl * nl * nl;
     double* dst = h.Lhat + (size_t)h.lev_off[l] * C;
     if (c->fixed) {
-      const int rc = fix_level(c, l, true, dst);
+      const int rc = fix_level(c, l, dst);
       if (rc != MC_OK) return rc;
       continue;
     }
@@ -287,7 +287,7 @@ int p2m_levels(mc_ctx* c) {
   if (h.L >= h.lmin) {
     // finest cells hold one unit each, so one task (warp) per cell
     double* M = c->d_mpole + (size_t)h.lev_off[h.L] * C;
-    k_p2m_level<<<grid_for(c->sms, (size_t)h.ncellL, MC_WARPS), MC_THREADS, 0, c->stream>>>(c->d_sys, h.L, 1, M);
+    k_p2m_finest<<<grid_for(c->sms, (size_t)h.ncellL, MC_WARPS), MC_THREADS, 0, c->stream>>>(c->d_sys, M);
     CK(cudaGetLastError());
   }
   for (int l = h.L - 1; l >= h.lmin; l--)
@@ -718,7 +718,7 @@ int mc_init(mc_ctx** out, int64_t n, const double* pos, const double* q, double 
   size_t need = 0;
   for (int l = h.lmin; l <= levels; l++) {
     const size_t ncl = (size_t)h.lev_n[l] * h.lev_n[l] * h.lev_n[l];
-    const int nchunk = c->fixed ? fix_chunks_for(h, c->sms, l, true, kScratchCap)
+    const int nchunk = c->fixed ? fix_chunks_for(h, c->sms, l, kScratchCap)
                                 : chunks_for_level(h, c->sms, l, kScratchCap);
     if (nchunk > 1) need = std::max(need, ncl * nchunk * C);
     // offset chunks of the fast setup's multipole-to-local pass

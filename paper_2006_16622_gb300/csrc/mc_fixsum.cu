@@ -74,7 +74,7 @@ constexpr int fix_ctas(int st) { return st <= 14 ? 4 : (st <= 23 ? 3 : 2); }
 // work, and each lane keeps the sums of its coefficients in registers.  The
 // CTA forms what depends on the displacement for 128 charges at a time, one
 // per thread, in shared memory, where all four warps read it.
-// Bound by the issue of integer instructions: 99 cycles of a sub-partition per
+// Bound by the issue of integer instructions: 107 cycles of a sub-partition per
 // coefficient and 32 charges, 78 of them for 18 multiply-adds of 64 bits.  One
 // level of N = 1e5, p = 12 takes 4.6 ms; the same sums in FP64 (64 cycles an
 // instruction) took 41 ms.
@@ -313,9 +313,9 @@ __global__ void __launch_bounds__(256)
 // (cell, neighbour): a lane per charge of the cell, the neighbour's charges
 // staged in shared memory and read by all lanes (or, where few of the cell's
 // charges are left, by the group of lanes whose turn they are: 4.00 -> 3.20 ms
-// for 1e6 charges, 30.5 a cell, and 121 -> 70 us for 3e4, 7.3 a cell).  About
-// 220 cycles of a sub-partition for 32 pairs, 64 of them (in parallel) the FP64
-// multiply-add.  Differences are exact
+// for 1e6 charges, 30.5 a cell, and 121 -> 70 us for 3e4, 7.3 a cell).  At
+// 30.5 a cell 310 cycles of a sub-partition for 32 pairs, idle lanes included;
+// the FP64 multiply-add takes 64 beside the integer ones.  Differences are exact
 // 64-bit integers; 1/r comes from a single-precision estimate and one
 // third-order step in integers on the difference shifted up to full length,
 // good to 2^-60, so only the last multiply-add is an FP64 instruction (one

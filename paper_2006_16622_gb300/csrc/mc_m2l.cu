@@ -25,6 +25,12 @@
 // (one target per lane loads an entry per product, which returns 32 lanes
 // even where all are the same: 8 cycles of the SM's shared memory for the 7.4
 // of its four sub-partitions' arithmetic).
+// Level 6 of N = 1e6, p = 12 (32768 cells): 427 ms in FP64, 21.5 ms here, level
+// 5 (4096 cells) 61 and 2.7; the arithmetic alone would take half of that, the
+// rest are the transforms and the barriers between tiles.  Leaving out the
+// columns that an offset without x, y or z part does not couple (39.5 of the 56
+// products remain) gained 3 % at 32768 cells and lost 5 to 11 % below: the
+// warps of a CTA skip different columns between the same barriers.
 #include <math.h>
 
 #include <algorithm>

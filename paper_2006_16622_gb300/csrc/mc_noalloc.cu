@@ -250,7 +250,7 @@ extern "C" int mc_p2l_level_noalloc(const double* d_part, const int* d_cell_star
   P.w = box / (double)nl;
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   // charges that lie in their cells and span a few powers of two are summed
-  // in fixed point (level 4 of N = 1e5, p = 12: 104 ms in FP64); the FP64
+  // in fixed point (level 4 of N = 1e5, p = 12: 4.7 ms, in FP64 104); the FP64
   // gather does the others, and returns at once otherwise
   if (cudaMemsetAsync(range, 0, 3 * sizeof(int), stream) != cudaSuccess) {
     cudaGetLastError();

@@ -799,13 +799,15 @@ __global__ void k_far_operator(int p, double a, const double* __restrict__ St, d
 // Sec. 3.2, last paragraph: multipoles of every cell, then each cell's
 // Psi^Delta as the sum of multipole-to-local translations from the cells of
 // its interaction list (no local-to-local pass).  Scaled multipoles
-// Khat_n^m = sum q conj Rt_n^m(r - R_cell) are formed directly on every level.
+// Khat_n^m = sum q conj Rt_n^m(r - R_cell) come from the charges on the finest
+// level and from the children above it.
 
-// one warp per (cell of level l, chunk of its finest cells); four charges per
-// step; chunk partials go to out[(cell * nchunk + chunk) * C] for
-// k_reduce_chunks (nchunk = 1 writes the level directly)
+// The finest level: one warp per cell, four charges per step (upper levels:
+// k_m2m_level).  Bound by the FP64 pipe: 84 instructions of 64 cycles for the
+// steps of four charges at p = 12, about 30 for what precedes them, 64 per cell
+// for the sum over the lane groups.
 __global__ void __launch_bounds__(MC_THREADS)
-    k_p2m_level(const McSys* __restrict__ sysp, int l, int nchunk, double* __restrict__ out) {
+    k_p2m_finest(const McSys* __restrict__ sysp, double* __restrict__ out) {
   __shared__ McSys S;
   __shared__ HarmTabs<double> tabs;
   __shared__ double stage[MC_WARPS][256];
@@ -813,42 +815,33 @@ __global__ void __launch_bounds__(MC_THREADS)
   harm_tabs_init<double>(&tabs);
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = lane >> 3;
-  const int p = S.p, C = S.C, L = S.L, nL = S.nL;
-  const int nl = S.lev_n[l], f = 1 << (L - l);
-  const double w = S.lev_w[l];
-  const int nf = f * f * f, per = (nf + nchunk - 1) / nchunk;
-  const int ntask = nl * nl * nl * nchunk;
-  for (int task = blockIdx.x * MC_WARPS + warp; task < ntask; task += gridDim.x * MC_WARPS) {
-    const int t = task / nchunk, ch = task % nchunk;
-    const int tc[3] = {t / (nl * nl), (t / nl) % nl, t % nl};
-    const double Rx = (tc[0] + 0.5) * w, Ry = (tc[1] + 0.5) * w, Rz = (tc[2] + 0.5) * w;
+  const int p = S.p, C = S.C, nL = S.nL;
+  const double w = S.lev_w[S.L];
+  for (int t = blockIdx.x * MC_WARPS + warp; t < S.ncellL; t += gridDim.x * MC_WARPS) {
+    const double Rx = (t / (nL * nL) + 0.5) * w, Ry = ((t / nL) % nL + 0.5) * w, Rz = (t % nL + 0.5) * w;
     double ar[MC_PMAX + 2], ai[MC_PMAX + 2];
 #pragma unroll
     for (int q = 0; q <= MC_PMAX + 1; q++) ar[q] = ai[q] = 0.0;
-    const int fb = ch * per, fe = min(nf, fb + per);
-    for (int fc = fb; fc < fe; fc++) {
-      const int gx = tc[0] * f + fc / (f * f), gy = tc[1] * f + (fc / f) % f, gz = tc[2] * f + fc % f;
-      const int cell = (gx * nL + gy) * nL + gz;
-      const int cnt = S.ccount[cell];
-      for (int s0 = 0; s0 < cnt; s0 += 4) {
-        const int s = s0 + grp;
-        double4 v = make_double4(Rx, Ry, Rz, 0.0);  // inactive: zero charge at the centre
-        if (s < cnt) v = S.cpos[(size_t)cell * S.cap + s];
-        // polynomial times column factor times charge: six FP64 instructions a
-        // step (eight with the recurrence on complex values)
-        double D1r, D1i, D2r, D2i, f1r = 0.0, f1i = 0.0, f2r = 0.0, f2i = 0.0;
-        regular_group_q<double>(&tabs, p, v.x - Rx, v.y - Ry, v.z - Rz, &D1r, &D1i, &D2r, &D2i,
-                                [&](int t2, int n, int m, bool vld, bool c1, double qv) {
-                                  if (t2 == 0) {
-                                    f1r = v.w * D1r;
-                                    f1i = v.w * D1i;
-                                    f2r = v.w * D2r;
-                                    f2i = v.w * D2i;
-                                  }
-                                  ar[t2] = fma(c1 ? f1r : f2r, qv, ar[t2]);
-                                  ai[t2] = fma(c1 ? -f1i : -f2i, qv, ai[t2]);
-                                });
-      }
+    const int cnt = S.ccount[t];
+    for (int s0 = 0; s0 < cnt; s0 += 4) {
+      const int s = s0 + grp;
+      double4 v = make_double4(Rx, Ry, Rz, 0.0);  // inactive: zero charge at the centre
+      if (s < cnt) v = S.cpos[(size_t)t * S.cap + s];
+      // polynomial times column factor times charge: six FP64 instructions a
+      // step (eight with the recurrence on complex values: 2.50 instead of
+      // 2.20 ms for 1e6 charges at L = 6, p = 12)
+      double D1r, D1i, D2r, D2i, f1r = 0.0, f1i = 0.0, f2r = 0.0, f2i = 0.0;
+      regular_group_q<double>(&tabs, p, v.x - Rx, v.y - Ry, v.z - Rz, &D1r, &D1i, &D2r, &D2i,
+                              [&](int t2, int n, int m, bool vld, bool c1, double qv) {
+                                if (t2 == 0) {
+                                  f1r = v.w * D1r;
+                                  f1i = v.w * D1i;
+                                  f2r = v.w * D2r;
+                                  f2i = v.w * D2i;
+                                }
+                                ar[t2] = fma(c1 ? f1r : f2r, qv, ar[t2]);
+                                ai[t2] = fma(c1 ? -f1i : -f2i, qv, ai[t2]);
+                              });
     }
     double* st = stage[warp];
 #pragma unroll
@@ -868,7 +861,7 @@ __global__ void __launch_bounds__(MC_THREADS)
       }
     }
     __syncwarp();
-    double* o = out + ((size_t)t * nchunk + ch) * C;
+    double* o = out + (size_t)t * C;
     for (int kk = lane; kk < C; kk += 32) o[kk] = st[kk];
     __syncwarp();
   }
