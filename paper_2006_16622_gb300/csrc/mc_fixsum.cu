@@ -325,14 +325,27 @@ struct NearArgs {
   int L, pbc;
   uint64_t rcp;
   int ea;
+  double a;
   double unit;  // 1 / (four finest cells)
 };
 
-// 1/|(x, y, z)| for a difference in units of 2^-62 (times the caller's unit)
-__device__ __forceinline__ double near_rinv(int64_t dx, int64_t dy, int64_t dz) {
-  const uint64_t m = (uint64_t)(dx < 0 ? -dx : dx) | (uint64_t)(dy < 0 ? -dy : dy) | (uint64_t)(dz < 0 ? -dz : dz);
-  if (m == 0) return __builtin_huge_val();
-  const int k = __clzll((long long)m) - 2;
+// Pairs closer than this (leading zeros of the difference with 2^62 = four
+// finest cells, so 2^-12 of them) take their distance from the coordinates
+// themselves: a coordinate below 2^-9 of the box has bits below the integers'
+// last one, and at this distance the integers still hold the difference to
+// 2^-45.  A few near pairs in 10^10 of a uniform system are that close; they
+// are left to a second look at the two cells (a call in the loop cost a fifth
+// of the kernel).
+constexpr int kNearClose = 12;
+__device__ __forceinline__ int near_zeros(int64_t dx, int64_t dy, int64_t dz) {
+  return __clzll((long long)((uint64_t)(dx < 0 ? -dx : dx) | (uint64_t)(dy < 0 ? -dy : dy) | (uint64_t)(dz < 0 ? -dz : dz))) - 2;
+}
+
+// 1/|(x, y, z)| for a non-zero difference in units of 2^-62 (times the caller's unit)
+// and the difference's leading zeros
+__device__ __forceinline__ double near_rinv(int64_t dx, int64_t dy, int64_t dz, int* zeros) {
+  const int k = near_zeros(dx, dy, dz);
+  *zeros = k;
   const Fx x = fx_split((int64_t)((uint64_t)dx << k)), y = fx_split((int64_t)((uint64_t)dy << k)),
            z = fx_split((int64_t)((uint64_t)dz << k));
   const int64_t n2 = fx_norm(x, y, z);  // 2^60, in [1/4, 3)
@@ -352,7 +365,37 @@ __device__ __forceinline__ double near_rinv(int64_t dx, int64_t dy, int64_t dz) 
   return __longlong_as_double((long long)(((uint64_t)ex << 52) | ((top >> 11) & 0xFFFFFFFFFFFFFull)));
 }
 
-__global__ void __launch_bounds__(256)
+// component of a difference with 2^62 = four finest cells
+__device__ __forceinline__ int64_t near_diff(int64_t xi, int64_t xj, int L) {
+  const int64_t v = (int64_t)((uint64_t)xi - (uint64_t)xj);
+  return L >= 3 ? (int64_t)((uint64_t)v << (L - 3)) : v >> 1;
+}
+
+// q_i q_j / r (in the kernel's unit) over this lane's close pairs of two cells
+// (the same one: j < i)
+__device__ __noinline__ double near_close_pairs(const double4* u, int nu, const double4* v, int nv, int L, double a,
+                                                double unit, uint64_t rcp, int ea, int im) {
+  const int ix = (im & 3) - 1, iy = ((im >> 2) & 3) - 1, iz = (im >> 4) - 1;
+  double acc = 0.0;
+  for (int i = threadIdx.x & 31; i < nu; i += 32) {
+    const double4 x = ldcg4(&u[i]);
+    const int nj = u == v ? i : nv;
+    for (int j = 0; j < nj; j++) {
+      const double4 y = ldcg4(&v[j]);
+      // the image's coordinate is t + i a; the sum that is exact comes first
+      auto diff = [&](double s, double t, int i) { return i > 0 ? (s - a) - t : s - (t + i * a); };
+      auto fixed = [&](double s, double t, int i) {
+        return near_diff(fx_coord(s, rcp, ea), fx_coord(t, rcp, ea) + (int64_t)((uint64_t)(int64_t)i << 62), L);
+      };
+      if (near_zeros(fixed(x.x, y.x, ix), fixed(x.y, y.y, iy), fixed(x.z, y.z, iz)) < kNearClose) continue;
+      const double dx = diff(x.x, y.x, ix), dy = diff(x.y, y.y, iy), dz = diff(x.z, y.z, iz);
+      acc += x.w * y.w / (sqrt(dx * dx + dy * dy + dz * dz) * unit);
+    }
+  }
+  return acc;
+}
+
+__global__ void __launch_bounds__(256, 4)
     k_fix_near(const __grid_constant__ NearArgs A, double* __restrict__ out) {
   __shared__ int64_t s_x[8][32][4];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -376,6 +419,7 @@ __global__ void __launch_bounds__(256)
     if (!ok) continue;
     const int other = (src[0] * nL + src[1]) * nL + src[2];
     const int ni = A.src.count[cell], nj = A.src.count[other];
+    bool close = false;
     for (int i0 = 0; i0 < ni; i0 += 32) {
       // fewer than 17 particles left: 2 to 32 groups of lanes share the other
       // cell's particles (at 30.5 a cell a second pass has five on average)
@@ -408,15 +452,18 @@ __global__ void __launch_bounds__(256)
           if (i >= ni || (o == 0 && j0 + j >= i)) continue;
           int64_t d[3];
 #pragma unroll
-          for (int a = 0; a < 3; a++) {
-            const int64_t v = (int64_t)((uint64_t)xi[a] - (uint64_t)x[a]);
-            d[a] = A.L >= 3 ? (int64_t)((uint64_t)v << (A.L - 3)) : v >> 1;
-          }
-          acc += __longlong_as_double(x[3]) * near_rinv(d[0], d[1], d[2]);
+          for (int a = 0; a < 3; a++) d[a] = near_diff(xi[a], x[a], A.L);
+          int k;
+          const double rinv = near_rinv(d[0], d[1], d[2], &k);
+          close |= k >= kNearClose;
+          acc += k >= kNearClose ? 0.0 : __longlong_as_double(x[3]) * rinv;
         }
       }
       total += qi * acc;
     }
+    if (__any_sync(0xffffffffu, close))
+      total += near_close_pairs(&rows[(size_t)cell * cap], ni, &rows[(size_t)other * cap], nj, A.L, A.a, A.unit, A.rcp, A.ea,
+                                (im[0] + 1) | (im[1] + 1) << 2 | (im[2] + 1) << 4);
   }
   total = warp_sum(total);
   if (lane == 0) out[(size_t)blockIdx.x * 8 + warp] = total * A.unit;
@@ -440,6 +487,7 @@ cudaError_t fix_near(int L, bool pbc, double a, const FixSource& src, int blocks
   A.src = src;
   A.L = L;
   A.pbc = pbc;
+  A.a = a;
   box_scale(a, &A.rcp, &A.ea);
   A.unit = (double)(1 << (L - 1)) / (4.0 * a);
   k_fix_near<<<blocks, 256, 0, st>>>(A, out);

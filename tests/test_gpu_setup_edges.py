@@ -102,6 +102,27 @@ def test_near_pairs_by_particle_count(L, bc, mode):
     g.close()
 
 
+@pytest.mark.parametrize("d", [1e-19, 1e-15, 1e-12, 1e-9, 1e-6, 9e-4, 1.1e-3])
+@pytest.mark.parametrize("where", ["corner", "face", "middle"])
+def test_near_pair_of_any_distance(d, where):
+    """two charges d finest cells apart: at the box's corner, where their
+    coordinates have bits below 2^-62 of the box, across a periodic face and
+    in a cell"""
+    a, L = 6.4, 4
+    w = a / (1 << (L - 1))
+    pos, q = uniform_system(60, a, seed=2)
+    i, j = int(np.argmax(q)), int(np.argmin(q))
+    pos[i] = {"corner": [0.0, 0.0, 0.0], "face": [0.0, 1.3, 2.9], "middle": [1.1, 1.3, 2.9]}[where]
+    step = np.array([0.6, 0.0, 0.8]) * d * w if where == "corner" else np.array([max(d, 1e-4) * w, 0.0, 0.0])
+    pos[j] = (pos[i] + (-step if where == "face" else step)) % a
+    g, o = mcfmm.Context(pos, q, a, L, 5), O.System(pos, q, a, L, 5)
+    g.setup(mcfmm.SETUP_FMM)
+    o.setup_fmm()
+    assert np.isfinite(o.energy())
+    _energies(g, o)
+    g.close()
+
+
 def test_fresh_energy_after_moves():
     a, L, p = 8.0, 3, 9
     pos, q = uniform_system(300, a, seed=3)
