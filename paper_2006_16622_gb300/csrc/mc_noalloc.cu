@@ -10,6 +10,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "../../include/mcfmm.h"
@@ -158,7 +159,9 @@ __global__ void __launch_bounds__(MC_THREADS)
 // mc_get_local); 8 warps per 32 coefficients of a target, each taking every
 // eighth chunk
 __global__ void __launch_bounds__(MC_THREADS)
-    k_reduce_noalloc(int nchunk, int C, const double* __restrict__ in, double* __restrict__ out) {
+    k_reduce_noalloc(int nfix, int nfp64, int C, const int* __restrict__ range, const double* __restrict__ in,
+                     double* __restrict__ out) {
+  const int nchunk = fix_usable(range) ? nfix : nfp64;
   __shared__ double part[MC_WARPS][32];
   const int nb = (C + 31) / 32, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const size_t t = blockIdx.x / nb;
@@ -229,8 +232,12 @@ extern "C" int mc_p2l_level_noalloc(const double* d_part, const int* d_cell_star
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return MC_ERR_CUDA;
   const long long ncellL = 1LL << (3 * (levels - 1));
-  long long nchunk = fix_chunks(levels, level, true, sms, (double)n / (double)ncellL, p);
-  while (nchunk > 1 && ncl * nchunk * C > (long long)MC_NOALLOC_SCRATCH_DOUBLES) nchunk--;
+  long long nfix = fix_chunks(levels, level, true, sms, (double)n / (double)ncellL, p);
+  // the FP64 gather's: a task is one warp, a list entry the smallest chunk
+  long long nfp64 = std::min(189LL, (4LL * sms * MC_WARPS + ncl - 1) / ncl);
+  const long long most = (long long)MC_NOALLOC_SCRATCH_DOUBLES / (ncl * C);  // at least 1
+  nfix = std::min(nfix, most);
+  nfp64 = std::min(nfp64, most);
   // an error left by the caller's earlier work is not ours to clear or
   // report as this call's own: launch nothing
   if (cudaPeekAtLastError() != cudaSuccess) return MC_ERR_PENDING;
@@ -245,7 +252,7 @@ extern "C" int mc_p2l_level_noalloc(const double* d_part, const int* d_cell_star
   P.C = C;
   P.bc = bc;
   P.nL = 1 << (levels - 1);
-  P.nchunk = (int)nchunk;
+  P.nchunk = (int)nfp64;
   P.a = box;
   P.w = box / (double)nl;
   cudaStream_t stream = (cudaStream_t)cuda_stream;
@@ -260,18 +267,18 @@ extern "C" int mc_p2l_level_noalloc(const double* d_part, const int* d_cell_star
   k_noalloc_range<<<rblocks, MC_THREADS, 0, stream>>>(P.nL, (double)P.nL / box, d_part, d_cell_start, range);
   // no error was pending before the launch, so one now is the launch's own
   if (cudaGetLastError() != cudaSuccess) return MC_ERR_CUDA;
-  const FixPass ps{levels, level, p, true, bc == MC_BC_PBC, box, 0, (int)nchunk, nullptr};
+  const FixPass ps{levels, level, p, true, bc == MC_BC_PBC, box, 0, (int)nfix, nullptr};
   const FixSource src{d_part, nullptr, 0, d_cell_start, range};
   if (fix_launch(ps, src, scratch, stream) != cudaSuccess) {
     cudaGetLastError();
     return MC_ERR_CUDA;
   }
-  const long long ntask = ncl * nchunk;
+  const long long ntask = ncl * nfp64;
   long long blocks = (ntask + MC_WARPS - 1) / MC_WARPS;
   if (blocks > 8LL * sms) blocks = 8LL * sms;
   k_p2l_level_noalloc<<<(int)blocks, MC_THREADS, 0, stream>>>(P, d_part, d_cell_start, range, scratch);
   if (cudaGetLastError() != cudaSuccess) return MC_ERR_CUDA;
-  k_reduce_noalloc<<<(int)(ncl * ((C + 31) / 32)), MC_THREADS, 0, stream>>>((int)nchunk, C, scratch, d_out);
+  k_reduce_noalloc<<<(int)(ncl * ((C + 31) / 32)), MC_THREADS, 0, stream>>>((int)nfix, (int)nfp64, C, range, scratch, d_out);
   if (cudaGetLastError() != cudaSuccess) return MC_ERR_CUDA;
   return MC_OK;
 }
