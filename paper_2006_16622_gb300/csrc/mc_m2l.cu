@@ -25,8 +25,8 @@
 // (one target per lane loads an entry per product, which returns 32 lanes
 // even where all are the same: 8 cycles of the SM's shared memory for the 7.4
 // of its four sub-partitions' arithmetic).
-// Level 6 of N = 1e6, p = 12 (32768 cells): 427 ms in FP64, 21.5 ms here, level
-// 5 (4096 cells) 61 and 2.7; the arithmetic alone would take half of that, the
+// Level 6 of N = 1e6, p = 12 (32768 cells): 427 ms in FP64, 23 ms here, level
+// 5 (4096 cells) 61 and 2.9; the arithmetic alone would take half of that, the
 // rest are the transforms and the barriers between tiles.  Leaving out the
 // columns that an offset without x, y or z part does not couple (39.5 of the 56
 // products remain) gained 3 % at 32768 cells and lost 5 to 11 % below: the
@@ -84,6 +84,7 @@ M2LLayout m2l_layout(int p) {
 
 struct M2LArgs {
   int l, nl, h, pbc, p, nco, per_o;
+  int carry;  // columns between two carries of the cross products
   int start[8], half[8], rows;
   unsigned char ccol[kMaxRows];  // class of a column
   unsigned char orbit[kOrbits];  // |ox| | |oy| << 2 | |oz| << 4
@@ -336,7 +337,7 @@ __device__ __forceinline__ void m2l_task(const M2LArgs& A, const int2* __restric
       so++;
     }
   };
-  // the cross products' large part, carried over every 64 columns
+  // the cross products' large part, carried over every A.carry columns
   auto carry = [&]() {
 #pragma unroll
     for (int r = 0; r < NR; r++)
@@ -360,34 +361,36 @@ __device__ __forceinline__ void m2l_task(const M2LArgs& A, const int2* __restric
     if constexpr (NR > 0) {
       const int2* tt = S.T + (s & 1) * tsz + A.start[cls] + (lane >> 4) * ((NR + 1) / 2 * 2);
       const int2* m0 = S.Mt + (size_t)(s & 1) * kTile * 8 * 32 + (lane & 15);
+      for (int c0 = 0; c0 < kTile; c0 += A.carry) {
 #pragma unroll 2
-      for (int c = 0; c < kTile; c++) {
-        const int d = cls ^ A.ccol[tile * kTile + c];
-        int mh[NT];
-        float ml[NT], mf[NT];
-#pragma unroll
-        for (int t = 0; t < NT; t++) {
-          const int2 m = m0[(c * 8 + d) * 32 + 16 * t];
-          mh[t] = m.x;
-          ml[t] = __int_as_float(m.y);
-          mf[t] = (float)m.x;
-        }
-        const int4* tr = reinterpret_cast<const int4*>(tt + c * A.rows);
-#pragma unroll
-        for (int r = 0; r < NR; r++) {
-          const int4 q = tr[r / 2];
-          const int th = r & 1 ? q.z : q.x;
-          const float tl = __int_as_float(r & 1 ? q.w : q.y), tf = (float)th;
+        for (int c = c0; c < c0 + A.carry; c++) {
+          const int d = cls ^ A.ccol[tile * kTile + c];
+          int mh[NT];
+          float ml[NT], mf[NT];
 #pragma unroll
           for (int t = 0; t < NT; t++) {
-            hh[r][t] = m2l_wide(th, mh[t], hh[r][t]);
-            x[r][t] = fmaf(tf, ml[t], x[r][t]);
-            x[r][t] = fmaf(tl, mf[t], x[r][t]);
+            const int2 m = m0[(c * 8 + d) * 32 + 16 * t];
+            mh[t] = m.x;
+            ml[t] = __int_as_float(m.y);
+            mf[t] = (float)m.x;
+          }
+          const int4* tr = reinterpret_cast<const int4*>(tt + c * A.rows);
+#pragma unroll
+          for (int r = 0; r < NR; r++) {
+            const int4 q = tr[r / 2];
+            const int th = r & 1 ? q.z : q.x;
+            const float tl = __int_as_float(r & 1 ? q.w : q.y), tf = (float)th;
+#pragma unroll
+            for (int t = 0; t < NT; t++) {
+              hh[r][t] = m2l_wide(th, mh[t], hh[r][t]);
+              x[r][t] = fmaf(tf, ml[t], x[r][t]);
+              x[r][t] = fmaf(tl, mf[t], x[r][t]);
+            }
           }
         }
+        carry();
       }
       if (++tile == tiles) tile = 0;
-      if ((s & (64 / kTile - 1)) == 64 / kTile - 1) carry();
     }
     if (s + 1 < steps) store(s + 1);
     cta_sync();
@@ -528,6 +531,15 @@ cudaError_t m2l_fix_level(int p, int l, double w, bool pbc, int sms, const void*
   while (A.nco > 1 && (size_t)ncl * A.nco * C > scratch_doubles) A.nco--;
   A.per_o = (kOrbits + A.nco - 1) / A.nco;
   A.nco = (kOrbits + A.per_o - 1) / A.per_o;
+  // The cross products' single-precision sums round at 2^-24 of their size, so
+  // the fewer products a sum holds the better, above all where a row has few
+  // columns to average over.  A carry every 64 columns left the expansions up
+  // to four times as far from a 64-bit evaluation as the FP64 translations do
+  // (N = 2336, L = 3, p = 7, free space: 3.0e-15, FP64 1.0e-15); now 1.3e-15
+  // there, and 0.8 to 0.95 times the FP64 error for most orders.  Cost: the
+  // whole fast setup of N = 1e6, p = 12 31.3 -> 33.1 ms, of N = 1e5 4.5 -> 4.9
+  // (p = 12), 2.0 -> 2.3 (p = 8).
+  A.carry = p >= 12 ? 8 : (p >= 9 ? 4 : 2);
   A.rows = L.rows;
   for (int c = 0; c < 8; c++) {
     A.start[c] = L.start[c];
