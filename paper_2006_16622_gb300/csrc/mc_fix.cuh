@@ -113,8 +113,9 @@ __host__ __device__ __forceinline__ void fx_turn(Fx a, Fx b, Fx c, Fx d, Fx dn, 
   *im = fx_shl(u, i, 2);
 }
 
-// x / a in units of 2^-62 for 0 <= x <= a: rcp = 2^115 / (mantissa of a),
-// ea the biased exponent of a
+// x / a in units of 2^-62 for 0 <= x <= a (1 + 2^-14): rcp = 2^115 / (mantissa
+// of a), ea the biased exponent of a.  A row just beyond the upper face may
+// have the next exponent (s = -1, where a is just below a power of two).
 __host__ __device__ __forceinline__ int64_t fx_coord(double x, uint64_t rcp, int ea) {
 #ifdef __CUDA_ARCH__
   const uint64_t u = (uint64_t)__double_as_longlong(x);
@@ -131,7 +132,7 @@ __host__ __device__ __forceinline__ int64_t fx_coord(double x, uint64_t rcp, int
 #else
   const uint64_t v = (uint64_t)(((unsigned __int128)m * rcp) >> 64);
 #endif
-  return (int64_t)(v >> (s < 0 ? 0 : s));
+  return (int64_t)(s < 0 ? v << 1 : v >> s);
 }
 // q / 2^E in units of 2^-62 for |q| <= 2^E (E biased by 1023 like an exponent)
 __host__ __device__ __forceinline__ int64_t fx_charge(double q, int Eb) {
