@@ -2,6 +2,7 @@
 // library (declared in include/mcfmm.h).  Host code only: argument checks,
 // device memory ownership, kernel launches and copies.
 #include <cuda_runtime.h>
+#include <float.h>
 #include <limits.h>
 #include <math.h>
 #include <stdint.h>
@@ -601,7 +602,8 @@ int mc_init(mc_ctx** out, int64_t n, const double* pos, const double* q, double 
   h.ncellL = h.nL * h.nL * h.nL;
   h.lmin = (bc == MC_BC_PBC) ? 2 : 3;
   // the charges' range: the fixed-point sums take them as fractions of the
-  // power of two above the largest
+  // power of two above the largest (which has to be a double, and subnormal
+  // charges have no leading bit to take)
   double qhi = 0.0, qlo = INFINITY;
   for (int64_t i = 0; i < n; i++) {
     const double v = fabs(q[i]);
@@ -613,7 +615,7 @@ int mc_init(mc_ctx** out, int64_t n, const double* pos, const double* q, double 
     if (frexp(qhi, &c->qexp) == 0.5) c->qexp--;
     frexp(qlo, &elo);
   }
-  c->fixed = qhi == 0.0 || c->qexp - elo <= MC_FIX_QSPAN;
+  c->fixed = qhi == 0.0 || (qlo >= DBL_MIN && c->qexp < DBL_MAX_EXP && c->qexp - elo <= MC_FIX_QSPAN);
   int off = 0;
   for (int l = 1; l <= levels; l++) {
     h.lev_n[l] = 1 << (l - 1);

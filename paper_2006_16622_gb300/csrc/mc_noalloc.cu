@@ -117,8 +117,8 @@ __global__ void __launch_bounds__(MC_THREADS)
   }
 }
 
-// The range of the charges and whether every charge lies in its cell (the
-// fixed-point sums rely on the distances that gives): one warp per finest
+// The range of the charges, whether all are normal numbers, and whether every
+// charge lies in its cell (the fixed-point sums rely on the distances that gives): one warp per finest
 // cell, combined with atomic maxima.
 __global__ void __launch_bounds__(MC_THREADS)
     k_noalloc_range(int nL, double inv_w, const double* __restrict__ part, const int* __restrict__ cstart,
@@ -135,10 +135,11 @@ __global__ void __launch_bounds__(MC_THREADS)
         if (!(x >= -1.0 / 16384.0 && x <= 1.0 + 1.0 / 16384.0 && v[d] >= 0.0)) bad = 1;
       }
       const int e = (int)((__double_as_longlong(v[3]) >> 52) & 0x7ff);
-      if (e == 0x7ff) bad = 1;
       if (v[3] != 0.0) {
-        emax = max(emax, max(e, 1));
-        emin = max(emin, 4096 - max(e, 1));
+        // subnormal, or the power of two above it is no double
+        if (e == 0 || e >= 0x7fe) bad = 1;
+        emax = max(emax, e);
+        emin = max(emin, 4096 - e);
       }
     }
   }
