@@ -509,15 +509,21 @@ __global__ void k_pack_positions(size_t n, const double4* __restrict__ in, doubl
     out[i] = reinterpret_cast<const double*>(in)[4 * (i / 3) + i % 3];
 }
 
+// The read-outs pack on the device and copy straight into the caller's array,
+// in pieces of the setup scratch.  They run on the legacy stream, whose work
+// comes after that of every stream which synchronises with it: a batch that
+// only enqueued runs the chains of all its members on the first one's stream,
+// not on the stream of the context that is read.
+constexpr cudaStream_t kReadStream = nullptr;
+
 // rows of C coefficients times their factors, into a host array
 int copy_scaled(mc_ctx* c, const double* in, size_t cnt, const RowScale& f, double* out) {
   const size_t most = c->scratch_doubles / c->h.C * c->h.C;
   for (size_t i = 0; i < cnt; i += most) {
     const size_t m = std::min(most, cnt - i);
-    k_scale_rows<<<grid_for(c->sms, m, 256), 256, 0, c->stream>>>(m, c->h.C, f, in + i, c->d_scratch);
+    k_scale_rows<<<grid_for(c->sms, m, 256), 256, 0, kReadStream>>>(m, c->h.C, f, in + i, c->d_scratch);
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(out + i, c->d_scratch, sizeof(double) * m, cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
+    CK(cudaMemcpy(out + i, c->d_scratch, sizeof(double) * m, cudaMemcpyDeviceToHost));
   }
   return MC_OK;
 }
@@ -956,15 +962,12 @@ int mc_get_positions(mc_ctx* c, double* pos_out) {
   if (!c || !pos_out) return MC_ERR_ARG;
   CK(cudaSetDevice(c->dev));
   CK(cudaStreamSynchronize(c->stream));
-  // packed on the device, in pieces of the setup scratch: the copy goes
-  // straight into the caller's array
   const size_t most = c->scratch_doubles / 3;
   for (size_t i = 0; i < (size_t)c->h.n; i += most) {
     const size_t m = std::min<size_t>(most, (size_t)c->h.n - i);
-    k_pack_positions<<<grid_for(c->sms, m, 256), 256, 0, c->stream>>>(m, c->h.ppos + i, c->d_scratch);
+    k_pack_positions<<<grid_for(c->sms, m, 256), 256, 0, kReadStream>>>(m, c->h.ppos + i, c->d_scratch);
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(pos_out + 3 * i, c->d_scratch, sizeof(double) * 3 * m, cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
+    CK(cudaMemcpy(pos_out + 3 * i, c->d_scratch, sizeof(double) * 3 * m, cudaMemcpyDeviceToHost));
   }
   return MC_OK;
 }
