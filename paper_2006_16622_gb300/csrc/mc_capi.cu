@@ -416,7 +416,7 @@ int energy_chunks(const McSys& h, int sms, int l, bool irregular) {
 int energy_into(mc_ctx* c, double* d_dst, bool mpole) {
   const McSys& h = c->h;
   if (c->fixed && !h.lj_on) {
-    const int nb = fix_near_blocks(h.L, c->sms), nnear = 8 * nb;
+    const int nb = fix_near_blocks(h.L, c->sms, h.cap), nnear = 8 * nb;
     CK(fix_near(h.L, h.bc == MC_BC_PBC, h.a, fix_source(h), nb, c->d_scratch, c->stream));
     int nexp = 0;
     if (h.method == 0 && mpole && c->d_mpole) {
@@ -737,7 +737,9 @@ int mc_init(mc_ctx** out, int64_t n, const double* pos, const double* q, double 
   need = std::max(need, (size_t)c->sms * 2 * MC_WARPS);
   if (c->fixed) {
     // the energy's partials: near pairs, then the expansions of every level
-    size_t e = 8 * (size_t)fix_near_blocks(levels, c->sms) + 2 * (size_t)c->sms;
+    const size_t nnear = 8 * (size_t)fix_near_blocks(levels, c->sms, cap);
+    need = std::max(need, nnear + fix_near_work(levels, cap));
+    size_t e = nnear + 2 * (size_t)c->sms;
     for (int l = h.lmin; l <= levels; l++)
       e += ((size_t)1 << (3 * (l - 1))) *
            std::max(energy_chunks(h, c->sms, l, false), energy_chunks(h, c->sms, l, true));

@@ -392,3 +392,26 @@ inline void fix_tab_build(FixTab* T, int p, bool irregular, double R) {
     }
   }
 }
+
+// Near pairs of the energy: the ni x nj pairs of a cell with another one (or
+// with itself, `same`: each pair once) in square tiles.  Tiles of a cell pair,
+// and rows and columns of tile k (the cell itself: tiles on and below the
+// diagonal).
+#define MC_NEAR_TILE 128
+__host__ __device__ __forceinline__ long long near_tiles(int ni, int nj, bool same) {
+  const long long a = (ni + MC_NEAR_TILE - 1) / MC_NEAR_TILE, b = (nj + MC_NEAR_TILE - 1) / MC_NEAR_TILE;
+  return same ? a * (a + 1) / 2 : a * b;
+}
+__host__ __device__ __forceinline__ void near_tile(long long k, int nj, bool same, int* ti, int* tj) {
+  if (same) {
+    long long i = (long long)((sqrt(8.0 * (double)k + 1.0) - 1.0) * 0.5);
+    while (i * (i + 1) / 2 > k) i--;
+    while ((i + 1) * (i + 2) / 2 <= k) i++;
+    *ti = (int)i;
+    *tj = (int)(k - i * (i + 1) / 2);
+  } else {
+    const long long b = (nj + MC_NEAR_TILE - 1) / MC_NEAR_TILE;
+    *ti = (int)(k / b);
+    *tj = (int)(k % b);
+  }
+}

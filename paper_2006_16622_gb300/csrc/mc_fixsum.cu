@@ -309,11 +309,16 @@ __global__ void __launch_bounds__(256)
 
 // ------------------------------------------------------ near pairs (energy)
 // q_i q_j / r_ij over the pairs of a cell with itself and with 13 of its 26
-// neighbours (the other 13 see the pair from their side).  One warp per
-// (cell, neighbour): a lane per charge of the cell, the neighbour's charges
-// staged in shared memory and read by all lanes (or, where few of the cell's
-// charges are left, by the group of lanes whose turn they are: 4.00 -> 3.20 ms
-// for 1e6 charges, 30.5 a cell, and 121 -> 70 us for 3e4, 7.3 a cell).  At
+// neighbours (the other 13 see the pair from their side).  One warp per tile of
+// 128 x 128 pairs of a (cell, neighbour): a lane per charge of the cell, the
+// neighbour's charges staged in shared memory and read by all lanes (or, where
+// few of the tile's charges are left, by the group of lanes whose turn they
+// are: 4.00 -> 3.20 ms for 1e6 charges, 30.5 a cell, and 121 -> 70 us for 3e4,
+// 7.3 a cell).  The first tiles of all (cell, neighbour) come first; where
+// cells may hold more than a tile, the others are counted by k_near_extra and
+// dealt out in order (4000 of 8000 charges in one cell, L = 5, whole fresh
+// energy: 79 ms with one warp for a (cell, neighbour), 0.93 now, 1.0 with the
+// FP64 kernel's warp per charge; 8 x 4000: 183, 5.7 and 37 ms).  At
 // 30.5 a cell 310 cycles of a sub-partition for 32 pairs, idle lanes included;
 // the FP64 multiply-add takes 64 beside the integer ones.  Differences are exact
 // 64-bit integers; 1/r comes from a single-precision estimate and one
@@ -327,7 +332,90 @@ struct NearArgs {
   int ea;
   double a;
   double unit;  // 1 / (four finest cells)
+  // tiles beyond the first ones, of every cell and of every 1024 cells (null:
+  // no cell can hold more than a tile)
+  const long long *cells, *blocks;
 };
+constexpr int kNearBlock = 1024;  // cells counted by a block of k_near_extra
+
+// neighbour o (0: itself, else one of 13) of a cell: its index, image shifts,
+// and whether it exists
+__device__ __forceinline__ bool near_neighbour(int cell, int o, int nL, bool pbc, int* other, int* im) {
+  const int c[3] = {cell / (nL * nL), (cell / nL) % nL, cell % nL}, k = 13 + o;
+  const int e[3] = {c[0] + k / 9 - 1, c[1] + (k / 3) % 3 - 1, c[2] + k % 3 - 1};
+  int src[3];
+  bool ok = true;
+#pragma unroll
+  for (int d = 0; d < 3; d++) {
+    src[d] = mc_wrap_coord(e[d], nL);
+    im[d] = (e[d] - src[d]) / nL;
+    if (!pbc && im[d]) ok = false;
+  }
+  *other = (src[0] * nL + src[1]) * nL + src[2];
+  return ok;
+}
+// tiles of (cell, neighbour o) beyond the first
+__device__ __forceinline__ long long near_extra(const NearArgs& A, int cell, int o, int nL) {
+  int other, im[3];
+  if (o >= 14 || !near_neighbour(cell, o, nL, A.pbc, &other, im)) return 0;
+  return max(near_tiles(A.src.count[cell], A.src.count[other], o == 0) - 1, 0ll);
+}
+
+__global__ void __launch_bounds__(kNearBlock)
+    k_near_extra(const __grid_constant__ NearArgs A, long long* __restrict__ cells, long long* __restrict__ blocks) {
+  __shared__ long long part[kNearBlock / 32];
+  const int nL = 1 << (A.L - 1), cell = blockIdx.x * kNearBlock + threadIdx.x;
+  long long v = 0;
+  if (cell < nL * nL * nL) {
+    for (int o = 0; o < 14; o++) v += near_extra(A, cell, o, nL);
+    cells[cell] = v;
+  }
+  for (int m = 16; m; m >>= 1) v += shfl_xor64(v, m);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kNearBlock / 32; w++) v += part[w];
+    blocks[blockIdx.x] = v;
+  }
+}
+
+// entry of 32 (one per lane) that item e of their sum lies in, the items
+// before it taken off e; 32 if e lies beyond them all
+__device__ __forceinline__ int near_find(long long v, long long* e) {
+  const int lane = threadIdx.x & 31;
+  long long inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long u = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += u;
+  }
+  const unsigned past = __ballot_sync(0xffffffffu, inc > *e);
+  const int k = past ? __ffs(past) - 1 : 32;
+  const long long before = __shfl_sync(0xffffffffu, inc - v, k & 31), all = __shfl_sync(0xffffffffu, inc, 31);
+  *e -= k < 32 ? before : all;
+  return k;
+}
+// cell, neighbour and tile of extra tile e (all lanes the same); false beyond
+// the last one
+__device__ __noinline__ bool near_locate(const NearArgs& A, long long e, int nL, int* cell, int* o, long long* tile) {
+  const int lane = threadIdx.x & 31, ncell = nL * nL * nL, nb = (ncell + kNearBlock - 1) / kNearBlock;
+  int b = 32;
+  for (int b0 = 0; b0 < nb && b == 32; b0 += 32) {
+    b = near_find(b0 + lane < nb ? A.blocks[b0 + lane] : 0ll, &e);
+    if (b < 32) {
+      for (int c0 = (b0 + b) * kNearBlock; c0 < (b0 + b + 1) * kNearBlock; c0 += 32) {
+        const int k = near_find(c0 + lane < ncell ? A.cells[c0 + lane] : 0ll, &e);
+        if (k == 32) continue;
+        *cell = c0 + k;
+        *o = near_find(near_extra(A, *cell, lane, nL), &e);
+        *tile = 1 + e;
+        return *o < 14;
+      }
+      return false;
+    }
+  }
+  return false;
+}
 
 // Pairs closer than this (leading zeros of the difference with 2^62 = four
 // finest cells, so 2^-12 of them) take their distance from the coordinates
@@ -371,16 +459,16 @@ __device__ __forceinline__ int64_t near_diff(int64_t xi, int64_t xj, int L) {
   return L >= 3 ? (int64_t)((uint64_t)v << (L - 3)) : v >> 1;
 }
 
-// q_i q_j / r (in the kernel's unit) over this lane's close pairs of two cells
-// (the same one: j < i)
-__device__ __noinline__ double near_close_pairs(const double4* u, int nu, const double4* v, int nv, int L, double a,
-                                                double unit, uint64_t rcp, int ea, int im) {
+// q_i q_j / r (in the kernel's unit) over this lane's close pairs of charges
+// i0..i1 of a cell and j0..j1 of another (the same one: j < i)
+__device__ __noinline__ double near_close_pairs(const double4* u, int i0, int i1, const double4* v, int j0, int j1, int L,
+                                                double a, double unit, uint64_t rcp, int ea, int im) {
   const int ix = (im & 3) - 1, iy = ((im >> 2) & 3) - 1, iz = (im >> 4) - 1;
   double acc = 0.0;
-  for (int i = threadIdx.x & 31; i < nu; i += 32) {
+  for (int i = i0 + (threadIdx.x & 31); i < i1; i += 32) {
     const double4 x = ldcg4(&u[i]);
-    const int nj = u == v ? i : nv;
-    for (int j = 0; j < nj; j++) {
+    const int je = u == v ? min(i, j1) : j1;
+    for (int j = j0; j < je; j++) {
       const double4 y = ldcg4(&v[j]);
       // the image's coordinate is t + i a; the sum that is exact comes first
       auto diff = [&](double s, double t, int i) { return i > 0 ? (s - a) - t : s - (t + i * a); };
@@ -403,24 +491,19 @@ __global__ void __launch_bounds__(256, 4)
   const long long tasks = 14LL * nL * nL * nL;
   const double4* rows = reinterpret_cast<const double4*>(A.src.rows);
   double total = 0.0;
-  for (long long task = (long long)blockIdx.x * 8 + warp; task < tasks; task += (long long)gridDim.x * 8) {
-    const int cell = (int)(task / 14), o = (int)(task % 14);  // o = 0: the cell itself
-    const int c[3] = {cell / (nL * nL), (cell / nL) % nL, cell % nL};
-    const int k = 13 + o;
-    int e[3] = {c[0] + k / 9 - 1, c[1] + (k / 3) % 3 - 1, c[2] + k % 3 - 1};
-    int src[3], im[3];
-    bool ok = true;
-#pragma unroll
-    for (int d = 0; d < 3; d++) {
-      src[d] = mc_wrap_coord(e[d], nL);
-      im[d] = (e[d] - src[d]) / nL;
-      if (!A.pbc && im[d]) ok = false;
-    }
-    if (!ok) continue;
-    const int other = (src[0] * nL + src[1]) * nL + src[2];
-    const int ni = A.src.count[cell], nj = A.src.count[other];
+  for (long long task = (long long)blockIdx.x * 8 + warp;; task += (long long)gridDim.x * 8) {
+    int cell = (int)(task / 14), o = (int)(task % 14), ti = 0, tj = 0;  // o = 0: the cell itself
+    long long tile = 0;
+    if (task >= tasks && !(A.cells && near_locate(A, task - tasks, nL, &cell, &o, &tile))) break;
+    int other, im[3];
+    if (!near_neighbour(cell, o, nL, A.pbc, &other, im)) continue;
+    int ni = A.src.count[cell], nj = A.src.count[other];
+    if (tile) near_tile(tile, nj, o == 0, &ti, &tj);
+    const int ib = ti * MC_NEAR_TILE, jb = tj * MC_NEAR_TILE;
+    ni = min(ni, ib + MC_NEAR_TILE);
+    nj = min(nj, jb + MC_NEAR_TILE);
     bool close = false;
-    for (int i0 = 0; i0 < ni; i0 += 32) {
+    for (int i0 = ib; i0 < ni; i0 += 32) {
       // fewer than 17 particles left: 2 to 32 groups of lanes share the other
       // cell's particles (at 30.5 a cell a second pass has five on average)
       const int sh = ni - i0 > 16 ? 5 : 32 - __clz(ni - i0 - 1);
@@ -434,7 +517,7 @@ __global__ void __launch_bounds__(256, 4)
         xi[2] = fx_coord(r.z, A.rcp, A.ea);
         qi = r.w;
       }
-      for (int j0 = 0; j0 < nj; j0 += 32) {
+      for (int j0 = jb; j0 < nj; j0 += 32) {
         if (o == 0 && j0 > i0) break;  // pairs i > j
         __syncwarp();
         if (j0 + lane < nj) {
@@ -462,16 +545,17 @@ __global__ void __launch_bounds__(256, 4)
       total += qi * acc;
     }
     if (__any_sync(0xffffffffu, close))
-      total += near_close_pairs(&rows[(size_t)cell * cap], ni, &rows[(size_t)other * cap], nj, A.L, A.a, A.unit, A.rcp, A.ea,
-                                (im[0] + 1) | (im[1] + 1) << 2 | (im[2] + 1) << 4);
+      total += near_close_pairs(&rows[(size_t)cell * cap], ib, ni, &rows[(size_t)other * cap], jb, nj, A.L, A.a, A.unit,
+                                A.rcp, A.ea, (im[0] + 1) | (im[1] + 1) << 2 | (im[2] + 1) << 4);
   }
   total = warp_sum(total);
   if (lane == 0) out[(size_t)blockIdx.x * 8 + warp] = total * A.unit;
 }
 
-int fix_near_blocks(int L, int sms) {
-  const long long b = (14LL << (3 * (L - 1))) / 8 + 1;
-  return (int)std::min<long long>(b, 8LL * sms);
+int fix_near_blocks(int L, int sms, int cap) {
+  // a warp per tile, if every cell were full
+  const double tiles = (double)(14LL << (3 * (L - 1))) * (double)near_tiles(cap, cap, false);
+  return (int)std::min(tiles / 8.0 + 1.0, 8.0 * sms);
 }
 
 static void box_scale(double a, uint64_t* rcp, int* ea) {
@@ -482,6 +566,11 @@ static void box_scale(double a, uint64_t* rcp, int* ea) {
   *rcp = (uint64_t)((((unsigned __int128)1 << 115) + m / 2) / m);
 }
 
+size_t fix_near_work(int L, int cap) {
+  const size_t ncell = (size_t)1 << (3 * (L - 1));
+  return cap <= MC_NEAR_TILE ? 0 : ncell + (ncell + kNearBlock - 1) / kNearBlock;
+}
+
 cudaError_t fix_near(int L, bool pbc, double a, const FixSource& src, int blocks, double* out, cudaStream_t st) {
   NearArgs A;
   A.src = src;
@@ -490,6 +579,16 @@ cudaError_t fix_near(int L, bool pbc, double a, const FixSource& src, int blocks
   A.a = a;
   box_scale(a, &A.rcp, &A.ea);
   A.unit = (double)(1 << (L - 1)) / (4.0 * a);
+  A.cells = A.blocks = nullptr;
+  if (fix_near_work(L, src.cap)) {
+    const int ncell = 1 << (3 * (L - 1)), nb = (ncell + kNearBlock - 1) / kNearBlock;
+    long long* cells = reinterpret_cast<long long*>(out + 8 * (size_t)blocks);
+    k_near_extra<<<nb, kNearBlock, 0, st>>>(A, cells, cells + ncell);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    A.cells = cells;
+    A.blocks = cells + ncell;
+  }
   k_fix_near<<<blocks, 256, 0, st>>>(A, out);
   return cudaGetLastError();
 }

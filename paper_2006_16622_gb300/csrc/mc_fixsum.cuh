@@ -36,8 +36,10 @@ int fix_chunks(int L, int l, bool irregular, int sms, double occupancy, int p);
 cudaError_t fix_launch(const FixPass& ps, const FixSource& src, double* out, cudaStream_t st);
 // Direct part of the energy: 1/r over the pairs of charges within near cells
 // (every pair and image once), one partial per warp of the returned number
-// of blocks of 256 threads
-int fix_near_blocks(int L, int sms);
+// of blocks of 256 threads, followed by the workspace of fix_near_work doubles
+// (of use until the call's kernels are done)
+int fix_near_blocks(int L, int sms, int cap);
+size_t fix_near_work(int L, int cap);
 cudaError_t fix_near(int L, bool pbc, double a, const FixSource& src, int blocks, double* out, cudaStream_t st);
 // charges of this span of exponents (largest minus smallest) keep the
 // fixed-point sums at least as accurate as FP64 ones
