@@ -134,6 +134,29 @@ __host__ __device__ __forceinline__ int64_t fx_coord(double x, uint64_t rcp, int
 #endif
   return (int64_t)(s < 0 ? v << 1 : v >> s);
 }
+// x in units of 2^-60 finest cells (2^62: four of them) modulo 2^64, for
+// 0 <= x < a and L levels: r1 2^64 + r0 = 2^179 / (mantissa of a).  Rounded
+// down by less than two units wherever x lies; a fraction of the box in 62
+// bits, shifted up, was off by up to 2^(L-3) units.
+__host__ __device__ __forceinline__ int64_t fx_cells(double x, uint64_t r1, uint64_t r0, int ea, int L) {
+#ifdef __CUDA_ARCH__
+  const uint64_t u = (uint64_t)__double_as_longlong(x);
+#else
+  uint64_t u;
+  __builtin_memcpy(&u, &x, 8);
+#endif
+  const int e = (int)((u >> 52) & 0x7ff), s = ea - e - (L - 3);
+  if (e == 0 || s > 62) return 0;
+  const uint64_t m = ((u & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 11;
+#ifdef __CUDA_ARCH__
+  const uint64_t h = __umul64hi(m, r1), l = __umul64hi(m, r0);
+#else
+  const uint64_t h = (uint64_t)(((unsigned __int128)m * r1) >> 64);
+  const uint64_t l = (uint64_t)(((unsigned __int128)m * r0) >> 64);
+#endif
+  const uint64_t lo = m * r1 + l, hi = h + (lo < l);
+  return (int64_t)(s > 0 ? hi >> s : s == 0 ? hi : (hi << -s) | (lo >> (64 + s)));
+}
 // q / 2^E in units of 2^-62 for |q| <= 2^E (E biased by 1023 like an exponent)
 __host__ __device__ __forceinline__ int64_t fx_charge(double q, int Eb) {
 #ifdef __CUDA_ARCH__

@@ -328,8 +328,9 @@ __global__ void __launch_bounds__(256)
 struct NearArgs {
   FixSource src;
   int L, pbc;
-  uint64_t rcp;
+  uint64_t rcp[2];  // fx_cells' reciprocal of the box side
   int ea;
+  uint64_t box;  // the box side in units of 2^-60 finest cells, modulo 2^64
   double a;
   double unit;  // 1 / (four finest cells)
   // tiles beyond the first ones, of every cell and of every 1024 cells (null:
@@ -418,13 +419,15 @@ __device__ __noinline__ bool near_locate(const NearArgs& A, long long e, int nL,
 }
 
 // Pairs closer than this (leading zeros of the difference with 2^62 = four
-// finest cells, so 2^-12 of them) take their distance from the coordinates
-// themselves: a coordinate below 2^-9 of the box has bits below the integers'
-// last one, and at this distance the integers still hold the difference to
-// 2^-45.  A few near pairs in 10^10 of a uniform system are that close; they
-// are left to a second look at the two cells (a call in the loop cost a fifth
-// of the kernel).
-constexpr int kNearClose = 12;
+// finest cells, so 2^-9 of them in every component) take their distance from
+// the coordinates themselves.  The two coordinates of a difference are rounded
+// down by up to 2^-60 of a cell, which is 2^-54 (rms) of the distance at this
+// line, as much as the FP64 operations of the other route; with the line at
+// 2^-12 it was 2^-51, and 2^(L-3) times that with coordinates in 2^-62 of the
+// box.  One own cell in a thousand at 24 charges a cell has such a pair; it is
+// left to a second look at the tile (a call in the loop cost a fifth of the
+// kernel).
+constexpr int kNearClose = 9;
 __device__ __forceinline__ int near_zeros(int64_t dx, int64_t dy, int64_t dz) {
   return __clzll((long long)((uint64_t)(dx < 0 ? -dx : dx) | (uint64_t)(dy < 0 ? -dy : dy) | (uint64_t)(dz < 0 ? -dz : dz))) - 2;
 }
@@ -453,16 +456,16 @@ __device__ __forceinline__ double near_rinv(int64_t dx, int64_t dy, int64_t dz, 
   return __longlong_as_double((long long)(((uint64_t)ex << 52) | ((top >> 11) & 0xFFFFFFFFFFFFFull)));
 }
 
-// component of a difference with 2^62 = four finest cells
-__device__ __forceinline__ int64_t near_diff(int64_t xi, int64_t xj, int L) {
-  const int64_t v = (int64_t)((uint64_t)xi - (uint64_t)xj);
-  return L >= 3 ? (int64_t)((uint64_t)v << (L - 3)) : v >> 1;
+// a coordinate in units of 2^-60 finest cells, modulo 2^64, of an image
+__device__ __forceinline__ int64_t near_coord(const NearArgs& A, double x, int image) {
+  return (int64_t)((uint64_t)fx_cells(x, A.rcp[0], A.rcp[1], A.ea, A.L) + (uint64_t)(int64_t)image * A.box);
 }
+__device__ __forceinline__ int64_t near_diff(int64_t xi, int64_t xj) { return (int64_t)((uint64_t)xi - (uint64_t)xj); }
 
 // q_i q_j / r (in the kernel's unit) over this lane's close pairs of charges
 // i0..i1 of a cell and j0..j1 of another (the same one: j < i)
-__device__ __noinline__ double near_close_pairs(const double4* u, int i0, int i1, const double4* v, int j0, int j1, int L,
-                                                double a, double unit, uint64_t rcp, int ea, int im) {
+__device__ __noinline__ double near_close_pairs(const NearArgs& A, const double4* u, int i0, int i1, const double4* v,
+                                                int j0, int j1, int im) {
   const int ix = (im & 3) - 1, iy = ((im >> 2) & 3) - 1, iz = (im >> 4) - 1;
   double acc = 0.0;
   for (int i = i0 + (threadIdx.x & 31); i < i1; i += 32) {
@@ -471,13 +474,11 @@ __device__ __noinline__ double near_close_pairs(const double4* u, int i0, int i1
     for (int j = j0; j < je; j++) {
       const double4 y = ldcg4(&v[j]);
       // the image's coordinate is t + i a; the sum that is exact comes first
-      auto diff = [&](double s, double t, int i) { return i > 0 ? (s - a) - t : s - (t + i * a); };
-      auto fixed = [&](double s, double t, int i) {
-        return near_diff(fx_coord(s, rcp, ea), fx_coord(t, rcp, ea) + (int64_t)((uint64_t)(int64_t)i << 62), L);
-      };
+      auto diff = [&](double s, double t, int i) { return i > 0 ? (s - A.a) - t : s - (t + i * A.a); };
+      auto fixed = [&](double s, double t, int i) { return near_diff(near_coord(A, s, 0), near_coord(A, t, i)); };
       if (near_zeros(fixed(x.x, y.x, ix), fixed(x.y, y.y, iy), fixed(x.z, y.z, iz)) < kNearClose) continue;
       const double dx = diff(x.x, y.x, ix), dy = diff(x.y, y.y, iy), dz = diff(x.z, y.z, iz);
-      acc += x.w * y.w / (sqrt(dx * dx + dy * dy + dz * dz) * unit);
+      acc += x.w * y.w / (sqrt(dx * dx + dy * dy + dz * dz) * A.unit);
     }
   }
   return acc;
@@ -512,9 +513,9 @@ __global__ void __launch_bounds__(256, 4)
       double qi = 0.0, acc = 0.0;
       if (i < ni) {
         const double4 r = ldcg4(&rows[(size_t)cell * cap + i]);
-        xi[0] = fx_coord(r.x, A.rcp, A.ea);
-        xi[1] = fx_coord(r.y, A.rcp, A.ea);
-        xi[2] = fx_coord(r.z, A.rcp, A.ea);
+        xi[0] = near_coord(A, r.x, 0);
+        xi[1] = near_coord(A, r.y, 0);
+        xi[2] = near_coord(A, r.z, 0);
         qi = r.w;
       }
       for (int j0 = jb; j0 < nj; j0 += 32) {
@@ -523,9 +524,9 @@ __global__ void __launch_bounds__(256, 4)
         if (j0 + lane < nj) {
           const double4 r = ldcg4(&rows[(size_t)other * cap + j0 + lane]);
           int64_t* x = s_x[warp][lane];
-          x[0] = fx_coord(r.x, A.rcp, A.ea) + (int64_t)((uint64_t)(int64_t)im[0] << 62);
-          x[1] = fx_coord(r.y, A.rcp, A.ea) + (int64_t)((uint64_t)(int64_t)im[1] << 62);
-          x[2] = fx_coord(r.z, A.rcp, A.ea) + (int64_t)((uint64_t)(int64_t)im[2] << 62);
+          x[0] = near_coord(A, r.x, im[0]);
+          x[1] = near_coord(A, r.y, im[1]);
+          x[2] = near_coord(A, r.z, im[2]);
           x[3] = __double_as_longlong(r.w);
         }
         __syncwarp();
@@ -535,7 +536,7 @@ __global__ void __launch_bounds__(256, 4)
           if (i >= ni || (o == 0 && j0 + j >= i)) continue;
           int64_t d[3];
 #pragma unroll
-          for (int a = 0; a < 3; a++) d[a] = near_diff(xi[a], x[a], A.L);
+          for (int a = 0; a < 3; a++) d[a] = near_diff(xi[a], x[a]);
           int k;
           const double rinv = near_rinv(d[0], d[1], d[2], &k);
           close |= k >= kNearClose;
@@ -545,8 +546,8 @@ __global__ void __launch_bounds__(256, 4)
       total += qi * acc;
     }
     if (__any_sync(0xffffffffu, close))
-      total += near_close_pairs(&rows[(size_t)cell * cap], ib, ni, &rows[(size_t)other * cap], jb, nj, A.L, A.a, A.unit,
-                                A.rcp, A.ea, (im[0] + 1) | (im[1] + 1) << 2 | (im[2] + 1) << 4);
+      total += near_close_pairs(A, &rows[(size_t)cell * cap], ib, ni, &rows[(size_t)other * cap], jb, nj,
+                                (im[0] + 1) | (im[1] + 1) << 2 | (im[2] + 1) << 4);
   }
   total = warp_sum(total);
   if (lane == 0) out[(size_t)blockIdx.x * 8 + warp] = total * A.unit;
@@ -577,7 +578,16 @@ cudaError_t fix_near(int L, bool pbc, double a, const FixSource& src, int blocks
   A.L = L;
   A.pbc = pbc;
   A.a = a;
-  box_scale(a, &A.rcp, &A.ea);
+  {
+    uint64_t u;
+    __builtin_memcpy(&u, &a, 8);
+    A.ea = (int)((u >> 52) & 0x7ff);
+    const uint64_t m = (u & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
+    const unsigned __int128 top = (unsigned __int128)1 << 115;
+    A.rcp[0] = (uint64_t)(top / m);
+    A.rcp[1] = (uint64_t)((top % m << 64) / m);
+  }
+  A.box = L < 5 ? 1ull << (59 + L) : 0ull;
   A.unit = (double)(1 << (L - 1)) / (4.0 * a);
   A.cells = A.blocks = nullptr;
   if (fix_near_work(L, src.cap)) {
