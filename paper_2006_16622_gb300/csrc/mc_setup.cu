@@ -818,20 +818,23 @@ __global__ void __launch_bounds__(MC_THREADS)
   const int p = S.p, C = S.C, nL = S.nL;
   const double w = S.lev_w[S.L];
   for (int t = blockIdx.x * MC_WARPS + warp; t < S.ncellL; t += gridDim.x * MC_WARPS) {
-    const double Rx = (t / (nL * nL) + 0.5) * w, Ry = ((t / nL) % nL + 0.5) * w, Rz = (t % nL + 0.5) * w;
+    // centre in cell widths; the differences below take it times w unrounded
+    // (rounded, it cost a digit: multipoles of 1200 charges at L = 3, p = 6
+    // were off by 1.7e-15 instead of 3.0e-16 of their norm)
+    const double gx = t / (nL * nL) + 0.5, gy = (t / nL) % nL + 0.5, gz = t % nL + 0.5;
     double ar[MC_PMAX + 2], ai[MC_PMAX + 2];
 #pragma unroll
     for (int q = 0; q <= MC_PMAX + 1; q++) ar[q] = ai[q] = 0.0;
     const int cnt = S.ccount[t];
     for (int s0 = 0; s0 < cnt; s0 += 4) {
       const int s = s0 + grp;
-      double4 v = make_double4(Rx, Ry, Rz, 0.0);  // inactive: zero charge at the centre
+      double4 v = make_double4(gx * w, gy * w, gz * w, 0.0);  // inactive: zero charge at the centre
       if (s < cnt) v = S.cpos[(size_t)t * S.cap + s];
       // polynomial times column factor times charge: six FP64 instructions a
       // step (eight with the recurrence on complex values: 2.50 instead of
       // 2.20 ms for 1e6 charges at L = 6, p = 12)
       double D1r, D1i, D2r, D2i, f1r = 0.0, f1i = 0.0, f2r = 0.0, f2i = 0.0;
-      regular_group_q<double>(&tabs, p, v.x - Rx, v.y - Ry, v.z - Rz, &D1r, &D1i, &D2r, &D2i,
+      regular_group_q<double>(&tabs, p, fma(-gx, w, v.x), fma(-gy, w, v.y), fma(-gz, w, v.z), &D1r, &D1i, &D2r, &D2i,
                               [&](int t2, int n, int m, bool vld, bool c1, double qv) {
                                 if (t2 == 0) {
                                   f1r = v.w * D1r;
