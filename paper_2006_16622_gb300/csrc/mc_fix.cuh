@@ -32,9 +32,9 @@
 #define MC_FIX_WARPS 4   // warps that share the columns
 #define MC_FIX_STEPS 34  // most recurrence steps of one warp (p = 15)
 // groups of 32 charges between two flushes of a lane's sums: one term is at
-// most 2^58, so 28 stay below 2^63, and after the shift by 5 the sum over
-// the 32 lanes does too (a bit more for the terms would double the flushes,
-// 3 % of the kernel)
+// most 2^58, so 28 stay below 2^63, and halved before each exchange the sum
+// over the 32 lanes does too (a bit more for the terms would double the
+// flushes, 3 % of the kernel)
 #define MC_FIX_FLUSH 28
 #define MC_FIX_PHASE 2  // cos m phi, sin m phi enter the terms as multiples of 2^-60
 
