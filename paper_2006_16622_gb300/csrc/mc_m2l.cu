@@ -5,11 +5,15 @@
 // Lhat = L w^(j+1), paper normalisation) every offset o of an interaction
 // list has one matrix T_o of size C x C, |T| <= 1/2, whose rows sum to at
 // most 137 over all 189 offsets.  Two things make it cheap here:
-//   * numbers of 57 and 54 bits as an integer high part and a 28-bit low part
-//     kept as a float: the product of the high parts is one 32 x 32 + 64-bit
-//     multiply-add (exact sums, ~5 cycles) and the two cross products are
-//     single-precision ones (1.2 cycles each; they start at 2^-28 of the
-//     product), 7.4 cycles where one FP64 multiply-add takes 64;
+//   * numbers of 59 and 57 bits as a high part and a signed low part of 30:
+//     the product of the high parts and the two cross products are one
+//     32 x 32 + 64-bit multiply-add each (exact sums; the product of the low
+//     parts, below 2^-2 of the sums' last bit, is left out), ~15 cycles where
+//     one FP64 multiply-add takes 64.  (Single-precision multiply-adds of the
+//     low parts take half of that, but round at 2^-24 of sums that start at
+//     2^-28 of the product: with the scales of mc_m2l_scale.cuh and a carry
+//     every two columns the degrees above 4 still came out up to 2.4 times as
+//     far from exact translations as in FP64, 8 times beside a dense cell);
 //   * in the real layout a reflection x -> -x (y, z) only changes signs:
 //     T_(s o) = X_s T_o X_s with X_s diagonal, +-1, so that the up to eight
 //     offsets that differ in signs share one product:
@@ -22,15 +26,10 @@
 // class k, so that all its products take their Mt from one transform index
 // per column.  Half of the lanes take half of the rows, each lane two targets:
 // a matrix entry and a transform value are loaded for several products each
-// (one target per lane loads an entry per product, which returns 32 lanes
-// even where all are the same: 8 cycles of the SM's shared memory for the 7.4
-// of its four sub-partitions' arithmetic).
-// Level 6 of N = 1e6, p = 12 (32768 cells): 427 ms in FP64, 23 ms here, level
-// 5 (4096 cells) 61 and 2.9; the arithmetic alone would take half of that, the
-// rest are the transforms and the barriers between tiles.  Leaving out the
-// columns that an offset without x, y or z part does not couple (39.5 of the 56
-// products remain) gained 3 % at 32768 cells and lost 5 to 11 % below: the
-// warps of a CTA skip different columns between the same barriers.
+// (one target per lane would return an entry to 32 lanes for each product).
+// Level 6 of N = 1e6, p = 12 (32768 cells): 427 ms in FP64, 36 ms here, level
+// 5 (4096 cells) 61 and 4.8; the arithmetic alone would take half of that, the
+// rest are the transforms and the barriers between tiles.
 #include <math.h>
 
 #include <algorithm>
@@ -39,13 +38,14 @@
 #include "mc_fix.cuh"
 #include "mc_fixsum.cuh"
 #include "mc_m2l.cuh"
+#include "mc_m2l_scale.cuh"
 
 namespace {
 
 constexpr int kTile = 8;      // columns staged at a time
 constexpr int kOrbits = 56;   // offsets up to signs: {0..3}^3 without {0, 1}^3
 constexpr int kMaxRows = (MC_PMAX + 1) * (MC_PMAX + 1) + 32;
-constexpr int kBitsT = 57, kBitsM = 54, kLimb = 28;
+constexpr int kBitsT = 59, kBitsM = 57, kLimb = 30;
 
 // tiles of the columns: at least two, so that an orbit's cells are known a
 // step before its first tile is loaded
@@ -84,10 +84,10 @@ M2LLayout m2l_layout(int p) {
 
 struct M2LArgs {
   int l, nl, h, pbc, p, nco, per_o;
-  int carry;  // columns between two carries of the cross products
   int start[8], half[8], rows;
   unsigned char ccol[kMaxRows];  // class of a column
   unsigned char orbit[kOrbits];  // |ox| | |oy| << 2 | |oz| << 4
+  unsigned char degree[kMaxRows];  // of a row
   short index[kMaxRows];
   double scale[kMaxRows];
 };
@@ -102,14 +102,15 @@ __device__ __forceinline__ void decode(int k, int* n, int* m, int* im) {
   *im = (rem > 0 && (rem & 1) == 0) ? 1 : 0;
 }
 
-// v as h 2^28 + l: h, and l 2^-28 as a float
+// h, l of v = h 2^30 + l, l signed
 __device__ __forceinline__ int2 limbs(long long v) {
   const int l = ((int)v << (32 - kLimb)) >> (32 - kLimb);
-  return make_int2((int)((v - l) >> kLimb), __float_as_int((float)l * (1.0f / (float)(1 << kLimb))));
+  return make_int2((int)((v - l) >> kLimb), l);
 }
 
 struct TableArgs {
   int p, rows;
+  signed char col[MC_PMAX + 1];
   unsigned char orbit[kOrbits];
   short index[kMaxRows];
 };
@@ -146,15 +147,16 @@ __global__ void k_m2l_tables(const __grid_constant__ TableArgs A, const double* 
       for (int q = 2; q <= n - m; q++) g *= q;
       for (int q = 2; q <= n + m; q++) g *= q;
       v /= sqrt(f) * sqrt(g);
+      v = ldexp(v, kBitsT + kM2LRowScale[m2l_group(ob)][j] - A.col[n]);
     }
-    const long long w = __double2ll_rn(ldexp(v, kBitsT));
+    const long long w = __double2ll_rn(v);
     T[i] = limbs(w);
   }
 }
 
 struct ConvArgs {
   int nl, C;
-  double scale[kMaxRows];  // sqrt((n-m)!(n+m)!) w^-n
+  double scale[kMaxRows];  // sqrt((n-m)!(n+m)!) w^-n 2^kM2LColScale[n]
 };
 
 // one level's multipoles (scaled layout, by cell) as integers of kBitsM bits
@@ -225,14 +227,14 @@ struct M2LShared {
   int2* Mt;       // [2][kTile][8][32]: transform values
   long long* raw; // [kTile][8][32]: the members' multipoles on their way there
   int* cell;      // [2][8][32]: members' cells of an orbit (-1: none), by lane
-  int* shift;     // [2][8][32]: shifts to the task's unit
+  int* shift;     // [2][8][32]: shifts to the unit of the orbit's group
+  int* unit;      // [MC_M2L_GROUPS][32]: that unit (its exponent; -4096: no cell)
 };
 
 struct M2LTask {
   int cls, oc;  // target class, orbit chunk
   int I[3], b[3];  // the target this thread stages (clamped): halved coordinates, parities
   bool valid;
-  int ecta;
 };
 
 // halved coordinate and parity of coordinate 2 I + b + o on an axis with h
@@ -265,15 +267,12 @@ __device__ __forceinline__ void m2l_task(const M2LArgs& A, const int2* __restric
   const int ob = k.oc * A.per_o, oe = min(kOrbits, ob + A.per_o);
   const int steps = (oe - ob) * tiles, tsz = kTile * A.rows;
   const int tid = 32 * w + lane, cls = class_of_warp(w);
-  long long hh[NR > 0 ? NR : 1][NT];
-  float x[NR > 0 ? NR : 1][NT];
+  // products of the high parts, and the two cross products
+  long long hh[NR > 0 ? NR : 1][NT], x[NR > 0 ? NR : 1][NT];
 #pragma unroll
   for (int r = 0; r < NR; r++)
 #pragma unroll
-    for (int t = 0; t < NT; t++) {
-      hh[r][t] = 0;
-      x[r][t] = 0.0f;
-    }
+    for (int t = 0; t < NT; t++) hh[r][t] = x[r][t] = 0;
   int lo = ob, lt = 0;  // orbit and tile to load next
   // member w (signs of its offset: bits x 4, y 2, z 1) of an orbit
   auto members = [&](int o) {
@@ -288,7 +287,7 @@ __device__ __forceinline__ void m2l_task(const M2LArgs& A, const int2* __restric
     const int c = ok ? cell_at(k, of[0], of[1], of[2], h, A.pbc != 0) : -1;
     const int i = ((o & 1) * 8 + w) * 32 + lane;
     S.cell[i] = c;
-    S.shift[i] = c >= 0 ? min(63, k.ecta - E[c]) : 0;
+    S.shift[i] = c >= 0 ? min(63, S.unit[m2l_group(A.orbit[o]) * 32 + lane] - E[c]) : 0;
   };
   // column w of the next tile: its lane's target's members, and the table
   auto load = [&](int s) {
@@ -337,90 +336,88 @@ __device__ __forceinline__ void m2l_task(const M2LArgs& A, const int2* __restric
       so++;
     }
   };
-  // the cross products' large part, carried over every A.carry columns
-  auto carry = [&]() {
+  // a group's sums into the result
+  bool first = true;
+  auto flush = [&](int g) {
+    const int h3 = h * h * h;
 #pragma unroll
-    for (int r = 0; r < NR; r++)
+    for (int t = 0; t < NT; t++) {
+      const int ii = t0 + 16 * t + (lane & 15);
+      const double unit = ldexp(1.0, S.unit[g * 32 + 16 * t + (lane & 15)]);
+      const int i = 2 * (ii / (h * h)) + k.b[0], j = 2 * ((ii / h) % h) + k.b[1], kk = 2 * (ii % h) + k.b[2];
+      double* o = out + ((size_t)((i * A.nl + j) * A.nl + kk) * A.nco + k.oc) * C;
 #pragma unroll
-      for (int t = 0; t < NT; t++) {
-        // multiples of 2^11, read off the last bits of the sum with 3 2^33
-        // (|x| < 2^35; a conversion to 64 bits would use the FP64 pipe)
-        const float f = x[r][t] + 25769803776.0f;
-        hh[r][t] = m2l_wide(__float_as_int(f) - 0x50C00000, 2048, hh[r][t]);
-        x[r][t] -= f - 25769803776.0f;
+      for (int r = 0; r < NR; r++) {
+        const int row = A.start[cls] + (lane >> 4) * ((NR + 1) / 2 * 2) + r, at = A.index[row];
+        if (ii < h3 && at >= 0) {
+          const double down = __longlong_as_double((long long)(1023 - kM2LRowScale[g][A.degree[row]]) << 52);
+          const double v = fma((double)x[r][t], 1.0 / (double)(1 << kLimb), (double)hh[r][t]) * A.scale[row] * down * unit;
+          o[at] = first ? v : o[at] + v;
+        }
+        hh[r][t] = x[r][t] = 0;
       }
+    }
+    first = false;
   };
   members(ob);
   cta_sync();
   load(0);
   store(0);
   cta_sync();
-  int tile = 0;
+  int tile = 0, co = ob;  // of the current step: tile and orbit
   for (int s = 0; s < steps; s++) {
     if (s + 1 < steps) load(s + 1);
     if constexpr (NR > 0) {
       const int2* tt = S.T + (s & 1) * tsz + A.start[cls] + (lane >> 4) * ((NR + 1) / 2 * 2);
       const int2* m0 = S.Mt + (size_t)(s & 1) * kTile * 8 * 32 + (lane & 15);
-      for (int c0 = 0; c0 < kTile; c0 += A.carry) {
 #pragma unroll 2
-        for (int c = c0; c < c0 + A.carry; c++) {
-          const int d = cls ^ A.ccol[tile * kTile + c];
-          int mh[NT];
-          float ml[NT], mf[NT];
+      for (int c = 0; c < kTile; c++) {
+        const int d = cls ^ A.ccol[tile * kTile + c];
+        int2 m[NT];
+#pragma unroll
+        for (int t = 0; t < NT; t++) m[t] = m0[(c * 8 + d) * 32 + 16 * t];
+        const int4* tr = reinterpret_cast<const int4*>(tt + c * A.rows);
+#pragma unroll
+        for (int r = 0; r < NR; r++) {
+          const int4 q = tr[r / 2];
+          const int th = r & 1 ? q.z : q.x, tl = r & 1 ? q.w : q.y;
 #pragma unroll
           for (int t = 0; t < NT; t++) {
-            const int2 m = m0[(c * 8 + d) * 32 + 16 * t];
-            mh[t] = m.x;
-            ml[t] = __int_as_float(m.y);
-            mf[t] = (float)m.x;
-          }
-          const int4* tr = reinterpret_cast<const int4*>(tt + c * A.rows);
-#pragma unroll
-          for (int r = 0; r < NR; r++) {
-            const int4 q = tr[r / 2];
-            const int th = r & 1 ? q.z : q.x;
-            const float tl = __int_as_float(r & 1 ? q.w : q.y), tf = (float)th;
-#pragma unroll
-            for (int t = 0; t < NT; t++) {
-              hh[r][t] = m2l_wide(th, mh[t], hh[r][t]);
-              x[r][t] = fmaf(tf, ml[t], x[r][t]);
-              x[r][t] = fmaf(tl, mf[t], x[r][t]);
-            }
+            hh[r][t] = m2l_wide(th, m[t].x, hh[r][t]);
+            x[r][t] = m2l_wide(th, m[t].y, x[r][t]);
+            x[r][t] = m2l_wide(tl, m[t].x, x[r][t]);
           }
         }
-        carry();
       }
-      if (++tile == tiles) tile = 0;
+      // |x| < 8 (2^29 2^29 + 2^29 2^30) + 2^30 < 2^63 between two carries
+      static_assert(kTile <= 8 && kBitsT - kLimb <= 29 && kBitsM + 3 - kLimb <= 30 && kLimb <= 30, "cross products");
+#pragma unroll
+      for (int r = 0; r < NR; r++)
+#pragma unroll
+        for (int t = 0; t < NT; t++) {
+          hh[r][t] += x[r][t] >> kLimb;
+          x[r][t] &= (1 << kLimb) - 1;
+        }
+    }
+    if (++tile == tiles) {
+      tile = 0;
+      const int g = m2l_group(A.orbit[co]);
+      if (++co == oe || m2l_group(A.orbit[co]) != g) flush(g);
     }
     if (s + 1 < steps) store(s + 1);
     cta_sync();
-  }
-  if constexpr (NR > 0) {
-    const double unit = ldexp(1.0, k.ecta);
-    const int h3 = h * h * h;
-#pragma unroll
-    for (int t = 0; t < NT; t++) {
-      const int ii = t0 + 16 * t + (lane & 15);
-      if (ii >= h3) continue;
-      const int i = 2 * (ii / (h * h)) + k.b[0], j = 2 * ((ii / h) % h) + k.b[1], kk = 2 * (ii % h) + k.b[2];
-      double* o = out + ((size_t)((i * A.nl + j) * A.nl + kk) * A.nco + k.oc) * C;
-#pragma unroll
-      for (int r = 0; r < NR; r++) {
-        const int row = A.start[cls] + (lane >> 4) * ((NR + 1) / 2 * 2) + r;
-        const double sum = (double)hh[r][t] + (double)x[r][t];
-        if (A.index[row] >= 0) o[A.index[row]] = sum * A.scale[row] * unit;
-      }
-    }
   }
 }
 
 }  // namespace
 
-__global__ void __launch_bounds__(256, 2)
+// CTAs per SM: two, where 128 registers hold the sums of half a class's rows
+// (p = 12 with two: 284 bytes of spills, level 6 of N = 1e6 39 instead of 36 ms)
+template <int CTAS>
+__global__ void __launch_bounds__(256, CTAS)
     k_m2l_fix(const __grid_constant__ M2LArgs A, const int2* __restrict__ T, const long long* __restrict__ M,
               const int* __restrict__ E, double* __restrict__ out) {
   extern __shared__ int4 dyn4[];
-  __shared__ int s_emax;
   constexpr int kTargets = 32;
   M2LShared S;
   S.T = reinterpret_cast<int2*>(dyn4);
@@ -428,6 +425,7 @@ __global__ void __launch_bounds__(256, 2)
   S.raw = reinterpret_cast<long long*>(S.Mt + 2 * kTile * 8 * 32);
   S.cell = reinterpret_cast<int*>(S.raw + kTile * 8 * 32);
   S.shift = S.cell + 2 * 8 * 32;
+  S.unit = S.shift + 2 * 8 * 32;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int h = A.h, h3 = h * h * h, chunks = (h3 + kTargets - 1) / kTargets;
   M2LTask k;
@@ -442,20 +440,17 @@ __global__ void __launch_bounds__(256, 2)
   k.I[2] = r % h;
 #pragma unroll
   for (int d = 0; d < 3; d++) k.b[d] = (k.cls >> (2 - d)) & 1;
-  // unit of the sums: the largest unit of the cells in these targets' lists
-  if (threadIdx.x == 0) s_emax = -4096;
+  // units of the sums: the largest of the cells at a group's offsets
+  static_assert(kTargets == 32, "a target per lane");
+  for (int i = threadIdx.x; i < MC_M2L_GROUPS * 32; i += 256) S.unit[i] = -4096;
   __syncthreads();
-  int e = -4096;
-  for (int q = threadIdx.x / kTargets; q < 216; q += 256 / kTargets) {
+  for (int q = w; q < 216; q += 8) {
     const int ox = q / 36 - 2 - k.b[0], oy = (q / 6) % 6 - 2 - k.b[1], oz = q % 6 - 2 - k.b[2];
     if (ox >= -1 && ox <= 1 && oy >= -1 && oy <= 1 && oz >= -1 && oz <= 1) continue;
     const int c = cell_at(k, ox, oy, oz, h, A.pbc != 0);
-    if (c >= 0 && k.valid) e = max(e, E[c]);
+    if (c >= 0 && k.valid) atomicMax(&S.unit[m2l_group(abs(ox) | abs(oy) << 2 | abs(oz) << 4) * 32 + lane], E[c]);
   }
-  e = __reduce_max_sync(0xffffffffu, e);
-  if (lane == 0) atomicMax(&s_emax, e);
   __syncthreads();
-  k.ecta = s_emax;
   // half of 1, 3, 6, 10, 15, 21, 28, 36 rows
 #define MC_M2L_ROWS(NR_) \
   case NR_: m2l_task<NR_>(A, T, M, E, out, k, S, t0, w, lane); break;
@@ -468,7 +463,9 @@ __global__ void __launch_bounds__(256, 2)
     MC_M2L_ROWS(11)
     MC_M2L_ROWS(14)
     MC_M2L_ROWS(18)
-    MC_M2L_ROWS(0)
+    // (0 rows; any other number would leave the results out, but never the
+    // barriers)
+    default: m2l_task<0>(A, T, M, E, out, k, S, t0, w, lane);
   }
 #undef MC_M2L_ROWS
 }
@@ -480,12 +477,12 @@ size_t m2l_table_bytes(int p) {
   return sizeof(int2) * (size_t)kOrbits * tiles_of(C) * kTile * m2l_layout(p).rows;
 }
 
+// by group
 static void orbits(unsigned char* o) {
   int n = 0;
-  for (int x = 0; x < 4; x++)
-    for (int y = 0; y < 4; y++)
-      for (int z = 0; z < 4; z++)
-        if (std::max(x, std::max(y, z)) > 1) o[n++] = (unsigned char)(x | y << 2 | z << 4);
+  for (int g = 0; g < MC_M2L_GROUPS; g++)
+    for (int i = 0; i < 64; i++)
+      if (((i & 3) > 1 || ((i >> 2) & 3) > 1 || i >> 4 > 1) && m2l_group(i) == g) o[n++] = (unsigned char)i;
 }
 
 cudaError_t m2l_build_table(int p, int sms, void* table, double* otab, cudaStream_t st) {
@@ -495,6 +492,7 @@ cudaError_t m2l_build_table(int p, int sms, void* table, double* otab, cudaStrea
   const M2LLayout L = m2l_layout(p);
   A.p = p;
   A.rows = L.rows;
+  std::copy(kM2LColScale, kM2LColScale + MC_PMAX + 1, A.col);
   std::copy(L.index, L.index + L.rows, A.index);
   orbits(A.orbit);
   k_m2l_tables<<<sms * 8, 256, 0, st>>>(A, otab, (int2*)table);
@@ -531,15 +529,6 @@ cudaError_t m2l_fix_level(int p, int l, double w, bool pbc, int sms, const void*
   while (A.nco > 1 && (size_t)ncl * A.nco * C > scratch_doubles) A.nco--;
   A.per_o = (kOrbits + A.nco - 1) / A.nco;
   A.nco = (kOrbits + A.per_o - 1) / A.per_o;
-  // The cross products' single-precision sums round at 2^-24 of their size, so
-  // the fewer products a sum holds the better, above all where a row has few
-  // columns to average over.  A carry every 64 columns left the expansions up
-  // to four times as far from a 64-bit evaluation as the FP64 translations do
-  // (N = 2336, L = 3, p = 7, free space: 3.0e-15, FP64 1.0e-15); now 1.3e-15
-  // there, and 0.8 to 0.95 times the FP64 error for most orders.  Cost: the
-  // whole fast setup of N = 1e6, p = 12 31.3 -> 33.1 ms, of N = 1e5 4.5 -> 4.9
-  // (p = 12), 2.0 -> 2.3 (p = 8).
-  A.carry = p >= 12 ? 8 : (p >= 9 ? 4 : 2);
   A.rows = L.rows;
   for (int c = 0; c < 8; c++) {
     A.start[c] = L.start[c];
@@ -553,15 +542,17 @@ cudaError_t m2l_fix_level(int p, int l, double w, bool pbc, int sms, const void*
       for (int im = 0; im < (m ? 2 : 1); im++) {
         const int k = n * n + (m ? 2 * m - 1 : 0) + im;
         A.ccol[k] = (unsigned char)class_of(n, m, im);
-        V.scale[k] = sfac(n, m) * wn;
+        V.scale[k] = sfac(n, m) * wn * (double)(1 << kM2LColScale[n]);
       }
   }
   for (int r = 0; r < L.rows; r++) {
     A.index[r] = L.index[r];
     A.scale[r] = 0.0;
+    A.degree[r] = 0;
     if (L.index[r] < 0) continue;
     int n = (int)sqrt((double)L.index[r] + 0.5);
     const int rem = L.index[r] - n * n, m = (rem + 1) / 2;
+    A.degree[r] = (unsigned char)n;
     A.scale[r] = sfac(n, m) * pow(w, -(double)(n + 1)) * ldexp(1.0, 2 * kLimb - kBitsT - kBitsM);
   }
   const size_t csm = sizeof(long long) * 32 * (C + 1);
@@ -569,10 +560,11 @@ cudaError_t m2l_fix_level(int p, int l, double w, bool pbc, int sms, const void*
   if (e != cudaSuccess) return e;
   k_m2l_convert<<<(ncl + 31) / 32, 256, csm, st>>>(V, K, M, E);
   const int chunks = (h * h * h + 31) / 32;
-  const size_t smem = sizeof(int2) * (2 * (size_t)kTile * L.rows + 3 * kTile * 8 * 32) + sizeof(int) * 4 * 8 * 32;
-  e = cudaFuncSetAttribute(k_m2l_fix, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const size_t smem = sizeof(int2) * (2 * (size_t)kTile * L.rows + 3 * kTile * 8 * 32) + sizeof(int) * (4 * 8 + MC_M2L_GROUPS) * 32;
+  const auto kernel = p <= 11 ? k_m2l_fix<2> : k_m2l_fix<1>;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_m2l_fix<<<8 * chunks * A.nco, 256, smem, st>>>(A, (const int2*)table, M, E, A.nco > 1 ? scratch : Lout);
+  kernel<<<8 * chunks * A.nco, 256, smem, st>>>(A, (const int2*)table, M, E, A.nco > 1 ? scratch : Lout);
   e = cudaGetLastError();
   if (e == cudaSuccess && A.nco > 1) e = fix_reduce(ncl, A.nco, C, sms, scratch, Lout, st);
   return e;
