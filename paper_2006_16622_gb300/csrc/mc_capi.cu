@@ -416,24 +416,24 @@ int energy_chunks(const McSys& h, int sms, int l, bool irregular) {
 int energy_into(mc_ctx* c, double* d_dst, bool mpole) {
   const McSys& h = c->h;
   if (c->fixed && !h.lj_on) {
-    const int nb = fix_near_blocks(h.L, c->sms, h.cap), nnear = 8 * nb;
-    CK(fix_near(h.L, h.bc == MC_BC_PBC, h.a, fix_source(h), nb, c->d_scratch, c->stream));
+    const int nnear = fix_near_blocks(h.L, c->sms, h.cap);  // pairs of doubles
+    CK(fix_near(h.L, h.bc == MC_BC_PBC, h.a, fix_source(h), nnear, c->d_scratch, c->stream));
     int nexp = 0;
     if (h.method == 0 && mpole && c->d_mpole) {
       nexp = 2 * c->sms;
       k_energy_dot<<<nexp, 256, 0, c->stream>>>((size_t)h.ncell_total * h.C, h.C, c->d_mpole, h.Lhat,
-                                                c->d_scratch + nnear);
+                                                c->d_scratch + 2 * nnear);
       CK(cudaGetLastError());
     } else {
       for (int l = h.lmin; l <= h.L; l++) {
         FixPass ps = fix_pass(c, l, h.method == 1);
         ps.nchunk = energy_chunks(h, c->sms, l, h.method == 1);
         ps.dot = (h.method == 1 ? h.Mhat : h.Lhat) + (size_t)h.lev_off[l] * h.C;
-        CK(fix_launch(ps, fix_source(h), c->d_scratch + nnear + nexp, c->stream));
+        CK(fix_launch(ps, fix_source(h), c->d_scratch + 2 * nnear + nexp, c->stream));
         nexp += (1 << (3 * (l - 1))) * ps.nchunk;
       }
     }
-    k_energy_sum<<<1, 1024, 0, c->stream>>>(c->d_sys, nnear, nexp, c->d_scratch, d_dst);
+    k_energy_sum<<<1, 256, 0, c->stream>>>(c->d_sys, nnear, nexp, c->d_scratch, d_dst);
     CK(cudaGetLastError());
     return MC_OK;
   }
@@ -737,7 +737,7 @@ int mc_init(mc_ctx** out, int64_t n, const double* pos, const double* q, double 
   need = std::max(need, (size_t)c->sms * 2 * MC_WARPS);
   if (c->fixed) {
     // the energy's partials: near pairs, then the expansions of every level
-    const size_t nnear = 8 * (size_t)fix_near_blocks(levels, c->sms, cap);
+    const size_t nnear = 2 * (size_t)fix_near_blocks(levels, c->sms, cap);
     need = std::max(need, nnear + fix_near_work(levels, cap));
     size_t e = nnear + 2 * (size_t)c->sms;
     for (int l = h.lmin; l <= levels; l++)

@@ -272,6 +272,20 @@ __device__ __forceinline__ float warp_sum(float v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
+// hi + lo + x, the rounding of the first sum kept in lo (Knuth's two-sum)
+__device__ __forceinline__ void two_add(double* hi, double* lo, double x) {
+  const double s = *hi + x, b = s - *hi;
+  *lo += (*hi - (s - b)) + (x - b);
+  *hi = s;
+}
+__device__ __forceinline__ void warp_two_sum(double* hi, double* lo) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double h = __shfl_xor_sync(0xffffffffu, *hi, o), l = __shfl_xor_sync(0xffffffffu, *lo, o);
+    two_add(hi, lo, h);
+    *lo += l;
+  }
+}
 template <typename T>
 __device__ __forceinline__ T half_sum(T v) {
 #pragma unroll

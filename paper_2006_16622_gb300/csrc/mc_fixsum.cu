@@ -322,12 +322,13 @@ __global__ void __launch_bounds__(256)
 // neighbour's charges staged in shared memory and read by all lanes (or, where
 // few of the tile's charges are left, by the group of lanes whose turn they
 // are: 4.00 -> 3.20 ms for 1e6 charges, 30.5 a cell, and 121 -> 70 us for 3e4,
-// 7.3 a cell).  The first tiles of all (cell, neighbour) come first; where
+// 7.3 a cell; 3.6 ms and 85 us with the roundings of the sums kept).  The first
+// tiles of all (cell, neighbour) come first; where
 // cells may hold more than a tile, the others are counted by k_near_extra and
 // dealt out in order (4000 of 8000 charges in one cell, L = 5, whole fresh
 // energy: 79 ms with one warp for a (cell, neighbour), 0.93 now, 1.0 with the
 // FP64 kernel's warp per charge; 8 x 4000: 183, 5.7 and 37 ms).  At
-// 30.5 a cell 310 cycles of a sub-partition for 32 pairs, idle lanes included;
+// 30.5 a cell 340 cycles of a sub-partition for 32 pairs, idle lanes included;
 // the FP64 multiply-add takes 64 beside the integer ones.  Differences are exact
 // 64-bit integers; 1/r comes from a single-precision estimate and one
 // third-order step in integers on the difference shifted up to full length,
@@ -499,7 +500,7 @@ __global__ void __launch_bounds__(256, 4)
   const int nL = 1 << (A.L - 1), cap = A.src.cap;
   const long long tasks = 14LL * nL * nL * nL;
   const double4* rows = reinterpret_cast<const double4*>(A.src.rows);
-  double total = 0.0;
+  double total = 0.0, low = 0.0;  // the sum and its rounding
   for (long long task = (long long)blockIdx.x * 8 + warp;; task += (long long)gridDim.x * 8) {
     int cell = (int)(task / 14), o = (int)(task % 14), ti = 0, tj = 0;  // o = 0: the cell itself
     long long tile = 0;
@@ -539,7 +540,13 @@ __global__ void __launch_bounds__(256, 4)
         }
         __syncwarp();
         const int jn = min(32, nj - j0);
-        for (int j = lane >> sh; j < jn; j += 32 >> sh) {
+        // eight pairs at a time, so that the running sum rounds at an eighth of
+        // the additions: a pair counts once here, in the FP64 kernel from both
+        // sides, which averages the rounding of two sums.  Energies of 2000
+        // charges at L = 3: 9.0e-14 (rms) off with one running sum and plain sums
+        // after it, 4.1e-14 now, FP64 5.4e-14
+        double part = 0.0;
+        for (int j = lane >> sh, u = 1; j < jn; j += 32 >> sh, u++) {
           const int64_t* x = s_x[warp][j];
           if (i >= ni || (o == 0 && j0 + j >= i)) continue;
           int64_t d[3];
@@ -548,17 +555,35 @@ __global__ void __launch_bounds__(256, 4)
           int k;
           const double rinv = near_rinv(d[0], d[1], d[2], &k);
           close |= k >= kNearClose;
-          acc += k >= kNearClose ? 0.0 : __longlong_as_double(x[3]) * rinv;
+          part += k >= kNearClose ? 0.0 : __longlong_as_double(x[3]) * rinv;
+          if ((u & 7) == 0) {
+            acc += part;
+            part = 0.0;
+          }
         }
+        acc += part;
       }
-      total += qi * acc;
+      two_add(&total, &low, qi * acc);
     }
     if (__any_sync(0xffffffffu, close))
-      total += near_close_pairs(A, &rows[(size_t)cell * cap], ib, ni, &rows[(size_t)other * cap], jb, nj,
-                                (im[0] + 1) | (im[1] + 1) << 2 | (im[2] + 1) << 4);
+      two_add(&total, &low, near_close_pairs(A, &rows[(size_t)cell * cap], ib, ni, &rows[(size_t)other * cap], jb, nj,
+                                             (im[0] + 1) | (im[1] + 1) << 2 | (im[2] + 1) << 4));
   }
-  total = warp_sum(total);
-  if (lane == 0) out[(size_t)blockIdx.x * 8 + warp] = total * A.unit;
+  warp_two_sum(&total, &low);
+  __shared__ double s_sum[8][2];
+  if (lane == 0) {
+    s_sum[warp][0] = total;
+    s_sum[warp][1] = low;
+  }
+  __syncthreads();
+  if (warp > 0) return;
+  total = lane < 8 ? s_sum[lane][0] : 0.0;
+  low = lane < 8 ? s_sum[lane][1] : 0.0;
+  warp_two_sum(&total, &low);
+  if (lane == 0) {
+    out[2 * blockIdx.x] = total;
+    out[2 * blockIdx.x + 1] = low;
+  }
 }
 
 int fix_near_blocks(int L, int sms, int cap) {
@@ -600,7 +625,7 @@ cudaError_t fix_near(int L, bool pbc, double a, const FixSource& src, int blocks
   A.cells = A.blocks = nullptr;
   if (fix_near_work(L, src.cap)) {
     const int ncell = 1 << (3 * (L - 1)), nb = (ncell + kNearBlock - 1) / kNearBlock;
-    long long* cells = reinterpret_cast<long long*>(out + 8 * (size_t)blocks);
+    long long* cells = reinterpret_cast<long long*>(out + 2 * (size_t)blocks);
     k_near_extra<<<nb, kNearBlock, 0, st>>>(A, cells, cells + ncell);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;

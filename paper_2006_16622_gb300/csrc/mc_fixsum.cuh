@@ -35,8 +35,8 @@ struct FixPass {
 int fix_chunks(int L, int l, bool irregular, int sms, double occupancy, int p);
 cudaError_t fix_launch(const FixPass& ps, const FixSource& src, double* out, cudaStream_t st);
 // Direct part of the energy: 1/r over the pairs of charges within near cells
-// (every pair and image once), one partial per warp of the returned number
-// of blocks of 256 threads, followed by the workspace of fix_near_work doubles
+// (every pair and image once) in units of 1 / (four finest cells), one partial
+// (a sum and its rounding) for each of the returned number of blocks, followed by the workspace of fix_near_work doubles
 // (of use until the call's kernels are done)
 int fix_near_blocks(int L, int sms, int cap);
 size_t fix_near_work(int L, int cap);

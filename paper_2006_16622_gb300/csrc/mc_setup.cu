@@ -430,32 +430,55 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// U from the partials of the near pairs and (twice) of the expansions, and the
-// periodic terms
-__global__ void __launch_bounds__(1024)
+// U from the partials of the near pairs (nnear times a sum and its rounding, in
+// units of 1 / (four finest cells)) and (twice) of the expansions, and the
+// periodic terms.  Sums keep their rounding: near pairs and expansions cancel to
+// a fraction of either.
+__global__ void __launch_bounds__(256)
     k_energy_sum(const McSys* __restrict__ sysp, int nnear, int nexp, const double* __restrict__ in,
                  double* __restrict__ dst) {
   const McSys& S = *sysp;
-  __shared__ double red[32];
+  __shared__ double red[8][2];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double s = 0.0;
-  for (int i = threadIdx.x; i < nnear; i += 1024) s += in[i];
-  for (int i = threadIdx.x; i < nexp; i += 1024) s += 0.5 * in[nnear + i];
+  double s = 0.0, e = 0.0;
+  for (int i = threadIdx.x; i < nnear; i += 256) {
+    two_add(&s, &e, in[2 * i]);
+    e += in[2 * i + 1];
+  }
+  {
+    // times 1 / (4 w), w = a / nL
+    const double x = s * (0.25 * S.nL), r = x / S.a;
+    e = (fma(-r, S.a, x) + e * (0.25 * S.nL)) / S.a;
+    s = r;
+  }
+  {
+    // (many and small)
+    double x = 0.0;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < nexp; i += 256) x += in[2 * nnear + i];
+    two_add(&s, &e, 0.5 * x);
+  }
   if (S.bc == 0)
-    for (int k = threadIdx.x; k < S.C; k += 1024) {
+    for (int k = threadIdx.x; k < S.C; k += 256) {
       const int r = (int)sqrtf((float)k + 0.5f);
-      s += (r * r == k ? 0.5 : 1.0) * (S.Khat[k] * S.Hhat[k]);
+      two_add(&s, &e, (r * r == k ? 0.5 : 1.0) * (S.Khat[k] * S.Hhat[k]));
     }
-  s = warp_sum(s);
-  if (lane == 0) red[warp] = s;
+  warp_two_sum(&s, &e);
+  if (lane == 0) {
+    red[warp][0] = s;
+    red[warp][1] = e;
+  }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < 32; w++) s += red[w];
+  if (warp > 0) return;
+  s = lane < 8 ? red[lane][0] : 0.0;
+  e = lane < 8 ? red[lane][1] : 0.0;
+  warp_two_sum(&s, &e);
+  if (lane == 0) {
     if (S.bc == 0 && S.dip == 0) {
       const double D2 = S.dipv[0] * S.dipv[0] + S.dipv[1] * S.dipv[1] + S.dipv[2] * S.dipv[2];
-      s += -2.0 * 3.141592653589793 / (3.0 * S.V) * D2;
+      two_add(&s, &e, -2.0 * 3.141592653589793 / (3.0 * S.V) * D2);
     }
-    dst[0] = s;
+    dst[0] = isfinite(s) ? s + e : s;  // (an infinite sum has no rounding)
   }
 }
 
