@@ -300,7 +300,7 @@ int mc_probe_fma_rate(int fp64, double target_seconds, double *flops_out);
  *   cuda_stream   stream to launch on (NULL = legacy stream); the call only
  *                 enqueues work and returns.
  * Intermediate sums live in one file-scope device array of
- * MC_NOALLOC_SCRATCH_DOUBLES doubles (and the range of the charges, three
+ * MC_NOALLOC_SCRATCH_DOUBLES doubles (and the range of the charges, four
  * integers, in a second one under the same rules).  A level whose 8^(level-1) (p+1)^2
  * coefficients exceed it is refused with MC_ERR_SCRATCH before any launch.
  * The first call on a device looks up the array's device address

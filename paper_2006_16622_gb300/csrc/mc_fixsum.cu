@@ -95,6 +95,7 @@ __global__ void __launch_bounds__(kThreads, fix_ctas(fix_shares(P).steps))
   __shared__ int s_cell[kRound], s_shift[kRound], s_pre[kRound + 1];
   extern __shared__ int64_t dyn[];
   if (A.src.range && !fix_usable(A.src.range)) return;
+  const int nchunk = A.src.range ? A.src.range[3] : A.nchunk;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   for (int i = tid; i < MC_FIX_WARPS * ST; i += nthr) s_step[i / ST][i % ST] = A.tab.step[i / ST][i % ST];
   const bool irr = A.irregular != 0, pbc = A.pbc != 0;
@@ -110,7 +111,8 @@ __global__ void __launch_bounds__(kThreads, fix_ctas(fix_shares(P).steps))
 #pragma unroll
   for (int d = 0; d < 3; d++) T[d] = (uint64_t)(2 * tc[d] + 1) << (62 - l);
   const long long units = (long long)(irr ? 189 : 1) << (3 * fb);
-  const long long per = (units + A.nchunk - 1) / A.nchunk;
+  if (ch >= nchunk) return;
+  const long long per = (units + nchunk - 1) / nchunk;
   const long long ub = (long long)ch * per, ue = ub + per < units ? ub + per : units;
   // steps where a column begins, from ballots so that the branch is uniform
   const unsigned turn_lo = __ballot_sync(0xffffffffu, (A.tab.turn[warp] >> lane) & 1ull);
@@ -656,10 +658,9 @@ int fix_chunks(int L, int l, bool irregular, int sms, double occupancy, int p) {
   const long long units = (irregular ? 189LL : 1LL) << (3 * (L - l));
   // about eight tasks per resident CTA ...
   const long long want = (8LL * fix_ctas(fix_shares(p).steps) * sms + ncl - 1) / ncl;
-  // ... of at least two staged batches of charges each
-  const double least = 2.0 * kThreads / std::max(occupancy, 0.25);
-  const long long most = std::max<long long>(1, (long long)((double)units / least));
-  return (int)std::max<long long>(1, std::min(std::min(want, most), units));
+  // ... that are worth it
+  static_assert(kThreads == 128, "fix_chunks_worth");
+  return (int)std::max<long long>(1, std::min(want, fix_chunks_worth(units, occupancy)));
 }
 
 cudaError_t fix_launch(const FixPass& ps, const FixSource& src, double* out, cudaStream_t st) {

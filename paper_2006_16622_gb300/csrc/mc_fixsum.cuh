@@ -13,7 +13,7 @@ struct FixSource {
   const int* start;
   // range of the charges found on the device (mc_noalloc.cu), or null:
   // {unusable, largest biased exponent e of a non-zero charge, largest
-  // 4096 - e}, all 0 without any
+  // 4096 - e}, all 0 without any, and the chunks in use
   const int* range;
 };
 
@@ -33,6 +33,14 @@ struct FixPass {
 // chunks per target that keep every SM busy without tasks too short to pay
 // for themselves (occupancy: mean charges of a finest cell)
 int fix_chunks(int L, int l, bool irregular, int sms, double occupancy, int p);
+// the part of it that needs the occupancy: chunks of `units` finest cells with
+// at least two staged batches of 128 charges each
+#ifdef __CUDACC__
+__host__ __device__ __forceinline__ long long fix_chunks_worth(long long units, double occupancy) {
+  const double n = (double)units / (256.0 / (occupancy > 0.25 ? occupancy : 0.25));
+  return n < 1.0 ? 1 : (n < (double)units ? (long long)n : units);
+}
+#endif
 cudaError_t fix_launch(const FixPass& ps, const FixSource& src, double* out, cudaStream_t st);
 // Direct part of the energy: 1/r over the pairs of charges within near cells
 // (every pair and image once) in units of 1 / (four finest cells), one partial

@@ -24,7 +24,7 @@
 static __device__ __align__(256) double g_noalloc_scratch[MC_NOALLOC_SCRATCH_DOUBLES];
 
 // what decides between the fixed-point sums and the FP64 ones (FixSource::range)
-static __device__ int g_noalloc_range[3];
+static __device__ int g_noalloc_range[4];
 
 namespace {
 
@@ -122,7 +122,11 @@ __global__ void __launch_bounds__(MC_THREADS)
 // cell, combined with atomic maxima.
 __global__ void __launch_bounds__(MC_THREADS)
     k_noalloc_range(int nL, double inv_w, const double* __restrict__ part, const int* __restrict__ cstart,
-                    int* __restrict__ range) {
+                    int nfix, long long units, int* __restrict__ range) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    const int ncell = nL * nL * nL;
+    range[3] = (int)min((long long)nfix, fix_chunks_worth(units, (double)(cstart[ncell] - cstart[0]) / (double)ncell));
+  }
   const int lane = threadIdx.x & 31;
   int bad = 0, emax = 0, emin = 0;
   for (int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < nL * nL * nL; c += (gridDim.x * blockDim.x) >> 5) {
@@ -162,14 +166,15 @@ __global__ void __launch_bounds__(MC_THREADS)
 __global__ void __launch_bounds__(MC_THREADS)
     k_reduce_noalloc(int nfix, int nfp64, int C, const int* __restrict__ range, const double* __restrict__ in,
                      double* __restrict__ out) {
-  const int nchunk = fix_usable(range) ? nfix : nfp64;
+  const bool fix = fix_usable(range);
+  const int nchunk = fix ? range[3] : nfp64, room = fix ? nfix : nfp64;
   __shared__ double part[MC_WARPS][32];
   const int nb = (C + 31) / 32, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const size_t t = blockIdx.x / nb;
   const int k = (blockIdx.x % nb) * 32 + lane;
   double s = 0.0;
   if (k < C)
-    for (int ch = warp; ch < nchunk; ch += MC_WARPS) s += in[(t * nchunk + ch) * C + k];
+    for (int ch = warp; ch < nchunk; ch += MC_WARPS) s += in[(t * room + ch) * C + k];
   part[warp][lane] = s;
   __syncthreads();
   if (warp == 0 && k < C) {
@@ -233,7 +238,10 @@ extern "C" int mc_p2l_level_noalloc(const double* d_part, const int* d_cell_star
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return MC_ERR_CUDA;
   const long long ncellL = 1LL << (3 * (levels - 1));
-  long long nfix = fix_chunks(levels, level, true, sms, (double)n / (double)ncellL, p);
+  // as many chunks as keep the SMs busy with full cells; how many are in use
+  // is for the charges in d_cell_start to say (n says nothing)
+  const long long units = 189LL << (3 * (levels - level));
+  long long nfix = fix_chunks(levels, level, true, sms, 256.0, p);
   // the FP64 gather's: a task is one warp, a list entry the smallest chunk
   long long nfp64 = std::min(189LL, (4LL * sms * MC_WARPS + ncl - 1) / ncl);
   const long long most = (long long)MC_NOALLOC_SCRATCH_DOUBLES / (ncl * C);  // at least 1
@@ -260,12 +268,12 @@ extern "C" int mc_p2l_level_noalloc(const double* d_part, const int* d_cell_star
   // charges that lie in their cells and span a few powers of two are summed
   // in fixed point (level 4 of N = 1e5, p = 12: 4.7 ms, in FP64 104); the FP64
   // gather does the others, and returns at once otherwise
-  if (cudaMemsetAsync(range, 0, 3 * sizeof(int), stream) != cudaSuccess) {
+  if (cudaMemsetAsync(range, 0, 4 * sizeof(int), stream) != cudaSuccess) {
     cudaGetLastError();
     return MC_ERR_CUDA;
   }
   const int rblocks = (int)((ncellL + MC_WARPS - 1) / MC_WARPS < 8LL * sms ? (ncellL + MC_WARPS - 1) / MC_WARPS : 8LL * sms);
-  k_noalloc_range<<<rblocks, MC_THREADS, 0, stream>>>(P.nL, (double)P.nL / box, d_part, d_cell_start, range);
+  k_noalloc_range<<<rblocks, MC_THREADS, 0, stream>>>(P.nL, (double)P.nL / box, d_part, d_cell_start, (int)nfix, units, range);
   // no error was pending before the launch, so one now is the launch's own
   if (cudaGetLastError() != cudaSuccess) return MC_ERR_CUDA;
   const FixPass ps{levels, level, p, true, bc == MC_BC_PBC, box, 0, (int)nfix, nullptr};
