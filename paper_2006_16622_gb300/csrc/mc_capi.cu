@@ -370,18 +370,20 @@ void m2l_table_release(mc_ctx* c) {
 int m2l_levels(mc_ctx* c) {
   McSys& h = c->h;
   const int C = h.C, p = h.p;
-  if (c->fixed) {
-    int rc = m2l_table_get(c);
-    if (rc != MC_OK) return rc;
-    if (!c->d_mfix && dalloc(c, (void**)&c->d_mfix, sizeof(long long) * (size_t)h.ncellL * C) != MC_OK)
-      return MC_ERR_NOMEM;
-    if (!c->d_mexp && dalloc(c, (void**)&c->d_mexp, sizeof(int) * (size_t)h.ncellL) != MC_OK) return MC_ERR_NOMEM;
+  // the fixed-point form needs the finest level's multipoles a second time:
+  // where they find no room, the FP64 form, which needs little, does the work
+  int rc = c->fixed ? m2l_table_get(c) : MC_ERR_NOMEM;
+  if (rc == MC_OK && !c->d_mexp) rc = dalloc(c, (void**)&c->d_mexp, sizeof(int) * (size_t)h.ncellL);
+  if (rc == MC_OK && !c->d_mfix) rc = dalloc(c, (void**)&c->d_mfix, sizeof(long long) * (size_t)h.ncellL * C);
+  if (rc == MC_OK) {
     for (int l = h.lmin; l <= h.L; l++)
       CK(m2l_fix_level(p, l, h.lev_w[l], h.bc == MC_BC_PBC, c->sms, c->m2l_table,
                        c->d_mpole + (size_t)h.lev_off[l] * C, c->d_mfix, c->d_mexp,
                        h.Lhat + (size_t)h.lev_off[l] * C, c->d_scratch, c->scratch_doubles, c->stream));
     return MC_OK;
   }
+  if (rc != MC_ERR_NOMEM) return rc;
+  m2l_table_release(c);
   const int per = (2 * p + 1) * (2 * p + 2) / 2;
   if (!c->d_otab) {
     if (dalloc(c, (void**)&c->d_otab, sizeof(double) * 2 * 343 * (size_t)per) != MC_OK)
