@@ -324,13 +324,12 @@ __global__ void __launch_bounds__(256)
 // neighbour's charges staged in shared memory and read by all lanes (or, where
 // few of the tile's charges are left, by the group of lanes whose turn they
 // are: 4.00 -> 3.20 ms for 1e6 charges, 30.5 a cell, and 121 -> 70 us for 3e4,
-// 7.3 a cell; 3.6 ms and 85 us with the roundings of the sums kept).  The first
-// tiles of all (cell, neighbour) come first; where
+// 7.3 a cell).  The first tiles of all (cell, neighbour) come first; where
 // cells may hold more than a tile, the others are counted by k_near_extra and
 // dealt out in order (4000 of 8000 charges in one cell, L = 5, whole fresh
 // energy: 79 ms with one warp for a (cell, neighbour), 0.93 now, 1.0 with the
 // FP64 kernel's warp per charge; 8 x 4000: 183, 5.7 and 37 ms).  At
-// 30.5 a cell 340 cycles of a sub-partition for 32 pairs, idle lanes included;
+// 30.5 a cell 310 cycles of a sub-partition for 32 pairs, idle lanes included;
 // the FP64 multiply-add takes 64 beside the integer ones.  Differences are exact
 // 64-bit integers; 1/r comes from a single-precision estimate and one
 // third-order step in integers on the difference shifted up to full length,
@@ -547,23 +546,24 @@ __global__ void __launch_bounds__(256, 4)
         // sides, which averages the rounding of two sums.  Energies of 2000
         // charges at L = 3: 9.0e-14 (rms) off with one running sum and plain sums
         // after it, 4.1e-14 now, FP64 5.4e-14
-        double part = 0.0;
-        for (int j = lane >> sh, u = 1; j < jn; j += 32 >> sh, u++) {
-          const int64_t* x = s_x[warp][j];
-          if (i >= ni || (o == 0 && j0 + j >= i)) continue;
-          int64_t d[3];
+        for (int j = lane >> sh; j < jn;) {
+          const int je = min(jn, j + (8 << (5 - sh)));
+          double part = 0.0;
+#pragma unroll 1
+          for (; j < je; j += 32 >> sh) {
+            const int64_t* x = s_x[warp][j];
+            if (i >= ni || (o == 0 && j0 + j >= i)) continue;
+            int64_t d[3];
 #pragma unroll
-          for (int a = 0; a < 3; a++) d[a] = near_diff(xi[a], x[a]);
-          int k;
-          const double rinv = near_rinv(d[0], d[1], d[2], &k);
-          close |= k >= kNearClose;
-          part += k >= kNearClose ? 0.0 : __longlong_as_double(x[3]) * rinv;
-          if ((u & 7) == 0) {
-            acc += part;
-            part = 0.0;
+            for (int a = 0; a < 3; a++) d[a] = near_diff(xi[a], x[a]);
+            int k;
+            const double rinv = near_rinv(d[0], d[1], d[2], &k);
+            close |= k >= kNearClose;
+            // (rinv is finite for any difference)
+            part = fma(k >= kNearClose ? 0.0 : __longlong_as_double(x[3]), rinv, part);
           }
+          acc += part;
         }
-        acc += part;
       }
       two_add(&total, &low, qi * acc);
     }
