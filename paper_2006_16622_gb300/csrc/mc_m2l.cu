@@ -27,9 +27,9 @@
 // per column.  Half of the lanes take half of the rows, each lane two targets:
 // a matrix entry and a transform value are loaded for several products each
 // (one target per lane would return an entry to 32 lanes for each product).
-// Level 6 of N = 1e6, p = 12 (32768 cells): 427 ms in FP64, 36 ms here, level
-// 5 (4096 cells) 61 and 4.8; the arithmetic alone would take half of that, the
-// rest are the transforms and the barriers between tiles.
+// Level 6 of N = 1e6, p = 12 (32768 cells): 427 ms in FP64, 31 ms here, level
+// 5 (4096 cells) 61 and 4.1; the multiply-adds alone would take 60 % of that,
+// the rest are the transforms and the barriers between tiles.
 #include <math.h>
 
 #include <algorithm>
@@ -42,14 +42,21 @@
 
 namespace {
 
-constexpr int kTile = 8;      // columns staged at a time
 constexpr int kOrbits = 56;   // offsets up to signs: {0..3}^3 without {0, 1}^3
 constexpr int kMaxRows = (MC_PMAX + 1) * (MC_PMAX + 1) + 32;
 constexpr int kBitsT = 59, kBitsM = 57, kLimb = 30;
 
-// tiles of the columns: at least two, so that an orbit's cells are known a
-// step before its first tile is loaded
-__host__ __device__ __forceinline__ int tiles_of(int C) { return C <= kTile ? 2 : (C + kTile - 1) / kTile; }
+// Form of a CTA: 8 warps, two CTAs per SM, or, where 128 registers do not hold
+// two targets' sums of half a class's rows, 16 warps of which two share a class's
+// targets (fast setup of N = 1e6, p = 12: 42.5 ms; 8 warps with spills 51.5, with
+// 240 registers and one CTA per SM 48.7)
+__host__ __device__ __forceinline__ int warps_of(int p) { return p <= 11 ? 8 : 16; }
+// columns staged at a time (one per warp), and tiles of the columns: at least
+// two, so that an orbit's cells are known a step before its first tile is loaded
+__host__ __device__ __forceinline__ int tiles_of(int p) {
+  const int C = (p + 1) * (p + 1), tile = warps_of(p);
+  return C <= tile ? 2 : (C + tile - 1) / tile;
+}
 
 // Rows by class; a class is two halves of `half` rows (the rows of the lower
 // and upper 16 lanes), each padded to an even number.
@@ -118,7 +125,7 @@ struct TableArgs {
 // T_o[row][col] from the scaled irregular harmonics of the integer offsets
 // (k_offset_table); entry (orbit, col, row)
 __global__ void k_m2l_tables(const __grid_constant__ TableArgs A, const double* __restrict__ otab, int2* __restrict__ T) {
-  const int p = A.p, C = (p + 1) * (p + 1), cpad = tiles_of(C) * kTile;
+  const int p = A.p, C = (p + 1) * (p + 1), cpad = tiles_of(p) * warps_of(p);
   const int per = (2 * p + 1) * (2 * p + 2) / 2;
   const long long total = (long long)kOrbits * cpad * A.rows;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
@@ -196,15 +203,18 @@ __global__ void __launch_bounds__(256)
     for (int col = warp; col < C; col += 8) M[(size_t)col * ncl + base + lane] = tile[lane * (C + 1) + col];
 }
 
-// a b + c in one instruction (the carry form of the sums over charges makes
-// this kernel 1.3 times slower: 28.7 instead of 21.6 ms at level 6)
+// a b + c in one instruction (with the carry form of the sums over charges the
+// fast setup of N = 1e6, p = 12 takes 49.5 instead of 42.5 ms)
 __device__ __forceinline__ long long m2l_wide(int a, int b, long long c) {
   long long r;
   asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
   return r;
 }
 
-__device__ __forceinline__ void cta_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+template <int W>
+__device__ __forceinline__ void cta_sync() {
+  asm volatile("bar.sync 1, %0;" ::"n"(32 * W) : "memory");
+}
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
@@ -223,9 +233,9 @@ __device__ __forceinline__ void cp_async8(void* dst, const void* src, bool valid
 }
 
 struct M2LShared {
-  int2* T;        // [2][kTile rows]: table columns
-  int2* Mt;       // [2][kTile][8][32]: transform values
-  long long* raw; // [kTile][8][32]: the members' multipoles on their way there
+  int2* T;        // [2][warps][rows]: table columns
+  int2* Mt;       // [2][warps][8][32]: transform values
+  long long* raw; // [warps][8][32]: the members' multipoles on their way there
   int* cell;      // [2][8][32]: members' cells of an orbit (-1: none), by lane
   int* shift;     // [2][8][32]: shifts to the unit of the orbit's group
   int* unit;      // [MC_M2L_GROUPS][32]: that unit (its exponent; -4096: no cell)
@@ -258,15 +268,17 @@ __device__ __forceinline__ int cell_at(const M2LTask& k, int ox, int oy, int oz,
 // One CTA's task, as the warp that owns class w of NR rows sees it: every
 // thread stages its target's part of the next tile's Mt and of the table
 // columns while its warp computes the current ones.
-template <int NR>  // rows of half a class
+template <int W, int NR>  // warps of the CTA, rows of half a class
 __device__ __forceinline__ void m2l_task(const M2LArgs& A, const int2* __restrict__ T, const long long* __restrict__ M,
                                          const int* __restrict__ E, double* __restrict__ out, const M2LTask& k,
                                          const M2LShared& S, int t0, int w, int lane) {
-  constexpr int NT = 2;
-  const int C = (A.p + 1) * (A.p + 1), tiles = tiles_of(C), h = A.h, ncl = A.nl * A.nl * A.nl;
+  constexpr int NT = 16 / W, kTile = W;
+  const int C = (A.p + 1) * (A.p + 1), tiles = (C + kTile - 1) / kTile > 1 ? (C + kTile - 1) / kTile : 2, h = A.h;
+  const int ncl = A.nl * A.nl * A.nl;
   const int ob = k.oc * A.per_o, oe = min(kOrbits, ob + A.per_o);
   const int steps = (oe - ob) * tiles, tsz = kTile * A.rows;
-  const int tid = 32 * w + lane, cls = class_of_warp(w);
+  const int tid = 32 * w + lane, cls = class_of_warp(w & 7);
+  const int tb = NT == 2 ? lane & 15 : (w >> 3) * 16 + (lane & 15);  // this lane's (first) target
   // products of the high parts, and the two cross products
   long long hh[NR > 0 ? NR : 1][NT], x[NR > 0 ? NR : 1][NT];
 #pragma unroll
@@ -276,6 +288,7 @@ __device__ __forceinline__ void m2l_task(const M2LArgs& A, const int2* __restric
   int lo = ob, lt = 0;  // orbit and tile to load next
   // member w (signs of its offset: bits x 4, y 2, z 1) of an orbit
   auto members = [&](int o) {
+    if (W > 8 && w >= 8) return;
     int of[3];
     bool ok = k.valid;
 #pragma unroll
@@ -301,7 +314,7 @@ __device__ __forceinline__ void m2l_task(const M2LArgs& A, const int2* __restric
     }
     const char* src = reinterpret_cast<const char*>(T + ((size_t)lo * tiles + lt) * tsz);
     char* dst = reinterpret_cast<char*>(S.T + (s & 1) * tsz);
-    for (int i = 16 * tid; i < tsz * (int)sizeof(int2); i += 16 * 256) cp_async16(dst + i, src + i);
+    for (int i = 16 * tid; i < tsz * (int)sizeof(int2); i += 16 * 32 * W) cp_async16(dst + i, src + i);
     asm volatile("cp.async.commit_group;" ::: "memory");
     if (++lt == tiles) {
       lt = 0;
@@ -342,8 +355,8 @@ __device__ __forceinline__ void m2l_task(const M2LArgs& A, const int2* __restric
     const int h3 = h * h * h;
 #pragma unroll
     for (int t = 0; t < NT; t++) {
-      const int ii = t0 + 16 * t + (lane & 15);
-      const double unit = ldexp(1.0, S.unit[g * 32 + 16 * t + (lane & 15)]);
+      const int ii = t0 + 16 * t + tb;
+      const double unit = ldexp(1.0, S.unit[g * 32 + 16 * t + tb]);
       const int i = 2 * (ii / (h * h)) + k.b[0], j = 2 * ((ii / h) % h) + k.b[1], kk = 2 * (ii % h) + k.b[2];
       double* o = out + ((size_t)((i * A.nl + j) * A.nl + kk) * A.nco + k.oc) * C;
 #pragma unroll
@@ -360,44 +373,47 @@ __device__ __forceinline__ void m2l_task(const M2LArgs& A, const int2* __restric
     first = false;
   };
   members(ob);
-  cta_sync();
+  cta_sync<W>();
   load(0);
   store(0);
-  cta_sync();
+  cta_sync<W>();
   int tile = 0, co = ob;  // of the current step: tile and orbit
   for (int s = 0; s < steps; s++) {
     if (s + 1 < steps) load(s + 1);
     if constexpr (NR > 0) {
       const int2* tt = S.T + (s & 1) * tsz + A.start[cls] + (lane >> 4) * ((NR + 1) / 2 * 2);
-      const int2* m0 = S.Mt + (size_t)(s & 1) * kTile * 8 * 32 + (lane & 15);
+      const int2* m0 = S.Mt + (size_t)(s & 1) * kTile * 8 * 32 + tb;
+#pragma unroll 1
+      for (int c0 = 0; c0 < kTile; c0 += 8) {
 #pragma unroll 2
-      for (int c = 0; c < kTile; c++) {
-        const int d = cls ^ A.ccol[tile * kTile + c];
-        int2 m[NT];
+        for (int c = c0; c < c0 + 8; c++) {
+          const int d = cls ^ A.ccol[tile * kTile + c];
+          int2 m[NT];
 #pragma unroll
-        for (int t = 0; t < NT; t++) m[t] = m0[(c * 8 + d) * 32 + 16 * t];
-        const int4* tr = reinterpret_cast<const int4*>(tt + c * A.rows);
+          for (int t = 0; t < NT; t++) m[t] = m0[(c * 8 + d) * 32 + 16 * t];
+          const int4* tr = reinterpret_cast<const int4*>(tt + c * A.rows);
 #pragma unroll
-        for (int r = 0; r < NR; r++) {
-          const int4 q = tr[r / 2];
-          const int th = r & 1 ? q.z : q.x, tl = r & 1 ? q.w : q.y;
+          for (int r = 0; r < NR; r++) {
+            const int4 q = tr[r / 2];
+            const int th = r & 1 ? q.z : q.x, tl = r & 1 ? q.w : q.y;
 #pragma unroll
-          for (int t = 0; t < NT; t++) {
-            hh[r][t] = m2l_wide(th, m[t].x, hh[r][t]);
-            x[r][t] = m2l_wide(th, m[t].y, x[r][t]);
-            x[r][t] = m2l_wide(tl, m[t].x, x[r][t]);
+            for (int t = 0; t < NT; t++) {
+              hh[r][t] = m2l_wide(th, m[t].x, hh[r][t]);
+              x[r][t] = m2l_wide(th, m[t].y, x[r][t]);
+              x[r][t] = m2l_wide(tl, m[t].x, x[r][t]);
+            }
           }
         }
+        // |x| < 8 (2^29 2^29 + 2^29 2^30) + 2^30 < 2^63 between two carries
+        static_assert(kBitsT - kLimb <= 29 && kBitsM + 3 - kLimb <= 30 && kLimb <= 30, "cross products");
+#pragma unroll
+        for (int r = 0; r < NR; r++)
+#pragma unroll
+          for (int t = 0; t < NT; t++) {
+            hh[r][t] += x[r][t] >> kLimb;
+            x[r][t] &= (1 << kLimb) - 1;
+          }
       }
-      // |x| < 8 (2^29 2^29 + 2^29 2^30) + 2^30 < 2^63 between two carries
-      static_assert(kTile <= 8 && kBitsT - kLimb <= 29 && kBitsM + 3 - kLimb <= 30 && kLimb <= 30, "cross products");
-#pragma unroll
-      for (int r = 0; r < NR; r++)
-#pragma unroll
-        for (int t = 0; t < NT; t++) {
-          hh[r][t] += x[r][t] >> kLimb;
-          x[r][t] &= (1 << kLimb) - 1;
-        }
     }
     if (++tile == tiles) {
       tile = 0;
@@ -405,25 +421,23 @@ __device__ __forceinline__ void m2l_task(const M2LArgs& A, const int2* __restric
       if (++co == oe || m2l_group(A.orbit[co]) != g) flush(g);
     }
     if (s + 1 < steps) store(s + 1);
-    cta_sync();
+    cta_sync<W>();
   }
 }
 
 }  // namespace
 
-// CTAs per SM: two, where 128 registers hold the sums of half a class's rows
-// (p = 12 with two: 284 bytes of spills, level 6 of N = 1e6 39 instead of 36 ms)
-template <int CTAS>
-__global__ void __launch_bounds__(256, CTAS)
+template <int W>
+__global__ void __launch_bounds__(32 * W, 16 / W)
     k_m2l_fix(const __grid_constant__ M2LArgs A, const int2* __restrict__ T, const long long* __restrict__ M,
               const int* __restrict__ E, double* __restrict__ out) {
   extern __shared__ int4 dyn4[];
   constexpr int kTargets = 32;
   M2LShared S;
   S.T = reinterpret_cast<int2*>(dyn4);
-  S.Mt = S.T + 2 * kTile * A.rows;
-  S.raw = reinterpret_cast<long long*>(S.Mt + 2 * kTile * 8 * 32);
-  S.cell = reinterpret_cast<int*>(S.raw + kTile * 8 * 32);
+  S.Mt = S.T + 2 * W * A.rows;
+  S.raw = reinterpret_cast<long long*>(S.Mt + 2 * W * 8 * 32);
+  S.cell = reinterpret_cast<int*>(S.raw + W * 8 * 32);
   S.shift = S.cell + 2 * 8 * 32;
   S.unit = S.shift + 2 * 8 * 32;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -442,9 +456,9 @@ __global__ void __launch_bounds__(256, CTAS)
   for (int d = 0; d < 3; d++) k.b[d] = (k.cls >> (2 - d)) & 1;
   // units of the sums: the largest of the cells at a group's offsets
   static_assert(kTargets == 32, "a target per lane");
-  for (int i = threadIdx.x; i < MC_M2L_GROUPS * 32; i += 256) S.unit[i] = -4096;
+  for (int i = threadIdx.x; i < MC_M2L_GROUPS * 32; i += 32 * W) S.unit[i] = -4096;
   __syncthreads();
-  for (int q = w; q < 216; q += 8) {
+  for (int q = w; q < 216; q += W) {
     const int ox = q / 36 - 2 - k.b[0], oy = (q / 6) % 6 - 2 - k.b[1], oz = q % 6 - 2 - k.b[2];
     if (ox >= -1 && ox <= 1 && oy >= -1 && oy <= 1 && oz >= -1 && oz <= 1) continue;
     const int c = cell_at(k, ox, oy, oz, h, A.pbc != 0);
@@ -453,19 +467,25 @@ __global__ void __launch_bounds__(256, CTAS)
   __syncthreads();
   // half of 1, 3, 6, 10, 15, 21, 28, 36 rows
 #define MC_M2L_ROWS(NR_) \
-  case NR_: m2l_task<NR_>(A, T, M, E, out, k, S, t0, w, lane); break;
-  switch (A.half[class_of_warp(w)]) {
+  case NR_: m2l_task<W, NR_>(A, T, M, E, out, k, S, t0, w, lane); break;
+  switch (A.half[class_of_warp(w & 7)]) {
     MC_M2L_ROWS(1)
     MC_M2L_ROWS(2)
     MC_M2L_ROWS(3)
     MC_M2L_ROWS(5)
     MC_M2L_ROWS(8)
     MC_M2L_ROWS(11)
-    MC_M2L_ROWS(14)
-    MC_M2L_ROWS(18)
-    // (0 rows; any other number would leave the results out, but never the
-    // barriers)
-    default: m2l_task<0>(A, T, M, E, out, k, S, t0, w, lane);
+    default:
+      // (0 rows; any other number would leave its results out, but no barrier)
+      if constexpr (W == 16) {
+        switch (A.half[class_of_warp(w & 7)]) {
+          MC_M2L_ROWS(14)
+          MC_M2L_ROWS(18)
+          default: m2l_task<W, 0>(A, T, M, E, out, k, S, t0, w, lane);
+        }
+      } else {
+        m2l_task<W, 0>(A, T, M, E, out, k, S, t0, w, lane);
+      }
   }
 #undef MC_M2L_ROWS
 }
@@ -473,8 +493,7 @@ __global__ void __launch_bounds__(256, CTAS)
 __global__ void k_offset_table(int p, double* __restrict__ out);
 
 size_t m2l_table_bytes(int p) {
-  const int C = (p + 1) * (p + 1);
-  return sizeof(int2) * (size_t)kOrbits * tiles_of(C) * kTile * m2l_layout(p).rows;
+  return sizeof(int2) * (size_t)kOrbits * tiles_of(p) * warps_of(p) * m2l_layout(p).rows;
 }
 
 // by group
@@ -560,11 +579,12 @@ cudaError_t m2l_fix_level(int p, int l, double w, bool pbc, int sms, const void*
   if (e != cudaSuccess) return e;
   k_m2l_convert<<<(ncl + 31) / 32, 256, csm, st>>>(V, K, M, E);
   const int chunks = (h * h * h + 31) / 32;
-  const size_t smem = sizeof(int2) * (2 * (size_t)kTile * L.rows + 3 * kTile * 8 * 32) + sizeof(int) * (4 * 8 + MC_M2L_GROUPS) * 32;
-  const auto kernel = p <= 11 ? k_m2l_fix<2> : k_m2l_fix<1>;
+  const int warps = warps_of(p);
+  const size_t smem = sizeof(int2) * (2 * (size_t)warps * L.rows + 3 * warps * 8 * 32) + sizeof(int) * (4 * 8 + MC_M2L_GROUPS) * 32;
+  const auto kernel = warps == 8 ? k_m2l_fix<8> : k_m2l_fix<16>;
   e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kernel<<<8 * chunks * A.nco, 256, smem, st>>>(A, (const int2*)table, M, E, A.nco > 1 ? scratch : Lout);
+  kernel<<<8 * chunks * A.nco, 32 * warps, smem, st>>>(A, (const int2*)table, M, E, A.nco > 1 ? scratch : Lout);
   e = cudaGetLastError();
   if (e == cudaSuccess && A.nco > 1) e = fix_reduce(ncl, A.nco, C, sms, scratch, Lout, st);
   return e;
