@@ -130,7 +130,8 @@ int mc_energy(mc_ctx *ctx, double *e_out);
 /* Total energy recomputed from the current expansions and positions. */
 int mc_energy_fresh(mc_ctx *ctx, double *e_out);
 /* Current positions (n, 3) into a host array: the PositionDat r that
- * accept() updates in Sec. 4.1. */
+ * accept() updates in Sec. 4.1.  (This and the read-outs of expansions and
+ * multipoles pass through the context's setup scratch, on the legacy stream.) */
 int mc_get_positions(mc_ctx *ctx, double *pos_out);
 /* Local coefficients L^Delta of level l (2..L), all cells, real layout,
  * paper normalisation; host array of 8^(l-1) * (p+1)^2 doubles. */
@@ -147,8 +148,9 @@ int mc_get_far(mc_ctx *ctx, double *K_out, double *H_out);
  * (MC_ERR_STATE until then). */
 int mc_set_lj(mc_ctx *ctx, double eps, double sigma, double cutoff);
 /* Work split of the near-field sum (Alg. 1) in the chain kernels: each of
- * the 27 near cells is summed by `parts` items per side (2 parts items when
- * r and r' share their finest cell), each taking every parts-th block of 32
+ * the 27 near cells is summed by `parts` items per side (in all forms but the
+ * FP64 barrier-free one 2 parts items for both sides when r and r' share their
+ * finest cell), each taking every parts-th block of 32
  * of the cell's charges.  parts = 0 restores the automatic choice made by
  * mc_init (one item per 48 charges of mean finest-cell occupancy, at most
  * 4); 1..4 forces it.  The result is the same sum in another order (dE

@@ -251,7 +251,7 @@ int run_setup(mc_ctx* c) {
   McSys& h = c->h;
   const int C = h.C;
   // Alg. L.3 per level: a gather over the interaction list of every cell,
-  // chunked where a level has few cells.  In fixed point (4.6 ms a
+  // chunked where a level has few cells.  In fixed point (4.7 ms a
   // level at N = 1e5, p = 12 instead of 41 in FP64, and at least as accurate)
   // unless the charges span more than MC_FIX_QSPAN powers of two
   for (int l = h.lmin; l <= h.L; l++) {

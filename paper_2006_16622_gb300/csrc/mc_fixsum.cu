@@ -84,7 +84,7 @@ constexpr int fix_ctas(int st) { return st <= 14 ? 4 : (st <= 23 ? 3 : 2); }
 // per thread, in shared memory, where all four warps read it.
 // Bound by the issue of integer instructions: 107 cycles of a sub-partition per
 // coefficient and 32 charges, 78 of them for 18 multiply-adds of 64 bits.  One
-// level of N = 1e5, p = 12 takes 4.6 ms; the same sums in FP64 (64 cycles an
+// level of N = 1e5, p = 12 takes 4.7 ms; the same sums in FP64 (64 cycles an
 // instruction) took 41 ms.
 template <int P>
 __global__ void __launch_bounds__(kThreads, fix_ctas(fix_shares(P).steps))

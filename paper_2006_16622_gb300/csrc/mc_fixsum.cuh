@@ -44,8 +44,9 @@ __host__ __device__ __forceinline__ long long fix_chunks_worth(long long units, 
 cudaError_t fix_launch(const FixPass& ps, const FixSource& src, double* out, cudaStream_t st);
 // Direct part of the energy: 1/r over the pairs of charges within near cells
 // (every pair and image once) in units of 1 / (four finest cells), one partial
-// (a sum and its rounding) for each of the returned number of blocks, followed by the workspace of fix_near_work doubles
-// (of use until the call's kernels are done)
+// (a sum and its rounding) for each of the returned number of blocks, followed by
+// the workspace of fix_near_work doubles (of use until the call's kernels are
+// done)
 int fix_near_blocks(int L, int sms, int cap);
 size_t fix_near_work(int L, int cap);
 cudaError_t fix_near(int L, bool pbc, double a, const FixSource& src, int blocks, double* out, cudaStream_t st);
