@@ -119,7 +119,7 @@ FixSource fix_source(const McSys& h) {
 }
 FixPass fix_pass(const mc_ctx* c, int l, bool irregular) {
   const McSys& h = c->h;
-  return FixPass{h.L, l, h.p, irregular, h.bc == MC_BC_PBC, h.a, c->qexp, 1, nullptr};
+  return FixPass{h.L, l, h.p, irregular, h.bc == MC_BC_PBC, h.a, c->qexp, 1, nullptr, h.n < h.ncellL};
 }
 // chunks of one Alg. L.3 pass, as many as the scratch holds
 int fix_chunks_for(const McSys& h, int sms, int l, size_t max_doubles) {
@@ -409,6 +409,19 @@ int energy_chunks(const McSys& h, int sms, int l, bool irregular) {
   return fix_chunks(h.L, l, irregular, sms, (double)h.n / (double)h.ncellL, h.p);
 }
 
+// Cell by cell costs by the cells, particle by particle by the charges.  Local
+// method: particles below 3/4 of a charge per finest cell (p = 8, by cells and by
+// particles: 0.25 a cell at L = 7 4.4 and 1.8 ms, 0.5 5.0 and 4.2, 1 6.1 and 10.4;
+// at L = 5 0.18 and 0.08, 0.19 and 0.12, 0.19 and 0.22).  Multipole method: about
+// 0.4 ms a level, with its 189 multipoles, for every particle of a warp, against
+// 12 ns an empty cell (L = 7, 1000 charges: 2.8 ms by particles, 6.1 by cells, 4096
+// 10.8 and 8.6; L = 6, 100: 2.0 and 0.66).
+bool energy_by_particles(const McSys& h, int sms) {
+  if (h.method == 0) return 4LL * h.n < 3LL * h.ncellL;
+  const long long turns = (h.n + 2 * sms * MC_WARPS - 1) / (2 * sms * MC_WARPS);
+  return turns * h.L * 30000 < h.ncellL;
+}
+
 // Total energy from the current expansions and positions into d_dst.  The
 // expansions' part is a contraction cell by cell: of the local expansions
 // with the cells' multipoles, or (multipole method) of the multipoles with
@@ -417,7 +430,7 @@ int energy_chunks(const McSys& h, int sms, int l, bool irregular) {
 // `mpole`: d_mpole holds the multipoles of the current positions.
 int energy_into(mc_ctx* c, double* d_dst, bool mpole) {
   const McSys& h = c->h;
-  if (c->fixed && !h.lj_on) {
+  if (c->fixed && !h.lj_on && !energy_by_particles(h, c->sms)) {
     const int nnear = fix_near_blocks(h.L, c->sms, h.cap);  // pairs of doubles
     CK(fix_near(h.L, h.bc == MC_BC_PBC, h.a, fix_source(h), nnear, c->d_scratch, c->stream));
     int nexp = 0;

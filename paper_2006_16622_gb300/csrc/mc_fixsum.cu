@@ -18,6 +18,7 @@ struct FixArgs {
   int ea;        // biased exponent of the box side
   int qexp;
   const double* dot;
+  int sparse;
 };
 
 // index of a coefficient with m = 0 (no imaginary part)
@@ -97,6 +98,22 @@ __global__ void __launch_bounds__(kThreads, fix_ctas(fix_shares(P).steps))
   if (A.src.range && !fix_usable(A.src.range)) return;
   const int nchunk = A.src.range ? A.src.range[3] : A.nchunk;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (A.sparse) {
+    // a cell without charges has no multipole, and nothing to contract (cells
+    // of up to 64 finest ones; 4096 charges at L = 7, p = 8, multipole method,
+    // whole energy: 14.4 -> 8.6 ms)
+    const int c = blockIdx.x / A.nchunk, n = 1 << (A.l - 1), b = A.L - A.l;
+    bool any = b > 2;
+    if (b <= 2 && tid < 1 << (3 * b)) {
+      const int x = ((c / (n * n)) << b) + (tid >> (2 * b)), y = (((c / n) % n) << b) + ((tid >> b) & ((1 << b) - 1)),
+                z = ((c % n) << b) + (tid & ((1 << b) - 1)), m = 1 << (A.L - 1);
+      any = A.src.count[(x * m + y) * m + z] > 0;
+    }
+    if (!__syncthreads_or(any)) {
+      if (tid == 0) out[blockIdx.x] = 0.0;
+      return;
+    }
+  }
   for (int i = tid; i < MC_FIX_WARPS * ST; i += nthr) s_step[i / ST][i % ST] = A.tab.step[i / ST][i % ST];
   const bool irr = A.irregular != 0, pbc = A.pbc != 0;
   const int qexp = A.src.range ? A.src.range[1] - 1022 : A.qexp;
@@ -583,8 +600,10 @@ __global__ void __launch_bounds__(256, 4)
   low = lane < 8 ? s_sum[lane][1] : 0.0;
   warp_two_sum(&total, &low);
   if (lane == 0) {
-    out[2 * blockIdx.x] = total;
-    out[2 * blockIdx.x + 1] = low;
+    // times 1 / (4 w), w = a / nL
+    const double x = total * (0.25 * nL), r = x / A.a;
+    out[2 * blockIdx.x] = r;
+    out[2 * blockIdx.x + 1] = (fma(-r, A.a, x) + low * (0.25 * nL)) / A.a;
   }
 }
 
@@ -675,6 +694,7 @@ cudaError_t fix_launch(const FixPass& ps, const FixSource& src, double* out, cud
   A.pbc = ps.pbc;
   A.qexp = ps.qexp;
   A.dot = ps.dot;
+  A.sparse = ps.dot && ps.sparse && !src.start;
   box_scale(ps.a, &A.rcp, &A.ea);
   const size_t smem = sizeof(int64_t) * (size_t)kThreads * (2 + 3 * (ps.p + 1));
   const long long ncl = 1LL << (3 * (ps.l - 1));

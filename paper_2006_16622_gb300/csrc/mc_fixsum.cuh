@@ -29,6 +29,7 @@ struct FixPass {
   int qexp;     // charges are at most 2^qexp in size
   int nchunk;   // chunks of the source units (finest cells) per target
   const double* dot;
+  bool sparse;  // with dot: most finest cells are empty (of use, not of need)
 };
 // chunks per target that keep every SM busy without tasks too short to pay
 // for themselves (occupancy: mean charges of a finest cell)
@@ -43,7 +44,7 @@ __host__ __device__ __forceinline__ long long fix_chunks_worth(long long units, 
 #endif
 cudaError_t fix_launch(const FixPass& ps, const FixSource& src, double* out, cudaStream_t st);
 // Direct part of the energy: 1/r over the pairs of charges within near cells
-// (every pair and image once) in units of 1 / (four finest cells), one partial
+// (every pair and image once), one partial
 // (a sum and its rounding) for each of the returned number of blocks, followed by
 // the workspace of fix_near_work doubles (of use until the call's kernels are
 // done)

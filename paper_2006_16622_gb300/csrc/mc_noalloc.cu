@@ -276,7 +276,7 @@ extern "C" int mc_p2l_level_noalloc(const double* d_part, const int* d_cell_star
   k_noalloc_range<<<rblocks, MC_THREADS, 0, stream>>>(P.nL, (double)P.nL / box, d_part, d_cell_start, (int)nfix, units, range);
   // no error was pending before the launch, so one now is the launch's own
   if (cudaGetLastError() != cudaSuccess) return MC_ERR_CUDA;
-  const FixPass ps{levels, level, p, true, bc == MC_BC_PBC, box, 0, (int)nfix, nullptr};
+  const FixPass ps{levels, level, p, true, bc == MC_BC_PBC, box, 0, (int)nfix, nullptr, false};
   const FixSource src{d_part, nullptr, 0, d_cell_start, range};
   if (fix_launch(ps, src, scratch, stream) != cudaSuccess) {
     cudaGetLastError();

@@ -430,9 +430,8 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// U from the partials of the near pairs (nnear times a sum and its rounding, in
-// units of 1 / (four finest cells)) and (twice) of the expansions, and the
-// periodic terms.  Sums keep their rounding: near pairs and expansions cancel to
+// U from the partials of the near pairs (nnear times a sum and its rounding) and
+// (twice) of the expansions, and the periodic terms.  Sums keep their rounding: near pairs and expansions cancel to
 // a fraction of either.
 __global__ void __launch_bounds__(256)
     k_energy_sum(const McSys* __restrict__ sysp, int nnear, int nexp, const double* __restrict__ in,
@@ -444,12 +443,6 @@ __global__ void __launch_bounds__(256)
   for (int i = threadIdx.x; i < nnear; i += 256) {
     two_add(&s, &e, in[2 * i]);
     e += in[2 * i + 1];
-  }
-  {
-    // times 1 / (4 w), w = a / nL
-    const double x = s * (0.25 * S.nL), r = x / S.a;
-    e = (fma(-r, S.a, x) + e * (0.25 * S.nL)) / S.a;
-    s = r;
   }
   {
     // (many and small)
