@@ -359,8 +359,9 @@ struct FixTab {
   unsigned char col[MC_FIX_WARPS][MC_PMAX + 1]; // the warp's columns in order
 };
 
-// R: the radius R0 in length units
-inline void fix_tab_build(FixTab* T, int p, bool irregular, double R) {
+// R: the radius R0 in length units; `unit` (optional) receives the scales for a
+// radius of 1 before they are rounded
+inline void fix_tab_build(FixTab* T, int p, bool irregular, double R, long double (*unit)[MC_FIX_STEPS] = nullptr) {
   const FixShares sh = fix_shares(p);
   int ncol[MC_FIX_WARPS] = {0, 0, 0, 0};
   for (int k = 0; k < MC_FIX_WARPS; k++) {
@@ -410,7 +411,9 @@ inline void fix_tab_build(FixTab* T, int p, bool irregular, double R) {
         }
       }
       const long double sign = (i & 2) ? -1.0L : 1.0L;
-      T->scale[k][t] = (double)(head * rad * sign * prod / (long double)(1ull << sigma) / 9007199254740992.0L);
+      const long double one = head * sign * prod / (long double)(1ull << sigma) / 9007199254740992.0L;
+      if (unit) unit[k][t] = one;
+      T->scale[k][t] = (double)(one * rad);
       T->index[k][t] = (short)(n * n + (m ? 2 * m - 1 : 0));
     }
   }

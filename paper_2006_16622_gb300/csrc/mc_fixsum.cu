@@ -1,6 +1,7 @@
 // Harmonic sums over the charges of cells in fixed point (mc_fix.cuh): the
 // Alg. L.3 gather of every setup, the multipoles of Eq. (4).
 #include <algorithm>
+#include <mutex>
 
 #include "mc_dev.cuh"
 #include "mc_fix.cuh"
@@ -682,10 +683,42 @@ int fix_chunks(int L, int l, bool irregular, int sms, double occupancy, int p) {
   return (int)std::max<long long>(1, std::min(want, fix_chunks_worth(units, occupancy)));
 }
 
+// Tables of an order for a radius of 1, formed on first use and never changed.
+// (Where long double is software, as on Arm hosts, forming them takes 7 to 85 us,
+// p = 4 to 15, which was longer than the kernels of a small system; the scales of
+// a radius take a tenth of that.)
+struct FixBase {
+  FixTab tab;
+  long double unit[MC_FIX_WARPS][MC_FIX_STEPS];
+};
+static const FixBase& fix_base(int p, bool irregular) {
+  static FixBase base[MC_PMAX + 1][2];
+  static std::once_flag once[MC_PMAX + 1][2];
+  std::call_once(once[p][irregular], [&] { fix_tab_build(&base[p][irregular].tab, p, irregular, 1.0, base[p][irregular].unit); });
+  return base[p][irregular];
+}
+
 cudaError_t fix_launch(const FixPass& ps, const FixSource& src, double* out, cudaStream_t st) {
+  if (ps.p < 0 || ps.p > MC_PMAX) return cudaErrorInvalidValue;
   FixArgs A;
   const double w = ps.a / (double)(1 << (ps.l - 1));
-  fix_tab_build(&A.tab, ps.p, ps.irregular, ps.irregular ? kFixR0 * w : w);
+  {
+    const FixBase& b = fix_base(ps.p, ps.irregular);
+    A.tab = b.tab;
+    // R^n, or R^-(n + 1)
+    const long double R = ps.irregular ? kFixR0 * w : w, step = ps.irregular ? 1.0L / R : R;
+    long double power[MC_PMAX + 1];
+    power[0] = ps.irregular ? step : 1.0L;
+    for (int n = 1; n <= ps.p; n++) power[n] = power[n - 1] * step;
+    for (int k = 0; k < MC_FIX_WARPS; k++)
+      for (int t = 0; t < MC_FIX_STEPS; t++) {
+        const int i = A.tab.index[k][t];
+        if (i < 0) continue;
+        int n = 0;
+        while ((n + 1) * (n + 1) <= i) n++;
+        A.tab.scale[k][t] = (double)(b.unit[k][t] * power[n]);
+      }
+  }
   A.src = src;
   A.L = ps.L;
   A.l = ps.l;
