@@ -412,12 +412,19 @@ int energy_chunks(const McSys& h, int sms, int l, bool irregular) {
 // Cell by cell costs by the cells, particle by particle by the charges.  Local
 // method: particles below 3/4 of a charge per finest cell (p = 8, by cells and by
 // particles: 0.25 a cell at L = 7 4.4 and 1.8 ms, 0.5 5.0 and 4.2, 1 6.1 and 10.4;
-// at L = 5 0.18 and 0.08, 0.19 and 0.12, 0.19 and 0.22).  Multipole method: about
+// at L = 5 0.18 and 0.08, 0.19 and 0.12, 0.19 and 0.22), and where a cell holds
+// twice the mean or more, which one block then sums on every level, up to 250
+// charges times 2^L (half of 2000 in one cell at L = 4 0.27 and 0.16, of 4000 0.37
+// and 0.36, at L = 5 of 4000 0.45 and 0.29, of 8000 0.77 and 0.78).  Multipole method: about
 // 0.4 ms a level, with its 189 multipoles, for every particle of a warp, against
 // 12 ns an empty cell (L = 7, 1000 charges: 2.8 ms by particles, 6.1 by cells, 4096
 // 10.8 and 8.6; L = 6, 100: 2.0 and 0.66).
 bool energy_by_particles(const McSys& h, int sms) {
-  if (h.method == 0) return 4LL * h.n < 3LL * h.ncellL;
+  if (h.method == 0) {
+    // cap is twice the fullest cell's count
+    const bool dense = fix_near_work(h.L, h.cap) > 0 && (long long)h.cap * h.ncellL > 4LL * h.n;
+    return 4LL * h.n < 3LL * h.ncellL || (dense && h.n < 250LL << h.L);
+  }
   const long long turns = (h.n + 2 * sms * MC_WARPS - 1) / (2 * sms * MC_WARPS);
   return turns * h.L * 30000 < h.ncellL;
 }

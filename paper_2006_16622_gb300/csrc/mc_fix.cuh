@@ -424,11 +424,12 @@ inline void fix_tab_build(FixTab* T, int p, bool irregular, double R, long doubl
 // and rows and columns of tile k (the cell itself: tiles on and below the
 // diagonal).
 #define MC_NEAR_TILE 128
-__host__ __device__ __forceinline__ long long near_tiles(int ni, int nj, bool same) {
-  const long long a = (ni + MC_NEAR_TILE - 1) / MC_NEAR_TILE, b = (nj + MC_NEAR_TILE - 1) / MC_NEAR_TILE;
+__host__ __device__ __forceinline__ long long near_tiles(int ni, int nj, bool same, int tile = MC_NEAR_TILE) {
+  const long long a = (ni + tile - 1) / tile, b = (nj + tile - 1) / tile;
   return same ? a * (a + 1) / 2 : a * b;
 }
-__host__ __device__ __forceinline__ void near_tile(long long k, int nj, bool same, int* ti, int* tj) {
+__host__ __device__ __forceinline__ void near_tile(long long k, int nj, bool same, int* ti, int* tj,
+                                                  int tile = MC_NEAR_TILE) {
   if (same) {
     long long i = (long long)((sqrt(8.0 * (double)k + 1.0) - 1.0) * 0.5);
     while (i * (i + 1) / 2 > k) i--;
@@ -436,7 +437,7 @@ __host__ __device__ __forceinline__ void near_tile(long long k, int nj, bool sam
     *ti = (int)i;
     *tj = (int)(k - i * (i + 1) / 2);
   } else {
-    const long long b = (nj + MC_NEAR_TILE - 1) / MC_NEAR_TILE;
+    const long long b = (nj + tile - 1) / tile;
     *ti = (int)(k / b);
     *tj = (int)(k % b);
   }

@@ -342,11 +342,14 @@ __global__ void __launch_bounds__(256)
 // neighbour's charges staged in shared memory and read by all lanes (or, where
 // few of the tile's charges are left, by the group of lanes whose turn they
 // are: 4.00 -> 3.20 ms for 1e6 charges, 30.5 a cell, and 121 -> 70 us for 3e4,
-// 7.3 a cell).  The first tiles of all (cell, neighbour) come first; where
+// 7.3 a cell; 3.26 ms and 99 us since the sums keep their rounding).  The first
+// tiles of all (cell, neighbour) come first; where
 // cells may hold more than a tile, the others are counted by k_near_extra and
-// dealt out in order (4000 of 8000 charges in one cell, L = 5, whole fresh
-// energy: 79 ms with one warp for a (cell, neighbour), 0.93 now, 1.0 with the
-// FP64 kernel's warp per charge; 8 x 4000: 183, 5.7 and 37 ms).  At
+// dealt out in order, in tiles of 64 x 64 (4000 of 8000 charges in one cell, L =
+// 5, whole fresh energy: 79 ms with one warp for a (cell, neighbour), 1.25 with
+// tiles of 128 and a second look at whole tiles, 0.77 now, 0.78 with the FP64
+// kernel's warp per charge; half of 16000: 1.9, 1.4 and 3.1 with the latter
+// three).  At
 // 30.5 a cell 310 cycles of a sub-partition for 32 pairs, idle lanes included;
 // the FP64 multiply-add takes 64 beside the integer ones.  Differences are exact
 // 64-bit integers; 1/r comes from a single-precision estimate and one
@@ -361,10 +364,15 @@ struct NearArgs {
   uint64_t box;  // the box side in units of 2^-60 finest cells, modulo 2^64
   double a;
   double unit;  // 1 / (four finest cells)
+  int tile;  // MC_NEAR_TILE, or MC_NEAR_DENSE
   // tiles beyond the first ones, of every cell and of every 1024 cells (null:
   // no cell can hold more than a tile)
   const long long *cells, *blocks;
 };
+// Tiles where cells may hold more than MC_NEAR_TILE charges: a warp takes 42 us
+// for one of 64 x 64, 170 for one of 128 x 128, which was the time of the kernel
+// for a few thousand charges (smaller ones cost more to find than they save)
+#define MC_NEAR_DENSE 64
 constexpr int kNearBlock = 1024;  // cells counted by a block of k_near_extra
 
 // neighbour o (0: itself, else one of 13) of a cell: its index, image shifts,
@@ -387,7 +395,7 @@ __device__ __forceinline__ bool near_neighbour(int cell, int o, int nL, bool pbc
 __device__ __forceinline__ long long near_extra(const NearArgs& A, int cell, int o, int nL) {
   int other, im[3];
   if (o >= 14 || !near_neighbour(cell, o, nL, A.pbc, &other, im)) return 0;
-  return max(near_tiles(A.src.count[cell], A.src.count[other], o == 0) - 1, 0ll);
+  return max(near_tiles(A.src.count[cell], A.src.count[other], o == 0, A.tile) - 1, 0ll);
 }
 
 __global__ void __launch_bounds__(kNearBlock)
@@ -453,7 +461,7 @@ __device__ __noinline__ bool near_locate(const NearArgs& A, long long e, int nL,
 // line, as much as the FP64 operations of the other route; with the line at
 // 2^-12 it was 2^-51, and 2^(L-3) times that with coordinates in 2^-62 of the
 // box.  One own cell in a thousand at 24 charges a cell has such a pair; it is
-// left to a second look at the tile (a call in the loop cost a fifth of the
+// left to a second look at the block of 32 x 32 pairs (a call in the loop cost a fifth of the
 // kernel).
 constexpr int kNearClose = 9;
 __device__ __forceinline__ int near_zeros(int64_t dx, int64_t dy, int64_t dz) {
@@ -527,11 +535,11 @@ __global__ void __launch_bounds__(256, 4)
     int other, im[3];
     if (!near_neighbour(cell, o, nL, A.pbc, &other, im)) continue;
     int ni = A.src.count[cell], nj = A.src.count[other];
-    if (tile) near_tile(tile, nj, o == 0, &ti, &tj);
-    const int ib = ti * MC_NEAR_TILE, jb = tj * MC_NEAR_TILE;
-    ni = min(ni, ib + MC_NEAR_TILE);
-    nj = min(nj, jb + MC_NEAR_TILE);
-    bool close = false;
+    if (tile) near_tile(tile, nj, o == 0, &ti, &tj, A.tile);
+    const int ib = ti * A.tile, jb = tj * A.tile;
+    ni = min(ni, ib + A.tile);
+    nj = min(nj, jb + A.tile);
+    unsigned close = 0;  // blocks of 32 x 32 pairs with close ones (bit 4 row + column)
     for (int i0 = ib; i0 < ni; i0 += 32) {
       // fewer than 17 particles left: 2 to 32 groups of lanes share the other
       // cell's particles (at 30.5 a cell a second pass has five on average)
@@ -559,6 +567,7 @@ __global__ void __launch_bounds__(256, 4)
         }
         __syncwarp();
         const int jn = min(32, nj - j0);
+        bool here = false;
         // eight pairs at a time, so that the running sum rounds at an eighth of
         // the additions: a pair counts once here, in the FP64 kernel from both
         // sides, which averages the rounding of two sums.  Energies of 2000
@@ -576,18 +585,21 @@ __global__ void __launch_bounds__(256, 4)
             for (int a = 0; a < 3; a++) d[a] = near_diff(xi[a], x[a]);
             int k;
             const double rinv = near_rinv(d[0], d[1], d[2], &k);
-            close |= k >= kNearClose;
+            here |= k >= kNearClose;
             // (rinv is finite for any difference)
             part = fma(k >= kNearClose ? 0.0 : __longlong_as_double(x[3]), rinv, part);
           }
           acc += part;
         }
+        if (here) close |= 1u << ((i0 - ib) / 32 * 4 + (j0 - jb) / 32);
       }
       two_add(&total, &low, qi * acc);
     }
-    if (__any_sync(0xffffffffu, close))
-      two_add(&total, &low, near_close_pairs(A, &rows[(size_t)cell * cap], ib, ni, &rows[(size_t)other * cap], jb, nj,
-                                             (im[0] + 1) | (im[1] + 1) << 2 | (im[2] + 1) << 4));
+    for (close = __reduce_or_sync(0xffffffffu, close); close; close &= close - 1) {
+      const int b = __ffs(close) - 1, i0 = ib + 32 * (b / 4), j0 = jb + 32 * (b % 4);
+      two_add(&total, &low, near_close_pairs(A, &rows[(size_t)cell * cap], i0, min(ni, i0 + 32), &rows[(size_t)other * cap],
+                                             j0, min(nj, j0 + 32), (im[0] + 1) | (im[1] + 1) << 2 | (im[2] + 1) << 4));
+    }
   }
   warp_two_sum(&total, &low);
   __shared__ double s_sum[8][2];
@@ -608,9 +620,11 @@ __global__ void __launch_bounds__(256, 4)
   }
 }
 
+static int near_size(int cap) { return cap <= MC_NEAR_TILE ? MC_NEAR_TILE : MC_NEAR_DENSE; }
+
 int fix_near_blocks(int L, int sms, int cap) {
   // a warp per tile, if every cell were full
-  const double tiles = (double)(14LL << (3 * (L - 1))) * (double)near_tiles(cap, cap, false);
+  const double tiles = (double)(14LL << (3 * (L - 1))) * (double)near_tiles(cap, cap, false, near_size(cap));
   return (int)std::min(tiles / 8.0 + 1.0, 8.0 * sms);
 }
 
@@ -644,6 +658,7 @@ cudaError_t fix_near(int L, bool pbc, double a, const FixSource& src, int blocks
   }
   A.box = L < 5 ? 1ull << (59 + L) : 0ull;
   A.unit = (double)(1 << (L - 1)) / (4.0 * a);
+  A.tile = near_size(src.cap);
   A.cells = A.blocks = nullptr;
   if (fix_near_work(L, src.cap)) {
     const int ncell = 1 << (3 * (L - 1)), nb = (ncell + kNearBlock - 1) / kNearBlock;
